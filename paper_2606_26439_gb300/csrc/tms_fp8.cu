@@ -20,62 +20,139 @@ namespace tms {
 namespace fp8 {
 
 constexpr int kQuantWarps = 8;
-constexpr int kMaxGroups = 8;  // d <= 1024: d / 4 groups of 4 elements over 32 lanes
+constexpr int kQuantUnits = 4;  // 8-element units of a row per lane: d <= 1024 over 32 lanes
 
+// Elements 8 u .. 8 u + 7 of x as fp32 (x 16-byte aligned).
 template <int DT>
-__device__ __forceinline__ float4 load4(const void* x, int64_t e) {
-    if (DT == TMS_F32) return *reinterpret_cast<const float4*>(static_cast<const float*>(x) + e);
-    const uint2 u = *reinterpret_cast<const uint2*>(static_cast<const uint16_t*>(x) + e);
-    float2 lo, hi;
-    if (DT == TMS_F16) {
-        lo = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
-        hi = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
+__device__ __forceinline__ void load8(const void* x, int64_t u, float (&v)[8]) {
+    if (DT == TMS_F32) {
+        const float4* p = static_cast<const float4*>(x) + 2 * u;
+        const float4 a = __ldcs(p), b = __ldcs(p + 1);
+        v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+        v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
     } else {
-        lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
-        hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+        const uint4 w = __ldcs(static_cast<const uint4*>(x) + u);
+        const uint32_t h[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 f = DT == TMS_F16 ? __half22float2(*reinterpret_cast<const __half2*>(&h[i]))
+                                           : __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h[i]));
+            v[2 * i] = f.x;
+            v[2 * i + 1] = f.y;
+        }
     }
-    return make_float4(lo.x, lo.y, hi.x, hi.y);
 }
 
-__device__ __forceinline__ uint32_t encode(float v, float s) {
-    if (s == 0.f) return 0u;
-    return static_cast<uint32_t>(__nv_cvt_float_to_fp8(__fdiv_rn(v, s), __NV_SATFINITE, __NV_E4M3));
+// x / s rounded to nearest even, from r = RN(1 / s): Markstein's final
+// division step (P. Markstein, "Computation of elementary functions on the
+// IBM RISC System/6000 processor", 1990) -- with r the correctly rounded
+// reciprocal and q within an ulp of x / s, q + r (x - q s) rounds to
+// RN(x / s).  x r alone can be two ulps off, so the step runs twice: once
+// to reach an ulp, once to round.  The residual is taken with its sign
+// reversed so that x = -0 keeps its sign.  Exact while no residual
+// underflows, which keeping s within kQuantMinScale .. kQuantMaxScale
+// ensures for every quotient that does not round to code 0.
+__device__ __forceinline__ float div_markstein(float x, float s, float r) {
+    float q = x * r;
+    q = fmaf(fmaf(q, s, -x), -r, q);
+    return fmaf(fmaf(q, s, -x), -r, q);
+}
+constexpr float kQuantMinScale = 0x1p-60f, kQuantMaxScale = 0x1p60f;
+
+// Two E4M3 codes (a in the low byte), nearest even, saturating.
+__device__ __forceinline__ uint32_t encode2(float a, float b) {
+    return __nv_cvt_float2_to_fp8x2(make_float2(a, b), __NV_SATFINITE, __NV_E4M3);
 }
 
-// One warp per row: amax over the row (fp32), s = amax / 448, code =
-// E4M3(x / s) rounded to nearest even with saturation; both divisions are
-// IEEE fp32.  Lane l holds groups l, l + 32, ... of 4 elements.
-template <int DT>
+// Per row: amax (fp32), s = amax / 448, code = E4M3(x / s) rounded to
+// nearest even with saturation, both quotients those of an IEEE fp32
+// division.  LP lanes share a row (a warp takes 32 / LP rows at once), each
+// with up to kQuantUnits of the row's 8-element units (l, l + LP, ...), all
+// loaded before their arithmetic.
+//
+// Few lanes per row, so that a row's shuffles and its two reciprocals are
+// spread over up to 32 elements per lane; every access still covers whole
+// 32-byte sectors.  Bound by HBM once the arithmetic is small enough.  4 M
+// fp16 rows of 128 (1.55 GB): one warp per row with 8-byte loads, an IEEE
+// division and a one-element conversion per code took 1,042 us (ALU 48%
+// busy, DRAM 18%); 16 lanes per row with one unit each 349 us (issue 61%
+// busy); 245 us as it is (0.93 of the measured copy rate).
+template <int DT, int LP>
 __global__ void __launch_bounds__(kQuantWarps * 32)
     quantize_kernel(const void* __restrict__ x, int64_t rows, int d, uint8_t* __restrict__ codes,
                     float* __restrict__ scales) {
     const int lane = threadIdx.x & 31;
-    const int ng = d >> 2;
-    for (int64_t r = static_cast<int64_t>(blockIdx.x) * kQuantWarps + (threadIdx.x >> 5); r < rows;
-         r += static_cast<int64_t>(gridDim.x) * kQuantWarps) {
-        float4 v[kMaxGroups];
+    const int l = lane & (LP - 1);
+    const int units = d >> 3;  // per row
+    griddep_wait();
+    griddep_launch_dependents();
+    const int64_t step = static_cast<int64_t>(gridDim.x) * kQuantWarps * (32 / LP);
+    int64_t row = (static_cast<int64_t>(blockIdx.x) * kQuantWarps + (threadIdx.x >> 5)) * (32 / LP) + lane / LP;
+    // rows of one warp step differ by lane: the warp leaves together
+    for (; __any_sync(0xffffffffu, row < rows); row += step) {
+        float v[kQuantUnits][8];
+#pragma unroll
+        for (int g = 0; g < kQuantUnits; ++g) {
+            const int u = l + g * LP;
+            if (row < rows && u < units) {
+                load8<DT>(x, row * units + u, v[g]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[g][i] = 0.f;
+            }
+        }
         float amax = 0.f;
 #pragma unroll
-        for (int g = 0; g < kMaxGroups; ++g) {
-            const int gi = lane + 32 * g;
-            if (gi < ng) {
-                v[g] = load4<DT>(x, r * d + 4 * gi);
-                amax = fmaxf(amax, fmaxf(fmaxf(fabsf(v[g].x), fabsf(v[g].y)), fmaxf(fabsf(v[g].z), fabsf(v[g].w))));
-            }
-        }
-        amax = warp_max(amax);
-        const float s = __fdiv_rn(amax, 448.f);
+        for (int g = 0; g < kQuantUnits; ++g)
 #pragma unroll
-        for (int g = 0; g < kMaxGroups; ++g) {
-            const int gi = lane + 32 * g;
-            if (gi < ng) {
-                const uint32_t w = encode(v[g].x, s) | (encode(v[g].y, s) << 8) | (encode(v[g].z, s) << 16) |
-                                   (encode(v[g].w, s) << 24);
-                *reinterpret_cast<uint32_t*>(codes + r * d + 4 * gi) = w;
+            for (int i = 0; i < 8; i += 2) amax = fmax3(amax, fabsf(v[g][i]), fabsf(v[g][i + 1]));
+#pragma unroll
+        for (int o = LP / 2; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+        const float s = amax >= kQuantMinScale && amax <= kQuantMaxScale ? div_markstein(amax, 448.f, 1.f / 448.f)
+                                                                         : __fdiv_rn(amax, 448.f);
+        if (row < rows) {
+            if (l == 0) scales[row] = s;
+            const bool plain = s >= kQuantMinScale && s <= kQuantMaxScale;
+            const float r = __frcp_rn(s);
+#pragma unroll
+            for (int g = 0; g < kQuantUnits; ++g) {
+                const int u = l + g * LP;
+                if (u >= units) break;
+                float y[8];
+                if (plain) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) y[i] = div_markstein(v[g][i], s, r);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) y[i] = s == 0.f ? 0.f : __fdiv_rn(v[g][i], s);
+                }
+                uint2 w;
+                w.x = encode2(y[0], y[1]) | (encode2(y[2], y[3]) << 16);
+                w.y = encode2(y[4], y[5]) | (encode2(y[6], y[7]) << 16);
+                __stcs(reinterpret_cast<uint2*>(codes) + row * units + u, w);
             }
         }
-        if (lane == 0) scales[r] = s;
     }
+}
+
+// The instantiation for d: a quarter as many lanes per row as it has
+// 8-element units, rounded up to a power of two.
+template <int DT>
+cudaError_t launch_quantize(int sm_count, const void* x, int64_t rows, int d, uint8_t* codes, float* scales,
+                            cudaStream_t stream) {
+    auto go = [&](auto kernel, int lp) {
+        const int64_t per_block = static_cast<int64_t>(kQuantWarps) * (32 / lp);
+        const int64_t want = (rows + per_block - 1) / per_block;
+        const unsigned grid = static_cast<unsigned>(std::min<int64_t>(want, int64_t(sm_count) * 8));
+        return launch_dependent(kernel, dim3(grid), dim3(kQuantWarps * 32), 0, stream, x, rows, d, codes, scales);
+    };
+    const int units = d / 8;
+    if (units <= 4) return go(quantize_kernel<DT, 1>, 1);
+    if (units <= 8) return go(quantize_kernel<DT, 2>, 2);
+    if (units <= 16) return go(quantize_kernel<DT, 4>, 4);
+    if (units <= 32) return go(quantize_kernel<DT, 8>, 8);
+    if (units <= 64) return go(quantize_kernel<DT, 16>, 16);
+    return go(quantize_kernel<DT, 32>, 32);
 }
 
 inline bool aligned4(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0; }
@@ -133,15 +210,12 @@ extern "C" tms_status tms_quantize_e4m3(const void* x, tms_dtype dtype, int64_t 
     DeviceInfo dev;
     tms_status st = current_device(&dev);
     if (st != TMS_OK) return st;
-    const int64_t want = (rows + fp8::kQuantWarps - 1) / fp8::kQuantWarps;
-    const unsigned grid = static_cast<unsigned>(std::min<int64_t>(want, int64_t(dev.sm_count) * 8));
-    const unsigned threads = fp8::kQuantWarps * 32;
     switch (dtype) {
-        case TMS_F16: fp8::quantize_kernel<TMS_F16><<<grid, threads, 0, stream>>>(x, rows, d, codes, scales); break;
-        case TMS_BF16: fp8::quantize_kernel<TMS_BF16><<<grid, threads, 0, stream>>>(x, rows, d, codes, scales); break;
-        default: fp8::quantize_kernel<TMS_F32><<<grid, threads, 0, stream>>>(x, rows, d, codes, scales); break;
+        case TMS_F16: return launch_status(fp8::launch_quantize<TMS_F16>(dev.sm_count, x, rows, d, codes, scales, stream));
+        case TMS_BF16:
+            return launch_status(fp8::launch_quantize<TMS_BF16>(dev.sm_count, x, rows, d, codes, scales, stream));
+        default: return launch_status(fp8::launch_quantize<TMS_F32>(dev.sm_count, x, rows, d, codes, scales, stream));
     }
-    return launch_status(cudaGetLastError());
 }
 
 namespace tms {

@@ -77,6 +77,28 @@ def test_quantize_bit_exact(cuda_lib, dtype, d):
     assert tms.device_error() == 0
 
 
+@pytest.mark.parametrize("dtype", ["f16", "bf16", "f32"])
+@pytest.mark.parametrize("rows,d", [(1, 32), (33, 48), (257, 64), (1031, 112), (65, 256), (7, 272), (41, 512), (19, 528)])
+def test_quantize_lane_layouts_and_extreme_scales(cuda_lib, dtype, rows, d):
+    """Every lanes-per-row split (units a power of two and not), row counts
+    that fill no block evenly, signed zeros, and (bf16 / fp32) rows whose
+    scale is too small or too large for the reciprocal-based quotient:
+    bit-exact against the oracle's IEEE divisions."""
+    from paper_2606_26439_gb300 import tms
+    g = np.random.default_rng(1000 * rows + d)
+    x = synth.unit_rows(rows, d, d, 5)
+    if dtype != "f16":
+        x *= 10.0 ** g.uniform(-36, 36, size=(rows, 1))
+    x[:, 1] = -0.0
+    x[rows // 2, 2:] = 0.0
+    xt = synth.cast(x, dtype)
+    want_c, want_s = _quantize_host(xt)
+    x_d, = gc.to_dev(xt)
+    codes, scales = tms.quantize_e4m3(x_d)
+    assert np.array_equal(scales.cpu().numpy().view(np.uint32), want_s.view(np.uint32))
+    assert np.array_equal(codes.cpu().numpy(), want_c)
+
+
 def test_quantize_rejects_bad_width(cuda_lib):
     import torch
     from paper_2606_26439_gb300 import tms
