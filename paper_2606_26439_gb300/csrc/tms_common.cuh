@@ -60,13 +60,11 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Wait for the phase of `bar` with parity `parity` to complete.  Returns
-// false (and raises the abort flag) once `budget` SM cycles have passed
-// (<= 0: kWaitBudgetCycles), or when another role of the CTA has already
-// aborted.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                          unsigned int* err, long long budget) {
-    if (mbar_try_wait(bar, parity)) return true;
+// The rest of mbar_wait once the phase was not complete at first: kept out
+// of line, since every role of a kernel waits at several places and the
+// roles' loops share the SM's instruction caches.
+static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                                   unsigned int* err, long long budget) {
     const long long limit = budget > 0 ? budget : kWaitBudgetCycles;
     const long long t0 = clock64();
     for (uint32_t it = 1;; ++it) {
@@ -80,6 +78,23 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
             }
         }
     }
+}
+
+// Wait for the phase of `bar` with parity `parity` to complete.  Returns
+// false (and raises the abort flag) once `budget` SM cycles have passed
+// (<= 0: kWaitBudgetCycles), or when another role of the CTA has already
+// aborted.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                          unsigned int* err, long long budget) {
+    if (mbar_try_wait(bar, parity)) return true;
+    return mbar_wait_slow(bar, parity, abort_flag, err, budget);
+}
+
+// True in one lane of a converged warp, always the same one.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
 }
 
 // 2-D tiled TMA load of box (x, y) of `map` into shared memory, completing

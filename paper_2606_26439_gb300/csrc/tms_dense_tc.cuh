@@ -17,19 +17,18 @@
 // (token blocks of one query, or the queries of a shared group) are
 // replicated down the 128 rows when they are fewer.
 //
-// Super-tiles: consecutive document tiles (up to 128 rows each, padded to
-// 8) are packed side by side into one super-tile of up to 256 rows (128
-// with two query halves), and one run of MMAs (N = the packed rows rounded
-// up to 16) scores them all.  The per-tile costs of the pipeline --
-// barrier round trips, commits, MMA issue -- are paid once per super-tile,
-// typically two to three documents.
+// Super-tiles: consecutive documents are packed in units of 8 rows, side by
+// side, into one super-tile of up to 256 or 128 rows, and one run of MMAs
+// (N = the packed rows rounded up to 16) scores them all.  The per-tile
+// costs of the pipeline -- barrier round trips, commits, MMA issue -- are
+// paid once per super-tile, typically two to three documents.
 //
 //   * Planner warp: takes the candidates 32 at a time, one per lane
 //     (metadata, validity, query, -inf / NaN for empty / bad documents),
-//     packs their tiles into super-tiles and publishes each super-tile as
-//     one record -- header plus tile list -- with a single barrier
-//     arrival.  It also loads each query's tile (replicated, see above)
-//     and, F8, every tile's row scales through a ring of small TMA loads.
+//     places their units in super-tiles with one scan and publishes each
+//     super-tile as one record -- header, tile list, documents that end in
+//     it -- with a single barrier arrival.  It also loads each query's tile
+//     (replicated, see above).
 //   * Loader warp: streams each super-tile from HBM into a ring of shared-
 //     memory chunk stages (STR rows x 128 bytes: 64 fp16/bf16 or 128 E4M3
 //     elements per row), one TMA box per tile and chunk, the tiles issued
@@ -46,16 +45,15 @@
 //     accumulating the partial dot products in tensor memory before any
 //     max is taken -- the paper's dimension tiling (Section 3), with the K
 //     loop running through TMEM.
-//   * Four epilogue warps: thread = query row (TMEM lane).  Documents are
-//     dealt round-robin to the copies of the query tile; the warps of a
-//     copy load their document's columns with tcgen05.ld, multiply column
-//     j by document row j's scale (F8), drop columns of other documents,
-//     and fold the rest into a running max.  At the document's end each
-//     warp sums its 32 query tokens (times their scales, F8); with one
-//     token block per copy that sum is the score, else the copy's warps
-//     add their sums in block order.  Each score is written once; the
-//     Nq x Nd similarity matrix never reaches HBM and no atomics or memset
-//     are needed.
+//   * Epilogue warps: thread = query row (TMEM lane).  Each warp takes its
+//     share of a super-tile's columns with tcgen05.ld, multiplies column j
+//     by document row j's scale (F8), and reduces them to a running max
+//     that starts again after each document's end; the values at documents'
+//     ends and at the end of its share go to shared memory.
+//   * Finisher warps: combine those values into each document's row maxima
+//     and sum them over the query tokens (times their scales, F8).  Each
+//     score is written once; the Nq x Nd similarity matrix never reaches
+//     HBM and no atomics or memset are needed.
 //
 // Every wait is bounded (see tms_common.cuh); a timeout sets
 // TMS_DEVERR_TIMEOUT and the CTA drains its in-flight copies and MMAs,
@@ -90,47 +88,57 @@ constexpr int kMaxSeg = 32;                   // tiles per super-tile (each >= 8
 // run ahead of the epilogue: with HBM latencies of a few microseconds under
 // load, the loads of many super-tiles must be in flight at once.
 __host__ __device__ constexpr int st_ring(int) { return 16; }
-constexpr int kEpiWarps = 4;
-constexpr int kLoaderWarp = 2 + kEpiWarps;
-constexpr int kThreads = 32 * (kLoaderWarp + 1);  // planner, MMA, four epilogue warps, loader
-constexpr int kSplitWarps = 4;                    // TF: splitter warps after the loader; kPQ: decompressors
-__host__ __device__ constexpr int kernel_threads(int kind) {
-    return kThreads + ((kind == kTF32 || kind == kPQ) ? 32 * kSplitWarps : 0);
+// Epilogue warps: one per tensor-memory lane quarter and query half.
+__host__ __device__ constexpr int epi_warps(int h) { return 4 * h; }
+constexpr int kSplitWarps = 4;  // TF: splitter warps after the loader; kPQ: decompressors
+// Finisher warps: they take the 32-row blocks of a super-tile in turn (two
+// blocks each for eight queries, all of a query's blocks for one).
+__host__ __device__ constexpr int fin_warps(bool sh) { return sh ? 4 : 1; }
+__host__ __device__ constexpr int fin_blocks(int h, bool sh) { return sh ? h : 4; }
+// planner, MMA, epilogue warps, loader, finishers, splitters / decompressors
+__host__ __device__ constexpr int kernel_threads(int kind, int h, bool sh) {
+    return 32 * (3 + epi_warps(h) + fin_warps(sh) + ((kind == kTF32 || kind == kPQ) ? kSplitWarps : 0));
 }
-// Accumulator buffers (each H x STR tensor-memory columns): as many as the
-// SM's 512 columns hold for the CTAs sharing it, at most one per epilogue
-// warp.
-__host__ __device__ constexpr int acc_count(int h, int str, int ctas) {
-    return 512 / (h * str * ctas) < kEpiWarps ? 512 / (h * str * ctas) : kEpiWarps;
+// Accumulator buffers of STR tensor-memory columns -- one holds one query
+// half of a super-tile -- as many as the SM's 512 columns give the CTAs
+// sharing it, at most four.
+__host__ __device__ constexpr int acc_count(int str, int ctas) {
+    return 512 / (str * ctas) < 4 ? 512 / (str * ctas) : 4;
 }
-constexpr int kMaxAcc = kEpiWarps;
 constexpr int kMaxStages = 16;
 constexpr int kSmemLimit = 232448;            // 227 KB opt-in maximum per CTA
 
-enum : int { kFirst = 1, kLast = 2, kEnd = 4, kStFirst = 8, kStLast = 16 };
+enum : int { kEnd = 1 };
 
-// One document tile inside a super-tile (16 bytes).
+// A super-tile is filled in units of 8 rows, each of one document: a document
+// of n tokens takes ceil(n / 8) units, the last of them partial (rows of the
+// next document past its end, dropped by the epilogue) if n % 8 != 0.
+
+// One document tile inside a super-tile: consecutive token rows.
 struct SegInfo {
-    int f;        // flat candidate index (shared mode: position in the candidate list)
-    int row0;     // token row of the tile's first row
-    short r;      // valid rows (1..128)
-    short col;    // first column (row of the super-tile), a multiple of 8
-    int flags;    // kFirst / kLast of the document
+    int row0;       // token row of the tile's first row
+    uint8_t nu;     // units (1..16)
+    uint8_t cu;     // first unit of the super-tile
+    uint16_t rows;  // rows that count (8 nu but for a partial last unit)
 };
 
 // One super-tile record (planner -> loader, MMA thread and epilogue).
 struct StHdr {
-    int q;      // query (group) whose tile it is scored against
-    int n;      // MMA N: packed rows rounded up to 16
-    int nseg;   // tiles
-    int flags;  // kEnd
-    int rows;   // packed rows (sum of the tiles' rows rounded up to 8)
-    int pad[3];
+    int q;            // query (group) whose tile it is scored against
+    int n;            // MMA N: packed rows rounded up to 16
+    int nseg;         // tiles
+    int flags;        // kEnd
+    int rows;         // packed rows: 8 x units
+    uint32_t ends;     // bit u: unit u is the last of a document (f[] in that order)
+    uint32_t partial;  // bit u: and not all of its rows count
+    int pad;
 };
 
 struct StSlot {
     StHdr h;
     SegInfo seg[kMaxSeg];
+    int f[kMaxSeg];          // documents that end here: flat candidate index (shared mode: position in the list)
+    uint8_t valid[kMaxSeg];  // by unit, where a document ends: its rows that count (1..8)
 };
 
 struct Args {
@@ -164,21 +172,28 @@ struct Args {
     int fault;                  // diagnostics: kFaultHoldAccumulator, else 0
 };
 
+// Stands in for the row scale of a column past its document's end.
+static __device__ const float kNanScale = __builtin_nanf("");
+
 // Diagnostics (tms_debug_set): the MMA thread of CTA 0 never signals its
 // first accumulator, so that CTA's epilogue wait runs out of budget and the
 // timeout path -- flag, abort, drain, tensor-memory release -- runs.
 constexpr int kFaultHoldAccumulator = TMS_FAULT_HOLD_ACCUMULATOR;
 
 struct Layout {
-    int q_off, qlo_off, stage_off, stage_stride, part_off, fin_off, sc_off, cb_off, code_off, st_off, bar_off, misc_off,
-        total;
+    int q_off, qlo_off, stage_off, stage_stride, um_off, um_stride, fin_off, sc_off, cb_off, code_off, st_off, bar_off,
+        misc_off, total;
 };
 
-// Finished documents waiting for their sum over query tokens, per epilogue
-// warp: kFinRows rows of 32 row maxima (one row per document and query
-// half), padded to 33 floats so that lane r reading row r walks distinct
-// banks, then each document's (candidate, query) pair.
-constexpr int kFinRows = 16;
+// Super-tiles whose unit maxima may wait for the finishers.  One is enough
+// where the MMAs of a super-tile take far longer than finishing one (three or
+// more dimension chunks), and leaves room for another chunk stage.
+__host__ __device__ constexpr int um_slots(int nchunks) { return nchunks >= 3 ? 1 : 2; }
+// Finished documents waiting for their sum over query tokens, per finisher
+// warp: kFinRows rows of 32 row maxima (one row per document and 32-row
+// block), padded to 33 floats so that lane r reading row r walks distinct
+// banks, then each row's (candidate, query or query of the group) pair.
+constexpr int kFinRows = 8;
 constexpr int kFinWarpBytes = kFinRows * 33 * 4 + kFinRows * 8;
 
 // Shared-memory carve-up; the same arithmetic runs on host and device.
@@ -193,7 +208,7 @@ constexpr int kFinWarpBytes = kFinRows * 33 * 4 + kFinRows * 8;
 // each chunk stage holds the str document rows, then the qrows query rows
 // of the same dimension chunk.
 __host__ __device__ inline Layout make_layout(int stages, int qslots, int nchunks, int rows_alloc, int str, int kind,
-                                              int kacc, bool fin, int qrows) {
+                                              int kacc, int blocks, int fins, int qrows) {
     const bool f8 = kind == kE4M3;
     const int twin = kind == kTF32 ? 2 : 1;
     Layout L;
@@ -201,15 +216,15 @@ __host__ __device__ inline Layout make_layout(int stages, int qslots, int nchunk
     L.qlo_off = qslots * nchunks * rows_alloc * 128;
     L.stage_off = (twin * L.qlo_off + 1023) & ~1023;
     L.stage_stride = twin * (str + qrows) * 128;
-    L.part_off = L.stage_off + stages * L.stage_stride;
-    L.fin_off = L.part_off + 128;  // after [2 copies][2 parities][4 blocks] partial sums
-    L.sc_off = L.fin_off + (fin ? kEpiWarps * kFinWarpBytes : 0);  // 128-byte aligned
+    L.um_off = L.stage_off + stages * L.stage_stride;
+    L.um_stride = (str / 8) * blocks * 128;  // [unit][32-row block][row] unit maxima
+    L.fin_off = L.um_off + um_slots(nchunks) * L.um_stride;
+    L.sc_off = (L.fin_off + fins * kFinWarpBytes + 127) & ~127;
     L.cb_off = L.sc_off + (f8 ? st_ring(str) * str * 4 : 0);  // F8: [st_ring][str] column scales
     L.code_off = L.cb_off + (kind == kPQ ? kPqCbBytes : 0);                        // kPQ: fp16 codebook
-    // kPQ: code-row ring, then per slot the valid rows of each 8-row group
-    L.st_off = L.code_off + (kind == kPQ ? kCodeRing * (str * kPqM + kMaxSeg * 4) : 0);
+    L.st_off = L.code_off + (kind == kPQ ? kCodeRing * str * kPqM : 0);  // kPQ: code-row ring
     L.bar_off = L.st_off + st_ring(str) * static_cast<int>(sizeof(StSlot));
-    const int nbar = 3 * stages + 2 * kacc + 3 * qslots + 3 * st_ring(str) + 8 + 1 + 2 * kCodeRing;
+    const int nbar = 3 * stages + 2 * kacc + 3 * qslots + 3 * st_ring(str) + 4 + 1 + 2 * kCodeRing;
     L.misc_off = L.bar_off + nbar * 8;
     L.total = L.misc_off + 16;
     return L;
@@ -249,23 +264,11 @@ __device__ __forceinline__ int meta_status(const Args& a, int id, int64_t off, i
     return (len < 0 || off < 0 || off + len > a.n_tokens) ? 2 : 0;
 }
 
-// Lane 0 polls the barrier and broadcasts the outcome; the warp barrier
-// orders the other lanes after lane 0's acquire.  For barriers guarding
-// data written by other threads or ordering tensor-core work.  Returns
-// false on timeout / abort.
+// Every lane waits, and so observes the phase (and what it publishes)
+// itself; the vote makes the outcome the warp's.  Returns false on timeout /
+// abort.
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                           unsigned int* err, long long budget) {
-    int ok = 1;
-    if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, abort_flag, err, budget) ? 1 : 0;
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    __syncwarp();
-    return ok != 0;
-}
-
-// Every lane waits (and so observes the phase itself): for barriers that
-// complete the TMA bytes the lanes then read.
-__device__ __forceinline__ bool warp_wait_all(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                              unsigned int* err, long long budget) {
     const bool ok = mbar_wait(bar, parity, abort_flag, err, budget);
     return __all_sync(0xffffffffu, ok) != 0;
 }
@@ -283,43 +286,20 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
 // reads from an fp32 element.
 __device__ __forceinline__ float tf32_trunc(float x) { return __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
 
-// Maxima of the four 8-column sub-blocks of 32 accumulator columns.
-// Document tiles start on 8-column boundaries, so a tile covers whole
-// sub-blocks except, at a document's end, a last partial one.
-__device__ __forceinline__ void sub_maxima8(const float (&v)[32], float (&sb)[4]) {
+// Maxima of the four units (8 columns each) of 32 accumulator columns.
+__device__ __forceinline__ void unit_maxima(const float (&v)[32], float (&um)[4]) {
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-        sb[k] = fmax3(fmax3(v[8 * k], v[8 * k + 1], v[8 * k + 2]), fmax3(v[8 * k + 3], v[8 * k + 4], v[8 * k + 5]),
+        um[k] = fmax3(fmax3(v[8 * k], v[8 * k + 1], v[8 * k + 2]), fmax3(v[8 * k + 3], v[8 * k + 4], v[8 * k + 5]),
                       fmaxf(v[8 * k + 6], v[8 * k + 7]));
 }
 
-// max(m, v[lo..hi)) for 0 <= lo < hi <= 32 with lo a multiple of 8: the
-// whole sub-blocks from their maxima sb, a partial last one (hi not a
-// multiple of 8) from its hi % 8 leading columns.  A tile covering the
-// whole group (the common case inside long documents) takes one branch
-// and two maxima.
-__device__ __forceinline__ float fold_cols(float m, const float (&v)[32], const float (&sb)[4], int lo, int hi) {
-    if (lo == 0 && hi == 32) return fmax3(m, fmax3(sb[0], sb[1], sb[2]), sb[3]);
-    const int kl = lo >> 3;
-    const int kf = hi >> 3;
-    // sub-blocks [kl, kf) as a 4-bit mask
-    const uint32_t whole = (0xfu >> (4 - kf)) & ~((1u << kl) - 1u);
-    float x[4];
+// Max of the first n (1..8) columns of unit K.
+template <int K>
+__device__ __forceinline__ float unit_max_n(const float (&v)[32], int n) {
+    float m = v[8 * K];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) x[k] = (whole >> k) & 1u ? sb[k] : -INFINITY;
-    m = fmax3(m, fmax3(x[0], x[1], x[2]), x[3]);
-    const int rem = hi & 7;
-    if (rem != 0) {  // sub-block kf < 4 holds rem columns of the tile
-        // the sub-block's first 7 columns, picked by kf, then masked to rem
-        float y[7];
-#pragma unroll
-        for (int j = 0; j < 7; ++j) {
-            const float lo2 = (kf & 1) ? v[8 + j] : v[j];
-            const float hi2 = (kf & 1) ? v[24 + j] : v[16 + j];
-            y[j] = j < rem ? ((kf & 2) ? hi2 : lo2) : -INFINITY;
-        }
-        m = fmax3(m, fmax3(y[0], y[1], y[2]), fmax3(y[3], y[4], fmaxf(y[5], y[6])));
-    }
+    for (int j = 1; j < 8; ++j) m = j < n ? fmaxf(m, v[8 * K + j]) : m;
     return m;
 }
 
@@ -333,8 +313,8 @@ struct Maps {
 
 // H: 128-row halves of the query tile (2 for a shared group of 8 queries).
 // STR: rows per super-tile (MMA N at most), 256 or 128.  CTAS: CTAs per SM
-// (1 or 2); the CTA holds KACC = acc_count(H, STR, CTAS) accumulators of
-// H x STR tensor-memory columns.
+// (1 or 2); the CTA holds KACC = acc_count(STR, CTAS) accumulators of STR
+// tensor-memory columns; half h of super-tile t is accumulator use H t + h.
 // SH (shared mode): the launch's queries all score one candidate list; a
 // "query" of the pipeline is then a group of up to 4 H queries stacked in
 // M, so each document tile is read once per group, and the epilogue
@@ -342,15 +322,19 @@ struct Maps {
 // F8: rows are E4M3 codes; similarities are scaled by the document row's
 // scale before the max and by the query token's scale before the sum.
 template <int H, int STR, int CTAS, bool SH, int KIND>
-__global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
+__global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
     dense_tc_kernel(const __grid_constant__ Maps maps, const Args a) {
     constexpr bool F8 = KIND == kE4M3;
     constexpr bool TF = KIND == kTF32;
     constexpr bool PQ = KIND == kPQ;
     constexpr int CE = chunk_elems(KIND);
     constexpr int STAGE_BYTES = STR * 128;
-    constexpr int KACC = acc_count(H, STR, CTAS);
-    constexpr uint32_t TCOLS = KACC * H * STR;
+    constexpr int KACC = acc_count(STR, CTAS);
+    constexpr uint32_t TCOLS = KACC * STR;
+    constexpr int kEpiWarps = epi_warps(H);
+    constexpr int kLoaderWarp = 2 + kEpiWarps;
+    constexpr int kFinWarp = kLoaderWarp + 1;              // the first of them
+    constexpr int kHelpWarp = kFinWarp + fin_warps(SH);    // TF / kPQ: the first splitter / decompressor
     constexpr int kStRing = st_ring(STR);
     static_assert(KACC >= 2 && TCOLS * CTAS <= 512, "tensor memory of one SM");
 
@@ -361,19 +345,19 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
     const int NCH = a.nchunks;
     const int qslot_bytes = NCH * a.rows_alloc * 128;
     const bool QSTREAM = QS == 0;  // the query rows come with every chunk stage
-    const Layout L = make_layout(S, QS, NCH, a.rows_alloc, STR, KIND, KACC, SH || a.bpc == 1, QSTREAM ? 128 * H : 0);
+    const Layout L = make_layout(S, QS, NCH, a.rows_alloc, STR, KIND, KACC, a.bpc, fin_warps(SH), QSTREAM ? 128 * H : 0);
+    const int UMS = um_slots(NCH);
     const int SSTRIDE = L.stage_stride;  // bytes between stages (TF: hi, then lo)
 
     uint8_t* q_base = smem + L.q_off;
     uint8_t* qlo_base = smem + L.qlo_off;  // TF: the lo twin of the query region
     uint8_t* stage_base = smem + L.stage_off;
-    float* part = reinterpret_cast<float*>(smem + L.part_off);  // [copy][parity][block]
-    uint8_t* fin_base = smem + L.fin_off;                       // [epilogue warp] finished-document rows
+    uint8_t* um_base = smem + L.um_off;    // [UMS][unit][block][row] unit maxima
+    uint8_t* fin_base = smem + L.fin_off;  // [finisher warp] finished-document rows
     float* sc = reinterpret_cast<float*>(smem + L.sc_off);      // F8: [kStRing][STR] scale of each column
     StSlot* slots = reinterpret_cast<StSlot*>(smem + L.st_off);
     uint8_t* cb = smem + L.cb_off;           // kPQ: fp16 codebook, entry (code, m) at (code * 16 + m) * 16
     uint8_t* code_ring = smem + L.code_off;  // kPQ: [kCodeRing][STR rows][16] code bytes
-    uint8_t* gvalid = code_ring + kCodeRing * STR * kPqM;  // kPQ: [kCodeRing][STR / 8] valid rows per 8-row group
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.bar_off);
     uint64_t* full = bars;
     uint64_t* empty = full + S;
@@ -383,9 +367,9 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
     uint64_t* qempty = qfull + QS;
     uint64_t* xfull = qempty + QS;          // [kStRing]
     uint64_t* xempty = xfull + kStRing;     // [kStRing]
-    uint64_t* pfull = xempty + kStRing;     // [copy][parity]
-    uint64_t* pempty = pfull + 4;           // [copy][parity]
-    uint64_t* scfull = pempty + 4;          // F8: [kStRing] a record slot's column scales landed
+    uint64_t* umfull = xempty + kStRing;    // [UMS <= 2] unit maxima written
+    uint64_t* umempty = umfull + 2;         // [UMS <= 2] unit maxima read
+    uint64_t* scfull = umempty + 2;          // F8: [kStRing] a record slot's column scales landed
     uint64_t* mdone = scfull + kStRing;
     uint64_t* conv = mdone + 1;   // TF: [S] stage split
     uint64_t* qconv = conv + S;   // TF: [QS] query tile split
@@ -394,7 +378,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L.misc_off);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L.misc_off + 4);
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);  // the same in every lane
     const int lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -404,8 +388,8 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
         }
         for (int i = 0; i < KACC; ++i) {
             mbar_init(&tfull[i], 1);
-            // the active epilogue warps: those whose row block belongs to a copy
-            mbar_init(&tempty[i], a.reps * a.bpc < kEpiWarps ? a.reps * a.bpc : kEpiWarps);
+            // the epilogue warps of a half whose row block belongs to a copy
+            mbar_init(&tempty[i], a.reps * a.bpc < 4 ? a.reps * a.bpc : 4);
         }
         for (int i = 0; i < QS; ++i) {
             mbar_init(&qfull[i], 1);
@@ -413,11 +397,13 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
         }
         for (int i = 0; i < kStRing; ++i) {
             mbar_init(&xfull[i], 1);
-            mbar_init(&xempty[i], 2 + kEpiWarps + ((TF || PQ) ? kSplitWarps : 0));  // loader, MMA, epilogue, splitters
+            // loader, MMA, epilogue, finishers, splitters
+            mbar_init(&xempty[i], 2 + kEpiWarps + fin_warps(SH) + ((TF || PQ) ? kSplitWarps : 0));
         }
-        for (int i = 0; i < 4; ++i) {
-            mbar_init(&pfull[i], a.bpc);
-            mbar_init(&pempty[i], 1);
+        for (int i = 0; i < 2; ++i) {
+            // the epilogue warps whose row block belongs to a copy
+            mbar_init(&umfull[i], H == 2 ? 8 : (a.reps * a.bpc < 4 ? a.reps * a.bpc : 4));
+            mbar_init(&umempty[i], fin_warps(SH));
         }
         for (int i = 0; i < kStRing; ++i) mbar_init(&scfull[i], 32);  // one cp.async arrival per loader lane
         mbar_init(mdone, 1);
@@ -472,39 +458,31 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
         int tst = 0;   // super-tiles published
         int qi = 0, cur_q = -1;
         bool aborted = false;
-        // The open super-tile: its tile i lives in lane i's registers.
-        int nseg = 0, rows_used = 0, st_q = 0;
-        int my_f = 0, my_r = 0, my_flags = 0, my_row0 = 0, my_col = 0;
+        // The open super-tile, written into its record slot as it fills.
+        int used = 0, nseg = 0, nfin = 0, st_q = 0;  // units, tiles, documents ended, query
+        unsigned ends = 0, partial = 0;
 
         // Publish the open super-tile: the record, and the query tile if the
         // query changed.
         auto close_st = [&]() -> bool {
-            const bool has = lane < nseg;
             const int xs = tst % kStRing;
-            if (!warp_wait(&xempty[xs], ((tst / kStRing) & 1) ^ 1, abort_flag, a.err, a.budget)) return false;
-            StSlot* x = &slots[xs];
-            if (has) {
-                SegInfo si;
-                si.f = my_f;
-                si.row0 = my_row0;
-                si.r = static_cast<short>(my_r);
-                si.col = static_cast<short>(my_col);
-                si.flags = my_flags;
-                x->seg[lane] = si;
-            }
             if (lane == 0) {
                 StHdr h;
                 h.q = st_q;
-                h.n = (rows_used + 15) & ~15;
+                h.n = (8 * used + 15) & ~15;
                 h.nseg = nseg;
                 h.flags = 0;
-                h.rows = rows_used;
-                h.pad[0] = h.pad[1] = h.pad[2] = 0;
-                x->h = h;
+                h.rows = 8 * used;
+                h.ends = ends;
+                h.partial = partial;
+                h.pad = 0;
+                slots[xs].h = h;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&xfull[xs]);
             ++tst;
+            used = nseg = nfin = 0;
+            ends = partial = 0;
             // A new query's rows go to the next query slot.  The record is
             // published first: the MMA thread releases the old slot only
             // once it sees the new query.
@@ -531,8 +509,6 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
                 ++qi;
                 cur_q = st_q;
             }
-            nseg = 0;
-            rows_used = 0;
             return true;
         };
 
@@ -587,37 +563,91 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
                 }
                 if (status != 0) atomicOr(a.err, status == 1 ? TMS_DEVERR_BAD_ID : TMS_DEVERR_BAD_RANGE);
             }
-            // pack the window's documents, in order, into super-tiles
-            unsigned docs = __ballot_sync(0xffffffffu, valid && status == 0 && cur.len > 0);
+            // Pack the window's documents, in order, into super-tiles: lane =
+            // document, [b, e) its units counted from the open super-tile's
+            // start.  Tiles of at most kRows rows fill a super-tile to its
+            // last unit: a document that does not fit is cut at the
+            // super-tile's end and continues in the next one.  All documents
+            // of one query are placed by one scan, and each super-tile they
+            // reach costs a fixed number of warp steps, whatever it holds
+            // (a loop over the documents, a few shuffles each, took ~1,500
+            // cycles per super-tile and bounded every 128-byte-row launch).
+            const int len = valid && status == 0 ? cur.len : 0;
+            const int nu = static_cast<int>((static_cast<unsigned>(len) + 7u) >> 3);
+            const bool huge = __any_sync(0xffffffffu, nu > (1 << 25));  // then one by one: their sum may not fit
+            int incl = nu;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += x;
+            }
+            const int fi = static_cast<int>(SH ? pos : f);
+            const int row = static_cast<int>(cur.off);
+            constexpr int C = STR / 8;  // units of a super-tile
+            unsigned docs = __ballot_sync(0xffffffffu, nu > 0);
             while (docs != 0u) {
-                const int i = __ffs(docs) - 1;
-                docs &= docs - 1u;
-                const int len = __shfl_sync(0xffffffffu, cur.len, i);
-                const int off = static_cast<int>(__shfl_sync(0xffffffffu, cur.off, i));
-                const int q = __shfl_sync(0xffffffffu, ql, i);
-                const int fi = static_cast<int>(__shfl_sync(0xffffffffu, SH ? pos : f, i));
-                // Tiles of at most kRows rows fill the open super-tile to its
-                // last 8-row group: a document that does not fit is cut at
-                // the super-tile's end and continues in the next one.
-                for (int r0 = 0; r0 < len;) {
-                    if (nseg > 0 && (q != st_q || rows_used == STR || nseg == STR / 8)) {
-                        if (!close_st()) {
-                            aborted = true;
-                            break;
+                const int first = __ffs(docs) - 1;
+                const int q = __shfl_sync(0xffffffffu, ql, first);
+                unsigned run = __ballot_sync(0xffffffffu, ql == q) & docs;  // consecutive among the documents
+                if (huge) run &= 0u - run;
+                docs &= ~run;
+                if (used > 0 && q != st_q && !close_st()) {
+                    aborted = true;
+                    break;
+                }
+                st_q = q;
+                const int base = used - __shfl_sync(0xffffffffu, incl - nu, first);
+                const bool in = (run >> lane) & 1u;
+                int e = huge ? used + nu : base + incl, b = e - nu;
+                int end = __shfl_sync(0xffffffffu, e, 31 - __clz(run));  // units from the open super-tile's start
+                int done = 0;  // units of this lane's document in earlier super-tiles
+                for (;;) {
+                    const int xs = tst % kStRing;
+                    if (used == 0 && !warp_wait(&xempty[xs], ((tst / kStRing) & 1) ^ 1, abort_flag, a.err, a.budget)) {
+                        aborted = true;
+                        break;
+                    }
+                    StSlot* x = &slots[xs];
+                    const int lo = max(b, 0), hi = min(e, C);
+                    const int n = in && hi > lo ? hi - lo : 0;  // units here: one tile, or two if more than kRows rows
+                    const bool two = n > kRows / 8;
+                    const bool last = n > 0 && e <= C;
+                    const unsigned m1 = __ballot_sync(0xffffffffu, n > 0), m2 = __ballot_sync(0xffffffffu, two);
+                    const unsigned ml = __ballot_sync(0xffffffffu, last);
+                    const unsigned below = (1u << lane) - 1u;
+                    if (n > 0) {
+                        SegInfo* sg = x->seg + nseg + __popc(m1 & below) + __popc(m2 & below);
+                        const int rows = min(8 * n, len - 8 * done);
+                        sg->row0 = row + 8 * done;
+                        sg->nu = static_cast<uint8_t>(two ? kRows / 8 : n);
+                        sg->cu = static_cast<uint8_t>(lo);
+                        sg->rows = static_cast<uint16_t>(min(rows, kRows));
+                        if (two) {
+                            sg[1].row0 = row + 8 * done + kRows;
+                            sg[1].nu = static_cast<uint8_t>(n - kRows / 8);
+                            sg[1].cu = static_cast<uint8_t>(lo + kRows / 8);
+                            sg[1].rows = static_cast<uint16_t>(rows - kRows);
                         }
+                        if (last) {
+                            x->f[nfin + __popc(ml & below)] = fi;
+                            x->valid[hi - 1] = static_cast<uint8_t>(len - 8 * (nu - 1));
+                        }
+                        done += n;
                     }
-                    if (nseg == 0) st_q = q;
-                    const int r = min(min(kRows, len - r0), STR - rows_used);
-                    if (lane == nseg) {
-                        my_f = fi;
-                        my_r = r;
-                        my_flags = (r0 == 0 ? kFirst : 0) | (r0 + r >= len ? kLast : 0);
-                        my_row0 = off + r0;
-                        my_col = rows_used;
+                    const unsigned bit = last ? 1u << (hi - 1) : 0u;
+                    ends |= __reduce_or_sync(0xffffffffu, bit);
+                    partial |= __reduce_or_sync(0xffffffffu, (len & 7) != 0 ? bit : 0u);
+                    nseg += __popc(m1) + __popc(m2);
+                    nfin += __popc(ml);
+                    used = min(end, C);
+                    if (used == C && !close_st()) {
+                        aborted = true;
+                        break;
                     }
-                    rows_used += (r + 7) & ~7;
-                    ++nseg;
-                    r0 += r;
+                    if (end <= C) break;
+                    b -= C;
+                    e -= C;
+                    end -= C;
                 }
                 if (aborted) break;
             }
@@ -626,7 +656,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
             nxt = load_meta(a, id_next2);
             id_next2 = load_id(a, k0 + 96 + lane);
         }
-        if (!aborted && nseg > 0 && !close_st()) aborted = true;
+        if (!aborted && used > 0 && !close_st()) aborted = true;
         if (!aborted) {
             const int xs = tst % kStRing;
             if (warp_wait(&xempty[xs], ((tst / kStRing) & 1) ^ 1, abort_flag, a.err, a.budget) && lane == 0) {
@@ -636,7 +666,9 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
                 h.nseg = 0;
                 h.flags = kEnd;
                 h.rows = 0;
-                h.pad[0] = h.pad[1] = h.pad[2] = 0;
+                h.ends = 0;
+                h.partial = 0;
+                h.pad = 0;
                 slots[xs].h = h;
                 mbar_arrive(&xfull[xs]);
             }
@@ -662,9 +694,9 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
             int r = 0, row0 = 0, col = 0;
             if (has) {
                 const SegInfo si = slots[xs].seg[lane];
-                r = si.r;
                 row0 = si.row0;
-                col = si.col;
+                col = 8 * si.cu;
+                r = si.rows;
             }
             int bytes = r * kPqM;
 #pragma unroll
@@ -673,10 +705,6 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
             if (lane == 0) mbar_arrive(&xempty[xs]);
             const int cs = t % kCodeRing;
             if (!warp_wait(&codeempty[cs], ((t / kCodeRing) & 1) ^ 1, abort_flag, a.err, a.budget)) break;
-            if (has)  // valid rows of each 8-row group of this tile (a prefix of the group)
-                for (int g8 = 0; g8 < (r + 7) >> 3; ++g8)
-                    gvalid[cs * (STR / 8) + (col >> 3) + g8] = static_cast<uint8_t>(min(8, r - 8 * g8));
-            __syncwarp();
             if (lane == 0) mbar_arrive_expect_tx(&codefull[cs], static_cast<uint32_t>(bytes));
             __syncwarp();
             if (has)
@@ -705,28 +733,34 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
             const StHdr h = slots[xs].h;
             if (h.flags & kEnd) break;
             const bool has = lane < h.nseg;
-            int n8 = 8, row0 = 0, col = 0, rr = 0;
+            int n8 = 8, row0 = 0, col = 0, rend = 0;
             if (has) {
                 const SegInfo si = slots[xs].seg[lane];
-                rr = si.r;
-                n8 = (si.r + 7) & ~7;
+                n8 = 8 * si.nu;
                 row0 = si.row0;
-                col = si.col;
+                col = 8 * si.cu;
+                rend = col + si.rows;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&xempty[xs]);
             if (F8) {
                 // Each tile's row scales to its columns of the record slot's
-                // scale array (4-byte copies: any row alignment; 32
-                // consecutive rows per warp step), completing on scfull[xs].
-                // The array is free: the slot was republished only after
-                // every epilogue warp had finished with its previous use.
+                // scale array (4-byte copies: any row alignment), completing
+                // on scfull[xs]; the columns past a document's end get NaN,
+                // which every max drops.  A lane finds the tile of its
+                // column by counting the tile starts up to its unit.  The
+                // array is free: the slot was republished only after every
+                // epilogue warp had finished with its previous use.
                 float* dst = sc + xs * STR;
-                for (int i = 0; i < h.nseg; ++i) {
-                    const int ri = __shfl_sync(0xffffffffu, rr, i);
-                    const int rowi = __shfl_sync(0xffffffffu, row0, i);
-                    const int coli = __shfl_sync(0xffffffffu, col, i);
-                    for (int j = lane; j < ri; j += 32) cp_async4(dst + coli + j, a.t_scales + rowi + j);
+                const unsigned starts = __reduce_or_sync(0xffffffffu, has ? 1u << (col >> 3) : 0u);
+                const int shift = row0 - col;  // row of column 0, were the tile to reach it
+#pragma unroll
+                for (int c0 = 0; c0 < STR; c0 += 32) {
+                    const int c = c0 + lane;
+                    const int i = max(__popc(starts & (2u * (1u << (c >> 3)) - 1u)) - 1, 0);
+                    const int r = __shfl_sync(0xffffffffu, shift, i) + c;
+                    const bool ok = c < __shfl_sync(0xffffffffu, rend, i);
+                    if (c < h.rows) cp_async4(dst + c, ok ? a.t_scales + r : &kNanScale);
                 }
                 cp_async_mbar_arrive(&scfull[xs]);
                 ++sc_sts;
@@ -787,16 +821,16 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
             }
         }
         __syncwarp();
-    } else if (PQ && warp > kLoaderWarp) {
+    } else if (PQ && warp >= kHelpWarp) {
         // ------------------------------------------------- decompressors
         // Thread = (row, 16-byte unit) pairs of every chunk stage: the unit
         // u of row R in chunk kc is the fp16 centroid of subspace 8 kc + u
         // for that row's code, written at unit u ^ (R % 8) -- the 128-byte
         // swizzle TMA would have produced -- so the MMA reads decompressed
-        // rows exactly as it reads loaded ones.  Padding rows of a tile are
-        // zero.  A quarter-warp covers one row: eight subspaces, eight
-        // distinct codebook bank groups, one 128-byte store.
-        const int tid = (warp - kLoaderWarp - 1) * 32 + lane;
+        // rows exactly as it reads loaded ones.  A quarter-warp covers one
+        // row: eight subspaces, eight distinct codebook bank groups, one
+        // 128-byte store.
+        const int tid = (warp - kHelpWarp) * 32 + lane;
         constexpr int kDecThreads = 32 * kSplitWarps;
         int s = 0;
         uint32_t ph = 0;
@@ -806,7 +840,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
             const StHdr h = slots[xs].h;
             if (h.flags & kEnd) break;
             const int cs = t % kCodeRing;
-            if (!warp_wait_all(&codefull[cs], (t / kCodeRing) & 1, abort_flag, a.err, a.budget)) break;
+            if (!warp_wait(&codefull[cs], (t / kCodeRing) & 1, abort_flag, a.err, a.budget)) break;
             const uint8_t* crow = code_ring + cs * STR * kPqM;
             bool ok = true;
             for (int kc = 0; kc < NCH; ++kc) {
@@ -815,15 +849,12 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
                     break;
                 }
                 uint8_t* stg = stage_base + s * SSTRIDE;
-                const uint8_t* gv = gvalid + cs * (STR / 8);
                 const int u = tid & 7;              // unit (subspace 8 kc + u) of every row this thread writes
                 const int m = kc * 8 + u;
                 // Rows tid / 8 + kRowStep j, eight per batch.  Every load of a
-                // batch is unconditional (a stale code byte of a padding row
-                // still indexes inside the codebook and the ring slot) and
-                // issued before the batch's stores, so the three dependent
-                // shared-memory loads of the eight rows overlap; padding rows
-                // are then written as zeros.
+                // batch is unconditional (any code byte indexes inside the
+                // codebook) and issued before the batch's stores, so the
+                // dependent shared-memory loads of the eight rows overlap.
                 constexpr int kBatch = 8;
                 constexpr int kRowStep = kDecThreads / 8;
                 for (int r0 = tid >> 3; r0 < h.rows; r0 += kRowStep * kBatch) {
@@ -832,9 +863,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
                     for (int j = 0; j < kBatch; ++j) {
                         const int R = min(r0 + kRowStep * j, STR - 1);
                         const uint32_t code = crow[R * kPqM + m];
-                        const uint4 e = *reinterpret_cast<const uint4*>(cb + (code * kPqM + m) * 16);
-                        const bool ok = (R & 7) < gv[R >> 3];
-                        v[j] = ok ? e : make_uint4(0u, 0u, 0u, 0u);
+                        v[j] = *reinterpret_cast<const uint4*>(cb + (code * kPqM + m) * 16);
                     }
 #pragma unroll
                     for (int j = 0; j < kBatch; ++j) {
@@ -857,7 +886,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
                 mbar_arrive(&xempty[xs]);
             }
         }
-    } else if (TF && warp > kLoaderWarp) {
+    } else if (TF && warp >= kHelpWarp) {
         // ------------------------------------------------------ splitters
         // Split each new query tile and every landed chunk stage: the MMA
         // reads an fp32 element as hi = tf32_trunc(x), so x stays in place
@@ -865,7 +894,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
         // to the twin region; then publish the split to the MMA thread.
         // Elements are independent, so the 128-byte swizzle needs no
         // decoding: x and lo keep the same byte positions.
-        const int tid = (warp - kLoaderWarp - 1) * 32 + lane;
+        const int tid = (warp - kHelpWarp) * 32 + lane;
         constexpr int kSplitThreads = 32 * kSplitWarps;
         auto split = [&](uint8_t* hi_p, uint8_t* lo_p, int bytes) {
             float4* hv = reinterpret_cast<float4*>(hi_p);
@@ -891,14 +920,14 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
             bool ok = true;
             if (h.q != cur_q) {
                 const int slot = qi % QS;
-                if (!warp_wait_all(&qfull[slot], (qi / QS) & 1, abort_flag, a.err, a.budget)) break;
+                if (!warp_wait(&qfull[slot], (qi / QS) & 1, abort_flag, a.err, a.budget)) break;
                 split(q_base + slot * qslot_bytes, qlo_base + slot * qslot_bytes, qslot_bytes);
                 if (lane == 0) mbar_arrive(&qconv[slot]);
                 ++qi;
                 cur_q = h.q;
             }
             for (int kc = 0; kc < NCH; ++kc) {
-                if (!warp_wait_all(&full[s], ph, abort_flag, a.err, a.budget)) {
+                if (!warp_wait(&full[s], ph, abort_flag, a.err, a.budget)) {
                     ok = false;
                     break;
                 }
@@ -913,175 +942,137 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------- MMA
-        // One thread runs this role: every wait is its own (no warp votes),
-        // and descriptors advance by adding the 16-byte-unit offset of each
+        // The whole warp runs this role, so that its control flow and the
+        // descriptors are uniform -- kept in uniform registers, where the
+        // MMA takes them from; a loop that one lane runs alone moves each
+        // of them there for every MMA -- and one elected lane issues.
+        // Descriptors advance by adding the 16-byte-unit offset of each
         // K-step to a per-stage base.
-        if (lane == 0) {
-            int s = 0;
-            uint32_t ph = 0;
-            int qi = 0, cur_q = -1, qslot = 0;
-            bool any = false;
-            for (int t = 0;; ++t) {
-                const int xs = t % kStRing;
-                if (!mbar_wait(&xfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
-                const StHdr x = slots[xs].h;
-                if (x.flags & kEnd) break;
-                mbar_arrive(&xempty[xs]);
-                if (!QSTREAM && x.q != cur_q) {
-                    if (cur_q >= 0) mma_commit(&qempty[qslot]);
-                    qslot = qi % QS;
-                    if (!mbar_wait(TF ? &qconv[qslot] : &qfull[qslot], (qi / QS) & 1, abort_flag, a.err, a.budget)) break;
-                    ++qi;
-                    cur_q = x.q;
+        int s = 0;
+        uint32_t ph = 0;
+        int qi = 0, cur_q = -1, qslot = 0;
+        bool any = false;
+        const uint32_t stage_sa = smem_u32(stage_base);
+        for (int t = 0;; ++t) {
+            const int xs = t % kStRing;
+            if (!warp_wait(&xfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
+            const StHdr* x = &slots[xs].h;
+            if (__any_sync(0xffffffffu, x->flags & kEnd)) break;
+            const int xq = __reduce_max_sync(0xffffffffu, x->q);
+            const int xn = __reduce_max_sync(0xffffffffu, x->n);
+            if (elect_one()) mbar_arrive(&xempty[xs]);
+            if (!QSTREAM && xq != cur_q) {
+                if (cur_q >= 0 && elect_one()) mma_commit(&qempty[qslot]);
+                qslot = qi % QS;
+                if (!warp_wait(TF ? &qconv[qslot] : &qfull[qslot], (qi / QS) & 1, abort_flag, a.err, a.budget)) break;
+                ++qi;
+                cur_q = xq;
+            }
+            bool ok = true;
+            const uint64_t q_desc = desc_sw128(smem_u32(q_base) + static_cast<uint32_t>(qslot * qslot_bytes));
+            const uint64_t qlo_desc = desc_sw128(smem_u32(qlo_base) + static_cast<uint32_t>(qslot * qslot_bytes));
+            const uint32_t idesc = a.idesc | (static_cast<uint32_t>(xn >> 3) << 17);
+            for (int kc = 0; kc < NCH; ++kc) {
+                if (!warp_wait(TF ? &conv[s] : &full[s], ph, abort_flag, a.err, a.budget)) {
+                    ok = false;
+                    break;
                 }
-                const int ab = t % KACC;
-                if (!mbar_wait(&tempty[ab], ((t / KACC) & 1) ^ 1, abort_flag, a.err, a.budget)) break;
                 tc_fence_after();
-                bool ok = true;
-                const uint32_t d_tmem = tbase + static_cast<uint32_t>(ab * H * STR);
-                const uint64_t q_desc = desc_sw128(smem_u32(q_base + qslot * qslot_bytes));
-                const uint64_t qlo_desc = desc_sw128(smem_u32(qlo_base + qslot * qslot_bytes));
-                const uint32_t idesc = a.idesc | (static_cast<uint32_t>(x.n >> 3) << 17);
-                for (int kc = 0; kc < NCH; ++kc) {
-                    if (!mbar_wait(TF ? &conv[s] : &full[s], ph, abort_flag, a.err, a.budget)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint64_t b_desc = desc_sw128(smem_u32(stage_base + s * SSTRIDE));
-                    const uint64_t blo_desc = desc_sw128(smem_u32(stage_base + s * SSTRIDE + STAGE_BYTES));
+                const uint64_t b_desc = desc_sw128(stage_sa + static_cast<uint32_t>(s * SSTRIDE));
+                const uint64_t blo_desc = desc_sw128(stage_sa + static_cast<uint32_t>(s * SSTRIDE + STAGE_BYTES));
 #pragma unroll
-                    for (int h = 0; h < H; ++h) {
-                        const uint64_t qoff =
-                            QSTREAM ? 0 : static_cast<uint64_t>(((kc * a.rows_alloc + h * 128) * 128) >> 4);
-                        const uint64_t a_desc =
-                            QSTREAM ? desc_sw128(smem_u32(stage_base + s * SSTRIDE + (STR + h * 128) * 128))
-                                    : q_desc + qoff;
+                for (int h = 0; h < H; ++h) {
+                    const int use = H * t + h;
+                    const int ab = use % KACC;
+                    const uint32_t d_tmem = tbase + static_cast<uint32_t>(ab * STR);
+                    if (kc == 0) {
+                        if (!warp_wait(&tempty[ab], ((use / KACC) & 1) ^ 1, abort_flag, a.err, a.budget)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                    }
+                    const uint64_t qoff =
+                        QSTREAM ? 0 : static_cast<uint64_t>(((kc * a.rows_alloc + h * 128) * 128) >> 4);
+                    const uint64_t a_desc =
+                        QSTREAM ? desc_sw128(stage_sa + static_cast<uint32_t>(s * SSTRIDE + (STR + h * 128) * 128))
+                                : q_desc + qoff;
+                    if (elect_one()) {
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {
                             const uint32_t accumulate = (kc > 0 || kk > 0) ? 1u : 0u;
                             if (TF) {  // hi.hi + hi.lo + lo.hi
-                                const uint32_t dt = d_tmem + static_cast<uint32_t>(h * STR);
-                                mma_tf32(dt, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
-                                mma_tf32(dt, a_desc + 2 * kk, blo_desc + 2 * kk, idesc, 1u);
-                                mma_tf32(dt, qlo_desc + qoff + 2 * kk, b_desc + 2 * kk, idesc, 1u);
+                                mma_tf32(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
+                                mma_tf32(d_tmem, a_desc + 2 * kk, blo_desc + 2 * kk, idesc, 1u);
+                                mma_tf32(d_tmem, qlo_desc + qoff + 2 * kk, b_desc + 2 * kk, idesc, 1u);
                             } else if (F8)
-                                mma_f8(d_tmem + static_cast<uint32_t>(h * STR), a_desc + 2 * kk, b_desc + 2 * kk, idesc,
-                                       accumulate);
+                                mma_f8(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
                             else
-                                mma_f16(d_tmem + static_cast<uint32_t>(h * STR), a_desc + 2 * kk, b_desc + 2 * kk,
-                                        idesc, accumulate);
+                                mma_f16(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
                         }
+                        if (kc == NCH - 1 && (a.fault != kFaultHoldAccumulator || blockIdx.x != 0 || t != 0))
+                            mma_commit(&tfull[ab]);
                     }
-                    mma_commit(&empty[s]);
                     any = true;
-                    if (++s == S) {
-                        s = 0;
-                        ph ^= 1;
-                    }
                 }
                 if (!ok) break;
-                if (a.fault != kFaultHoldAccumulator || blockIdx.x != 0 || t != 0)
-                    mma_commit(&tfull[ab]);
+                if (elect_one()) mma_commit(&empty[s]);
+                if (++s == S) {
+                    s = 0;
+                    ph ^= 1;
+                }
             }
-            // Every MMA this thread issued must finish before TMEM is freed.
-            if (any) {
-                mma_commit(mdone);
-                drain_wait(mdone, 0);
-            }
+            if (!ok) break;
+        }
+        // Every MMA this warp issued must finish before TMEM is freed.
+        if (any && elect_one()) {
+            mma_commit(mdone);
+            drain_wait(mdone, 0);
         }
         __syncwarp();
-    } else {
-        // ----------------------------------------------------- epilogue
-        // Thread = query row 128 h + 32 qd + lane of half h (TMEM lane
-        // 32 qd + lane).  Row block 4 h + qd is copy (4 h + qd) / bpc of
-        // block (4 h + qd) % bpc; the copies hold the same sums.  Documents
-        // are dealt round-robin to the copies (by their order in the
-        // records), so each warp owns whole documents: rmax[h] is the
-        // running max of its row over the current document's columns, kept
-        // in registers from one super-tile to the next when a document is
-        // cut at a super-tile's end.  Every active warp passes every
-        // super-tile and loads only the column groups of its documents.
-        const int qd = warp & 3;
-        const int copy = qd / a.bpc;
-        const int blk = qd - copy * a.bpc;
-        const bool active = copy < a.reps;
-        float rmax[H];
+    } else if (warp >= kFinWarp) {
+        // ----------------------------------------------------- finishers
+        // lane = row of a 32-row block (a query token); warp w takes blocks
+        // w, w + fin_warps, ...  m[b] is the running max of the lane's row
+        // of block b over the current document's columns, carried from one
+        // super-tile to the next when a document is cut at a super-tile's
+        // end.
+        constexpr int FB = fin_blocks(H, SH);
+        constexpr int FW = fin_warps(SH);
+        const int fw = warp - kFinWarp;
+        const int nb = fw < a.bpc ? (a.bpc - fw + FW - 1) / FW : 0;  // its blocks, <= FB
+        float m[FB], qsc[FB];  // qsc, F8: the row's query-token scale, reloaded when the query changes
 #pragma unroll
-        for (int h = 0; h < H; ++h) rmax[h] = -INFINITY;
-        uint32_t ord = 0;     // documents begun (all copies)
-        uint32_t mydocs = 0;  // documents this warp finished
-        bool mine = false;
-        bool aborted = false;
-        // F8: this thread's query-token scale(s), reloaded when the query changes
-        float qsc[H];
+        for (int b = 0; b < FB; ++b) m[b] = -INFINITY, qsc[b] = 1.f;
         int qsc_q = -1;
-#pragma unroll
-        for (int h = 0; h < H; ++h) qsc[h] = 1.f;
-
-        // A document's score(s) from its row maxima m.  False on abort.
-        auto finish_now = [&](int64_t f, int q, const float (&m)[H]) -> bool {
-            if (SH) {
-#pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    const int b = (4 * h + qd) % a.bpc;
-                    const int qq = q * a.group + b;
-                    const float sum = warp_sum(lane < a.nq ? (F8 ? m[h] * qsc[h] : m[h]) : 0.f);
-                    if (lane == 0 && qq < a.n_queries) a.out[static_cast<int64_t>(qq) * a.n_cand + f] = sum;
-                }
-            } else {
-                const int tok = blk * 32 + lane;
-                float v = 0.f;
-                if (tok < a.nq) v = F8 ? m[0] * qsc[0] : m[0];
-                const float sum = warp_sum(v);
-                if (a.bpc == 1) {
-                    if (lane == 0) a.out[f] = sum;
-                } else {
-                    // the copy's warps add their block sums in block order
-                    const int pb = copy * 2 + (mydocs & 1);
-                    const uint32_t use = mydocs >> 1;
-                    if (!warp_wait(&pempty[pb], (use & 1) ^ 1, abort_flag, a.err, a.budget)) return false;
-                    if (lane == 0) {
-                        part[pb * 4 + blk] = sum;
-                        mbar_arrive(&pfull[pb]);
-                    }
-                    if (blk == 0) {
-                        if (!warp_wait(&pfull[pb], use & 1, abort_flag, a.err, a.budget)) return false;
-                        if (lane == 0) {
-                            float tot = part[pb * 4];
-                            for (int bb = 1; bb < a.bpc; ++bb) tot += part[pb * 4 + bb];
-                            a.out[f] = tot;
-                            mbar_arrive(&pempty[pb]);
-                        }
-                    }
-                }
-            }
-            ++mydocs;
-            return true;
+        // Row r of block b of a document of query (group) q, if it counts.
+        auto row_value = [&](int b) {
+            const int tok = SH ? lane : b * 32 + lane;
+            return tok < a.nq ? (F8 ? m[b] * qsc[b] : m[b]) : 0.f;
         };
-        // Documents are finished in batches, off the path that releases the
-        // accumulator: their 32 row maxima (times the query-token scales,
-        // F8; 0 past nq) go to this warp's rows in shared memory, and every
-        // kFinRows / 2 rows lane r sums row r in token order and stores the
-        // score -- the same fixed order for every document, wherever it
-        // sits in a batch.  With several 32-token blocks per query (nq > 32)
-        // the copy's warps combine block sums at once instead (finish_now).
+        // Documents are finished in batches: their 32 row maxima (times the
+        // query-token scales, F8; 0 past nq) go to this warp's rows in
+        // shared memory, and when they are full lane r sums row r in token
+        // order and stores the score -- the same fixed order for every
+        // document, wherever it sits in a batch.  With several 32-token
+        // blocks per query (nq > 32) each block is summed across the warp
+        // and the blocks are added in order instead.
         const bool batched = SH || a.bpc == 1;
-        float* fin_rows = reinterpret_cast<float*>(fin_base + qd * kFinWarpBytes);
-        int* fin_ids = reinterpret_cast<int*>(fin_base + qd * kFinWarpBytes + kFinRows * 33 * 4);
+        float* fin_rows = reinterpret_cast<float*>(fin_base + fw * kFinWarpBytes);
+        int* fin_ids = reinterpret_cast<int*>(fin_base + fw * kFinWarpBytes + kFinRows * 33 * 4);
         int nfin = 0;  // rows in use
         auto flush = [&]() {
             __syncwarp();
             if (lane < nfin) {
+                float x[32];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) x[i] = fin_rows[lane * 33 + i];
                 float sum = 0.f;
-#pragma unroll 8
-                for (int i = 0; i < 32; ++i) sum += fin_rows[lane * 33 + i];
-                const int doc = lane / H;
-                const int f = fin_ids[2 * doc];
-                const int q = fin_ids[2 * doc + 1];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) sum += x[i];
+                const int f = fin_ids[2 * lane];
+                const int qq = fin_ids[2 * lane + 1];  // shared mode: the row's query
                 if (SH) {
-                    const int b = (4 * (lane % H) + qd) % a.bpc;
-                    const int qq = q * a.group + b;
                     if (qq < a.n_queries) a.out[static_cast<int64_t>(qq) * a.n_cand + f] = sum;
                 } else {
                     a.out[f] = sum;
@@ -1090,59 +1081,97 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
             __syncwarp();
             nfin = 0;
         };
-        auto finish = [&](int64_t f, int q, const float (&m)[H]) -> bool {
-            if (!batched) return finish_now(f, q, m);
+        for (int t = 0;; ++t) {
+            const int xs = t % kStRing;
+            if (!warp_wait(&xfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
+            const StHdr xh = slots[xs].h;
+            if (xh.flags & kEnd) break;
+            if (F8 && xh.q != qsc_q) {
+                qsc_q = xh.q;
 #pragma unroll
-            for (int h = 0; h < H; ++h) {
-                const int tok = SH ? lane : blk * 32 + lane;
-                fin_rows[(nfin + h) * 33 + lane] = tok < a.nq ? (F8 ? m[h] * qsc[h] : m[h]) : 0.f;
+                for (int b = 0; b < FB; ++b) {
+                    const int blk = fw + b * FW;
+                    const int qq = SH ? xh.q * a.group + blk : xh.q;
+                    const int tok = SH ? lane : blk * 32 + lane;
+                    qsc[b] = (b < nb && tok < a.nq && qq < a.n_queries)
+                                 ? __ldg(a.q_scales + static_cast<int64_t>(qq) * a.nq + tok)
+                                 : 0.f;
+                }
             }
-            if (lane == 0) {
-                fin_ids[2 * (nfin / H)] = static_cast<int>(f);
-                fin_ids[2 * (nfin / H) + 1] = q;
-            }
-            nfin += H;
-            if (nfin == kFinRows) flush();
-            return true;
-        };
-        // 32 accumulator columns of this warp's lanes in each half, and
-        // their 8-column sub-block maxima.  F8: each column times its
-        // document row's scale; the scales, the same for every half, are
-        // read from shared memory once, before the tensor-memory loads,
-        // and every half's load is in flight before one wait (for bf16 /
-        // fp16 the half-by-half order measured faster).
-        auto load_group = [&](uint32_t taddr, const float* scales, float (&v)[H][32], float (&sb)[H][4]) {
-            if constexpr (F8) {
-                float4 s4[8];
-                const float4* p4 = reinterpret_cast<const float4*>(scales);
+            const int us = t % UMS;
+            if (!warp_wait(&umfull[us], (t / UMS) & 1, abort_flag, a.err, a.budget)) break;
+            const float* um = reinterpret_cast<const float*>(um_base + us * L.um_stride) + fw * 32 + lane;
+            // Units with a value: a document's last one, and the last one of
+            // a copy's share of the columns, where its document goes on.
+            uint32_t shares = 0x80000000u >> (32 - STR / 8);
+            if (a.reps >= 2) shares |= shares >> (STR / 16);
+            if (a.reps >= 4) shares |= shares >> (STR / 32);
+            const int units = xh.rows >> 3;
+            uint32_t todo = (shares & (units == 32 ? 0xffffffffu : (1u << units) - 1u)) | xh.ends;
+            int e = 0;  // documents ended so far in this super-tile
+#pragma unroll 1
+            while (todo != 0u) {
+                const int u = __ffs(todo) - 1;
+                todo &= todo - 1u;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) s4[i] = p4[i];
-                uint32_t r[H][32];
+                for (int b = 0; b < FB; ++b)
+                    if (b < nb) m[b] = fmaxf(m[b], um[(u * a.bpc + b * FW) * 32]);
+                if ((xh.ends >> u) & 1u) {
+                    const int f = slots[xs].f[e++];
+                    if (batched) {
 #pragma unroll
-                for (int h = 0; h < H; ++h) tmem_ld32_issue(taddr + static_cast<uint32_t>(h * STR), r[h]);
+                        for (int b = 0; b < (SH ? FB : 1); ++b) {
+                            if (b < nb) {
+                                fin_rows[nfin * 33 + lane] = row_value(b);
+                                if (lane == 0) {
+                                    fin_ids[2 * nfin] = f;
+                                    fin_ids[2 * nfin + 1] = xh.q * a.group + fw + b * FW;
+                                }
+                                ++nfin;
+                            }
+                        }
+                        if (nfin > kFinRows - FB) flush();
+                    } else {
+                        float tot = 0.f;
 #pragma unroll
-                for (int h = 0; h < H; ++h) tmem_ld_wait32(r[h]);
-#pragma unroll
-                for (int h = 0; h < H; ++h) {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) v[h][i] = __uint_as_float(r[h][i]);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        mul_f32x2(v[h][4 * i], v[h][4 * i + 1], s4[i].x, s4[i].y);
-                        mul_f32x2(v[h][4 * i + 2], v[h][4 * i + 3], s4[i].z, s4[i].w);
+                        for (int b = 0; b < FB; ++b) {
+                            if (b < nb) {
+                                const float sum = warp_sum(row_value(b));
+                                tot = b == 0 ? sum : tot + sum;
+                            }
+                        }
+                        if (lane == 0) a.out[f] = tot;
                     }
-                    sub_maxima8(v[h], sb[h]);
-                }
-            } else {
 #pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    tmem_ld32(taddr + static_cast<uint32_t>(h * STR), v[h]);
-                    sub_maxima8(v[h], sb[h]);
+                    for (int b = 0; b < FB; ++b) m[b] = -INFINITY;
                 }
             }
-        };
-
-        for (int t = 0; !aborted; ++t) {
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&umempty[us]);
+                mbar_arrive(&xempty[xs]);
+            }
+        }
+        if (nfin > 0) flush();
+    } else {
+        // ----------------------------------------------------- epilogue
+        // Thread = query row 128 hh + 32 qd + lane of the warp's half hh (TMEM
+        // lane 32 qd + lane).  Row block 4 hh + qd is copy (4 hh + qd) / bpc
+        // of block (4 hh + qd) % bpc; the copies hold the same sums, so each
+        // copy's warps take their share of the columns.  A warp reduces its
+        // columns to a running max that starts again after each document's
+        // end, and leaves its value at every end and at its last unit to the
+        // finishers, which know whose columns they are: the code is short
+        // and nearly free of branches, and every warp has the same work.
+        // (Walking the documents and summing their rows here took 500-600
+        // instructions per warp for 128 columns of a shared list.)
+        const int qd = warp & 3;
+        const int hh = (warp - 2) >> 2;  // 0 for H = 1
+        const int copy = H == 1 ? qd / a.bpc : 0;
+        const int blk = 4 * hh + qd - copy * a.bpc;  // block of the copy: token block, or query of the group
+        const bool active = copy < a.reps;
+        const int share = STR / 8 / a.reps;  // units per copy, a multiple of 4
+        for (int t = 0;; ++t) {
             const int xs = t % kStRing;
             if (!warp_wait(&xfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
             const StHdr xh = slots[xs].h;
@@ -1152,64 +1181,58 @@ __global__ void __launch_bounds__(kernel_threads(KIND), CTAS)
                 if (lane == 0) mbar_arrive(&xempty[xs]);
                 continue;
             }
-            const int ab = t % KACC;
-            if (!warp_wait(&tfull[ab], (t / KACC) & 1, abort_flag, a.err, a.budget)) break;
-            tc_fence_after();
-            if (F8 && xh.q != qsc_q) {
-                qsc_q = xh.q;
-#pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    const int b = (4 * h + qd) % a.bpc;
-                    const int qq = SH ? xh.q * a.group + b : xh.q;
-                    const int tok = SH ? lane : b * 32 + lane;
-                    qsc[h] = (tok < a.nq && qq < a.n_queries)
-                                 ? __ldg(a.q_scales + static_cast<int64_t>(qq) * a.nq + tok)
-                                 : 0.f;
-                }
-            }
-            if (F8 && !warp_wait_all(&scfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
+            const int units = xh.rows >> 3;
+            const int u1 = min(units, (copy + 1) * share);
+            const int us = t % UMS;
+            float* um_out = reinterpret_cast<float*>(um_base + us * L.um_stride) + blk * 32 + lane;
             const float* scol = sc + xs * STR;  // F8: scale of each column's document row
-            float v[H][32], sb[H][4];
-            int held = -1;  // the column group in v
-            for (int i = 0; i < xh.nseg; ++i) {
-                const SegInfo si = slots[xs].seg[i];
-                if (si.flags & kFirst) {
-                    mine = static_cast<int>(ord & static_cast<uint32_t>(a.reps - 1)) == copy;
-                    ++ord;
-                    if (mine) {
-#pragma unroll
-                        for (int h = 0; h < H; ++h) rmax[h] = -INFINITY;
-                    }
+            const int use = H * t + hh;
+            const int ab = use % KACC;
+            const uint32_t tacc = tbase + (static_cast<uint32_t>(qd * 32) << 16) + static_cast<uint32_t>(ab * STR);
+            if (!warp_wait(&umempty[us], ((t / UMS) & 1) ^ 1, abort_flag, a.err, a.budget)) break;
+            if (F8 && !warp_wait(&scfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
+            if (!warp_wait(&tfull[ab], (use / KACC) & 1, abort_flag, a.err, a.budget)) break;
+            tc_fence_after();
+            float m = -INFINITY;
+#pragma unroll 1
+            for (int u = copy * share; u < u1; u += 4) {  // a group of four units: 32 columns
+                float v[32], um[4];
+                tmem_ld32(tacc + static_cast<uint32_t>(8 * u), v);
+                if (F8) scale32(v, scol + 8 * u);  // columns past a document's end have scale NaN
+                unit_maxima(v, um);
+                if (!F8 && ((xh.partial >> u) & 15u) != 0u) {
+                    const uint8_t* valid = slots[xs].valid + u;
+                    if ((xh.partial >> u) & 1u) um[0] = unit_max_n<0>(v, valid[0]);
+                    if ((xh.partial >> u) & 2u) um[1] = unit_max_n<1>(v, valid[1]);
+                    if ((xh.partial >> u) & 4u) um[2] = unit_max_n<2>(v, valid[2]);
+                    if ((xh.partial >> u) & 8u) um[3] = unit_max_n<3>(v, valid[3]);
                 }
-                if (!mine) continue;
-                const int c_hi = si.col + si.r;
-                for (int g0 = si.col & ~31; g0 < c_hi; g0 += 32) {
-                    if (g0 != held) {
-                        load_group(tbase + (static_cast<uint32_t>(qd * 32) << 16) +
-                                       static_cast<uint32_t>(ab * H * STR + g0),
-                                   scol + g0, v, sb);
-                        held = g0;
-                    }
-                    const int lo = max(si.col - g0, 0);
-                    const int hi = min(c_hi - g0, 32);
+                const uint32_t eg = (xh.ends >> u) & 15u;
+                if (eg == 0u) {
+                    m = fmax3(m, fmax3(um[0], um[1], um[2]), um[3]);
+                } else {
+                    float* o = um_out + u * a.bpc * 32;
 #pragma unroll
-                    for (int h = 0; h < H; ++h) rmax[h] = fold_cols(rmax[h], v[h], sb[h], lo, hi);
-                }
-                if ((si.flags & kLast) && !finish(si.f, xh.q, rmax)) {
-                    aborted = true;
-                    break;
+                    for (int k = 0; k < 4; ++k) {
+                        m = fmaxf(m, um[k]);
+                        if ((eg >> k) & 1u) {
+                            o[k * a.bpc * 32] = m;
+                            m = -INFINITY;
+                        }
+                    }
                 }
             }
-            if (aborted) break;
+            // the share's last unit, unless a document (or the whole super-tile) ended before or there
+            const int ul = (copy + 1) * share - 1;
+            if (ul < units && ((xh.ends >> ul) & 1u) == 0u) um_out[ul * a.bpc * 32] = m;
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(&tempty[ab]);
+                mbar_arrive(&umfull[us]);
                 mbar_arrive(&xempty[xs]);
             }
-            if (nfin >= kFinRows / 2) flush();
         }
-        if (!aborted && nfin > 0) flush();
     }
 
     tc_fence_before();
@@ -1326,8 +1349,8 @@ tms_status plan_tc(const DeviceInfo& dev, const Args& a, const Config* force, Pl
         int best = -1;
         for (int qs = stream ? 0 : 2; qs >= (stream ? 0 : 1); --qs) {
             if (!stream && want_qs && qs != want_qs) continue;
-            const Layout L0 = make_layout(0, qs, a.nchunks, 32 * a.bpc * rp, str, KIND, acc_count(H, str, ctas),
-                                          SH || a.bpc == 1, stream ? 128 * H : 0);
+            const Layout L0 = make_layout(0, qs, a.nchunks, 32 * a.bpc * rp, str, KIND, acc_count(str, ctas),
+                                          a.bpc, fin_warps(SH), stream ? 128 * H : 0);
             int sts = std::min(kMaxStages, (limit - L0.total) / (L0.stage_stride + 24));
             if (cap > 0 && sts > cap) sts = cap;
             if (sts > best) {
@@ -1439,8 +1462,8 @@ tms_status launch_tc(const DeviceInfo& dev, const void* queries, tms_dtype dtype
     a.idesc = make_idesc(128, 0, TF ? 2u : ((!F8 && dtype == TMS_BF16) ? 1u : 0u));
     a.stages = stages;
     a.qslots = qslots;
-    const Layout L = make_layout(stages, qslots, a.nchunks, a.rows_alloc, str, KIND, acc_count(H, str, ctas),
-                                 SH || a.bpc == 1, qslots == 0 ? 128 * H : 0);
+    const Layout L = make_layout(stages, qslots, a.nchunks, a.rows_alloc, str, KIND, acc_count(str, ctas),
+                                 a.bpc, fin_warps(SH), qslots == 0 ? 128 * H : 0);
     const int smem = L.total + 1024;
     void (*kern)(const Maps, const Args);
     if constexpr (H == 2) {
@@ -1456,7 +1479,7 @@ tms_status launch_tc(const DeviceInfo& dev, const void* queries, tms_dtype dtype
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return launch_status(cudaErrorInvalidValue);
     const int64_t grid = std::min<int64_t>(static_cast<int64_t>(dev.sm_count) * ctas, a.n_flat);
-    return launch_status(launch_dependent(kern, dim3(static_cast<unsigned>(grid)), dim3(kernel_threads(KIND)),
+    return launch_status(launch_dependent(kern, dim3(static_cast<unsigned>(grid)), dim3(kernel_threads(KIND, H, SH)),
                                           static_cast<size_t>(smem), stream, maps, a));
 }
 
