@@ -83,11 +83,12 @@ bool load_encoder() {
 struct TmapKey {
     CUtensorMapDataType dtype;
     const void* base;
-    uint64_t cols, rows, row_bytes;
-    uint32_t box_cols, box_rows;
+    uint64_t cols, rows, planes, row_bytes;  // planes 0: a 2-D map
+    uint32_t box_cols, box_rows, box_planes;
     bool operator==(const TmapKey& o) const {
-        return dtype == o.dtype && base == o.base && cols == o.cols && rows == o.rows && row_bytes == o.row_bytes &&
-               box_cols == o.box_cols && box_rows == o.box_rows;
+        return dtype == o.dtype && base == o.base && cols == o.cols && rows == o.rows && planes == o.planes &&
+               row_bytes == o.row_bytes && box_cols == o.box_cols && box_rows == o.box_rows &&
+               box_planes == o.box_planes;
     }
 };
 constexpr int kTmapCache = 32;
@@ -97,12 +98,9 @@ struct TmapCache {
     int used = 0, next = 0;
 };
 thread_local TmapCache t_tmaps;
-}  // namespace
 
-tms_status encode_tmap_2d(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, uint64_t cols,
-                          uint64_t rows, uint64_t row_bytes, uint32_t box_cols, uint32_t box_rows) {
+tms_status encode(CUtensorMap* map, const TmapKey& key) {
     if (!load_encoder()) return TMS_ERR_CUDA;
-    const TmapKey key{dtype, base, cols, rows, row_bytes, box_cols, box_rows};
     TmapCache& c = t_tmaps;
     for (int i = 0; i < c.used; ++i)
         if (c.key[i] == key) {
@@ -111,18 +109,31 @@ tms_status encode_tmap_2d(CUtensorMap* map, CUtensorMapDataType dtype, const voi
         }
     // A zero-row tensor is not encodable; callers never load from it then,
     // so describe one row (the box reads zero fill beyond it).
-    const cuuint64_t dims[2] = {cols, rows > 0 ? rows : 1};
-    const cuuint64_t strides[1] = {row_bytes};
-    const cuuint32_t box[2] = {box_cols, box_rows};
-    const cuuint32_t estr[2] = {1, 1};
+    const cuuint64_t dims[3] = {key.cols, key.rows > 0 ? key.rows : 1, key.planes};
+    const cuuint64_t strides[2] = {key.row_bytes, key.row_bytes * key.rows};
+    const cuuint32_t box[3] = {key.box_cols, key.box_rows, key.box_planes};
+    const cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = g_encode.load(std::memory_order_relaxed)(
-        map, dtype, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        map, key.dtype, key.planes > 0 ? 3 : 2, const_cast<void*>(key.base), dims, strides, box, estr,
+        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return TMS_ERR_INVALID_ARG;
     const int slot = c.used < kTmapCache ? c.used++ : (c.next++ % kTmapCache);
     c.key[slot] = key;
     std::memcpy(&c.map[slot], map, sizeof(CUtensorMap));
     return TMS_OK;
+}
+}  // namespace
+
+tms_status encode_tmap_2d(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, uint64_t cols,
+                          uint64_t rows, uint64_t row_bytes, uint32_t box_cols, uint32_t box_rows) {
+    return encode(map, TmapKey{dtype, base, cols, rows, 0, row_bytes, box_cols, box_rows, 0});
+}
+
+tms_status encode_tmap_3d(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, uint64_t cols,
+                          uint64_t rows, uint64_t planes, uint64_t row_bytes, uint32_t box_cols, uint32_t box_rows,
+                          uint32_t box_planes) {
+    return encode(map, TmapKey{dtype, base, cols, rows, planes, row_bytes, box_cols, box_rows, box_planes});
 }
 
 }  // namespace tms

@@ -183,37 +183,53 @@ __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem desc] * B[smem desc]^T, kind::f16 (fp16/bf16 in, fp32 acc).
-__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                        uint32_t accumulate) {
+// Shared-memory matrix descriptors for K-major operands stored in the
+// 128-byte-swizzle layout TMA writes (8-row x 128-byte atoms, atoms 1024 B
+// apart): the low word holds the start address and is what changes between
+// MMAs, the high word is the same for all.
+__device__ __forceinline__ uint32_t desc_sw128(uint32_t saddr) {
+    return ((saddr & 0x3FFFFu) >> 4)  // start address: the first element; its atom must be 1024-byte aligned
+           | (1u << 16);              // leading byte offset (unused for SW128 K-major)
+}
+constexpr uint32_t kDescHigh = (1024u >> 4)   // stride byte offset: 8 rows x 128 B
+                               | (1u << 14)   // descriptor version (sm_100 family)
+                               | (2u << 29);  // layout: SWIZZLE_128B
+
+// D[tmem] (+)= A[smem] * B[smem]^T (low descriptor words), kind::f16 (fp16/bf16
+// in, fp32 accumulation).
+__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %5};\n\t"
+        "mov.b64 db, {%2, %5};\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a), "r"(b), "r"(idesc), "r"(accumulate), "n"(kDescHigh)
         : "memory");
 }
 
-// D[tmem] (+)= A * B^T, kind::f8f6f4 (both operands E4M3 per the
-// instruction descriptor, fp32 accumulator; K = 32 elements).
-__device__ __forceinline__ void mma_f8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                       uint32_t accumulate) {
+// kind::f8f6f4 (both operands E4M3 per the instruction descriptor, fp32
+// accumulation; K = 32 elements).
+__device__ __forceinline__ void mma_f8(uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %5};\n\t"
+        "mov.b64 db, {%2, %5};\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a), "r"(b), "r"(idesc), "r"(accumulate), "n"(kDescHigh)
         : "memory");
 }
 
-// D[tmem] (+)= A * B^T, kind::tf32 (fp32 containers read as tf32, fp32 acc).
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
+// kind::tf32 (fp32 containers read as tf32, fp32 accumulation).
+__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %5};\n\t"
+        "mov.b64 db, {%2, %5};\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a), "r"(b), "r"(idesc), "r"(accumulate), "n"(kDescHigh)
         : "memory");
 }
 
@@ -268,18 +284,6 @@ __device__ __forceinline__ void mul_f32x2(float& a, float& b, float x, float y) 
         : "f"(x), "f"(y));
 }
 
-// v[c] *= s[c] for 32 columns, two at a time; `s` 16-byte aligned in shared
-// memory, read as eight broadcast 128-bit loads.
-__device__ __forceinline__ void scale32(float (&v)[32], const float* s) {
-    const float4* s4 = reinterpret_cast<const float4*>(s);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const float4 k = s4[i];
-        mul_f32x2(v[4 * i], v[4 * i + 1], k.x, k.y);
-        mul_f32x2(v[4 * i + 2], v[4 * i + 3], k.z, k.w);
-    }
-}
-
 // Programmatic dependent launch (see launch_dependent): wait for the
 // previous kernel of the stream to complete, and let the next one be
 // scheduled.
@@ -318,6 +322,32 @@ __device__ __forceinline__ void tmem_ld_wait32(uint32_t (&r)[32]) {
                  : "memory");
 }
 
+// The same 32 columns of the same 32 lanes as 8-column blocks (.16x256b.x4,
+// lanes 0-15 and 16-31): register 4 j + e of slab s holds column 8 j + 2 (t %
+// 4) + e % 2 of lane 16 s + 8 (e / 2) + t / 4, t the thread -- a thread sees
+// two columns of a block for four lanes, instead of eight for one.
+__device__ __forceinline__ void tmem_ld_blocks(uint32_t taddr, uint32_t (&r)[2][16]) {
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+        asm volatile(
+            "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+            "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+            : "=r"(r[s][0]), "=r"(r[s][1]), "=r"(r[s][2]), "=r"(r[s][3]), "=r"(r[s][4]), "=r"(r[s][5]),
+              "=r"(r[s][6]), "=r"(r[s][7]), "=r"(r[s][8]), "=r"(r[s][9]), "=r"(r[s][10]), "=r"(r[s][11]),
+              "=r"(r[s][12]), "=r"(r[s][13]), "=r"(r[s][14]), "=r"(r[s][15])
+            : "r"(taddr + (static_cast<uint32_t>(16 * s) << 16))
+            : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0][0]), "+r"(r[0][1]), "+r"(r[0][2]), "+r"(r[0][3]), "+r"(r[0][4]), "+r"(r[0][5]),
+                   "+r"(r[0][6]), "+r"(r[0][7]), "+r"(r[0][8]), "+r"(r[0][9]), "+r"(r[0][10]), "+r"(r[0][11]),
+                   "+r"(r[0][12]), "+r"(r[0][13]), "+r"(r[0][14]), "+r"(r[0][15]), "+r"(r[1][0]), "+r"(r[1][1]),
+                   "+r"(r[1][2]), "+r"(r[1][3]), "+r"(r[1][4]), "+r"(r[1][5]), "+r"(r[1][6]), "+r"(r[1][7]),
+                   "+r"(r[1][8]), "+r"(r[1][9]), "+r"(r[1][10]), "+r"(r[1][11]), "+r"(r[1][12]), "+r"(r[1][13]),
+                   "+r"(r[1][14]), "+r"(r[1][15])
+                 :
+                 : "memory");
+}
+
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     uint32_t r[32];
     tmem_ld32_issue(taddr, r);
@@ -327,20 +357,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 }
 
 
-
-// Shared-memory matrix descriptor for a K-major operand stored in the
-// 128-byte-swizzle layout TMA writes (8-row x 128-byte atoms, atoms 1024 B
-// apart).  `saddr` is the shared address of the first element to use; its
-// atom must be 1024-byte aligned.
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);  // start address
-    d |= static_cast<uint64_t>(1) << 16;                  // leading byte offset (unused for SW128 K-major)
-    d |= static_cast<uint64_t>(1024 >> 4) << 32;          // stride byte offset: 8 rows x 128 B
-    d |= static_cast<uint64_t>(1) << 46;                  // descriptor version (sm_100 family)
-    d |= static_cast<uint64_t>(2) << 61;                  // layout: SWIZZLE_128B
-    return d;
-}
 
 // Instruction descriptor: fp32 accumulate, K-major A and B, shape M x N.
 // a_fmt: 0 = f16, 1 = bf16 (kind::f16); 2 = tf32 (kind::tf32).

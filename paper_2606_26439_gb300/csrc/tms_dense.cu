@@ -157,7 +157,6 @@ tms_status score_dense(const void* queries, tms_dtype dtype, int n_queries, int 
     a.n_queries = n_queries;
     a.nq = nq;
     a.bpc = (nq + 31) / 32;
-    a.qbox = 32 * a.bpc;
 
     if (dtype == TMS_F32) {
         // split TF32 on the tensor cores; the exact CUDA-core kernel below

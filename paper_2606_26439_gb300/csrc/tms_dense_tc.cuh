@@ -90,14 +90,21 @@ constexpr int kMaxSeg = 32;                   // tiles per super-tile (each >= 8
 __host__ __device__ constexpr int st_ring(int) { return 16; }
 // Epilogue warps: one per tensor-memory lane quarter and query half.
 __host__ __device__ constexpr int epi_warps(int h) { return 4 * h; }
-constexpr int kSplitWarps = 4;  // TF: splitter warps after the loader; kPQ: decompressors
-// Finisher warps: they take the 32-row blocks of a super-tile in turn (two
-// blocks each for eight queries, all of a query's blocks for one).
-__host__ __device__ constexpr int fin_warps(bool sh) { return sh ? 4 : 1; }
-__host__ __device__ constexpr int fin_blocks(int h, bool sh) { return sh ? h : 4; }
-// planner, MMA, epilogue warps, loader, finishers, splitters / decompressors
+// Warps that prepare every chunk stage.  TF: splitters -- four of them took
+// 1,150 cycles per 16 KB stage, against 770 for its MMAs and 670 for its bytes
+// from HBM; kPQ: decompressors.
+__host__ __device__ constexpr int help_warps(int kind) { return kind == kTF32 ? 8 : 4; }
+// Finisher warp, where the copies of a query's blocks share a super-tile's
+// columns (per-query lists).
+__host__ __device__ constexpr int fin_warps(bool sh) { return sh ? 0 : 1; }
+constexpr int kMaxBlocks = 4;  // 32-token blocks of a query
+// MMA warps, taking super-tiles in turn: issuing an MMA takes its thread about
+// 50 cycles, a commit 64, a wait that need not wait 70 (measured), so beside
+// 64- or 128-cycle MMAs one thread cannot keep the tensor core busy.
+constexpr int kMmaWarps = 2;
+// planner, MMA warps, loader, epilogue warps, finisher, splitters / decompressors
 __host__ __device__ constexpr int kernel_threads(int kind, int h, bool sh) {
-    return 32 * (3 + epi_warps(h) + fin_warps(sh) + ((kind == kTF32 || kind == kPQ) ? kSplitWarps : 0));
+    return 32 * (2 + kMmaWarps + epi_warps(h) + fin_warps(sh) + ((kind == kTF32 || kind == kPQ) ? help_warps(kind) : 0));
 }
 // Accumulator buffers of STR tensor-memory columns -- one holds one query
 // half of a super-tile -- as many as the SM's 512 columns give the CTAs
@@ -131,7 +138,9 @@ struct StHdr {
     int rows;         // packed rows: 8 x units
     uint32_t ends;     // bit u: unit u is the last of a document (f[] in that order)
     uint32_t partial;  // bit u: and not all of its rows count
-    int pad;
+    // per-query lists, bit u: the epilogue leaves a value at unit u, the last of
+    // a document, or of a copy's share of the columns where its document goes on
+    uint32_t values;
 };
 
 struct StSlot {
@@ -155,6 +164,9 @@ struct Args {
     int64_t n_cand;    // entries of cand_ids
     int64_t n_flat;    // work items: n_cand, or n_groups * n_cand in shared mode
     int group;         // shared mode: queries per group; 0 otherwise
+    int rounds;        // shared mode: see Work; set by launch_tc
+    int round_groups;  // groups of every round but the last
+    int last_groups;   // groups of the last round
     int n_queries;
     int nq;
     int nchunks;     // ceil(d / chunk_elems)
@@ -163,7 +175,6 @@ struct Args {
     int bpc;         // 32-row query blocks per copy: ceil(nq / 32) token blocks, or the group's queries
     int reps;        // copies of the blocks stacked in M (1, 2 or 4); documents are dealt round-robin to them
     int rows_alloc;  // query rows held per dimension chunk: 32 * bpc * reps
-    int qbox;        // rows of one query TMA box: 32 * bpc (per-query), 32 (shared)
     uint32_t idesc;  // instruction descriptor, N field left 0 (set per super-tile)
     const uint8_t* pq_codes;    // kPQ: [n_tokens][16] uint8
     const float* pq_codebook;   // kPQ: [16][pq_k][8] fp32
@@ -181,18 +192,17 @@ static __device__ const float kNanScale = __builtin_nanf("");
 constexpr int kFaultHoldAccumulator = TMS_FAULT_HOLD_ACCUMULATOR;
 
 struct Layout {
-    int q_off, qlo_off, stage_off, stage_stride, um_off, um_stride, fin_off, sc_off, cb_off, code_off, st_off, bar_off,
+    int q_off, qlo_off, stage_off, stage_stride, um_off, um_stride, fin_off, bias_off, sc_off, cb_off, code_off, st_off, bar_off,
         misc_off, total;
 };
 
-// Super-tiles whose unit maxima may wait for the finishers.  One is enough
-// where the MMAs of a super-tile take far longer than finishing one (three or
-// more dimension chunks), and leaves room for another chunk stage.
-__host__ __device__ constexpr int um_slots(int nchunks) { return nchunks >= 3 ? 1 : 2; }
-// Finished documents waiting for their sum over query tokens, per finisher
-// warp: kFinRows rows of 32 row maxima (one row per document and 32-row
+// Per-query lists: super-tiles whose row maxima may wait for the finisher.
+constexpr int kUmSlots = 2;
+// Finished documents waiting for their sum over query tokens, per epilogue warp
+// (shared lists) or the finisher: kFinRows rows of 32 row maxima (one row per document and 32-row
 // block), padded to 33 floats so that lane r reading row r walks distinct
-// banks, then each row's (candidate, query or query of the group) pair.
+// banks, then each row's (candidate, query) pair.  A group of four units ends
+// at most four documents, so a group starts with at most kFinRows - 4 in use.
 constexpr int kFinRows = 8;
 constexpr int kFinWarpBytes = kFinRows * 33 * 4 + kFinRows * 8;
 
@@ -208,7 +218,7 @@ constexpr int kFinWarpBytes = kFinRows * 33 * 4 + kFinRows * 8;
 // each chunk stage holds the str document rows, then the qrows query rows
 // of the same dimension chunk.
 __host__ __device__ inline Layout make_layout(int stages, int qslots, int nchunks, int rows_alloc, int str, int kind,
-                                              int kacc, int blocks, int fins, int qrows) {
+                                              int kacc, int blocks, bool sh, int qrows, int h) {
     const bool f8 = kind == kE4M3;
     const int twin = kind == kTF32 ? 2 : 1;
     Layout L;
@@ -217,14 +227,15 @@ __host__ __device__ inline Layout make_layout(int stages, int qslots, int nchunk
     L.stage_off = (twin * L.qlo_off + 1023) & ~1023;
     L.stage_stride = twin * (str + qrows) * 128;
     L.um_off = L.stage_off + stages * L.stage_stride;
-    L.um_stride = (str / 8) * blocks * 128;  // [unit][32-row block][row] unit maxima
-    L.fin_off = L.um_off + um_slots(nchunks) * L.um_stride;
-    L.sc_off = (L.fin_off + fins * kFinWarpBytes + 127) & ~127;
+    L.um_stride = sh ? 0 : (str / 8) * blocks * 128;  // [unit][32-row block][row] row maxima
+    L.fin_off = L.um_off + kUmSlots * L.um_stride;
+    L.bias_off = (L.fin_off + (sh ? epi_warps(h) : 1) * kFinWarpBytes + 127) & ~127;
+    L.sc_off = L.bias_off + 256;
     L.cb_off = L.sc_off + (f8 ? st_ring(str) * str * 4 : 0);  // F8: [st_ring][str] column scales
     L.code_off = L.cb_off + (kind == kPQ ? kPqCbBytes : 0);                        // kPQ: fp16 codebook
     L.st_off = L.code_off + (kind == kPQ ? kCodeRing * str * kPqM : 0);  // kPQ: code-row ring
     L.bar_off = L.st_off + st_ring(str) * static_cast<int>(sizeof(StSlot));
-    const int nbar = 3 * stages + 2 * kacc + 3 * qslots + 3 * st_ring(str) + 4 + 1 + 2 * kCodeRing;
+    const int nbar = 3 * stages + 2 * kacc + 3 * qslots + 3 * st_ring(str) + 2 * kUmSlots + kMmaWarps + 2 * kCodeRing;
     L.misc_off = L.bar_off + nbar * 8;
     L.total = L.misc_off + 16;
     return L;
@@ -240,11 +251,61 @@ struct Meta {
     int id;
 };
 
-__device__ __forceinline__ int load_id(const Args& a, int64_t k) {
-    const int64_t f = static_cast<int64_t>(blockIdx.x) + k * gridDim.x;
-    if (f >= a.n_flat) return -1;
-    return __ldg(a.cand_ids + (a.group ? f % a.n_cand : f));
-}
+// The work items of one CTA, numbered k = 0, 1, ...
+// Per-query lists: flat index blockIdx + k x grid, candidates dealt in turn.
+// Shared lists: the groups are taken in rounds of `round_groups` (the last
+// round `last_groups`); in a round the CTAs are dealt to its groups in turn
+// and a group's candidates to its CTAs in turn, so CTAs of different groups
+// read the same documents at about the same time: from HBM once per round,
+// and from L2 for the rest (group after group over the whole list, every
+// group read all of it from HBM).
+template <bool SH>
+struct Work {
+    int64_t n;              // items of this CTA
+    int b, grid;
+    int n1, q1, c1, j1;     // SH, full rounds: items of one, group offset, first candidate, stride
+    int64_t full;           // SH: items of all full rounds
+    int ql, cl, jl;         // SH, last round: group, first candidate, stride
+
+    __device__ __forceinline__ explicit Work(const Args& a) : b(blockIdx.x), grid(gridDim.x) {
+        if (SH) {
+            auto count = [&](int c, int j) {
+                return c < j && c < a.n_cand ? static_cast<int>((a.n_cand - c + j - 1) / j) : 0;
+            };
+            q1 = b % a.round_groups;
+            c1 = b / a.round_groups;
+            j1 = grid / a.round_groups;
+            n1 = a.rounds > 1 ? count(c1, j1) : 0;
+            full = static_cast<int64_t>(a.rounds - 1) * n1;
+            ql = (a.rounds - 1) * a.round_groups + b % a.last_groups;
+            cl = b / a.last_groups;
+            jl = grid / a.last_groups;
+            n = full + count(cl, jl);
+        } else {
+            n = a.n_flat > b ? (a.n_flat - b + grid - 1) / grid : 0;
+        }
+    }
+    // Item k < n: its query (group; SH only) and its entry of the list.
+    __device__ __forceinline__ void at(const Args& a, int64_t k, int* q, int64_t* pos) const {
+        if (!SH) {
+            *pos = b + k * grid;
+        } else if (k < full) {
+            const int r = static_cast<int>(k / n1);
+            *q = r * a.round_groups + q1;
+            *pos = c1 + (k - static_cast<int64_t>(r) * n1) * j1;
+        } else {
+            *q = ql;
+            *pos = cl + (k - full) * jl;
+        }
+    }
+    __device__ __forceinline__ int load_id(const Args& a, int64_t k) const {
+        if (k >= n) return -1;
+        int q;
+        int64_t pos;
+        at(a, k, &q, &pos);
+        return __ldg(a.cand_ids + pos);
+    }
+};
 
 __device__ __forceinline__ Meta load_meta(const Args& a, int id) {
     Meta m;
@@ -294,13 +355,28 @@ __device__ __forceinline__ void unit_maxima(const float (&v)[32], float (&um)[4]
                       fmaxf(v[8 * k + 6], v[8 * k + 7]));
 }
 
-// Max of the first n (1..8) columns of unit K.
+// Max of the columns of unit K that count, with b[0..1] their row of the bias
+// table (0, or -inf for the columns past the document's end).
 template <int K>
-__device__ __forceinline__ float unit_max_n(const float (&v)[32], int n) {
-    float m = v[8 * K];
-#pragma unroll
-    for (int j = 1; j < 8; ++j) m = j < n ? fmaxf(m, v[8 * K + j]) : m;
-    return m;
+__device__ __forceinline__ float unit_max_bias(const float (&v)[32], const float4* b) {
+    const float4 x = b[0], y = b[1];
+    return fmax3(fmax3(v[8 * K] + x.x, v[8 * K + 1] + x.y, v[8 * K + 2] + x.z),
+                 fmax3(v[8 * K + 3] + x.w, v[8 * K + 4] + y.x, v[8 * K + 5] + y.y),
+                 fmaxf(v[8 * K + 6] + y.z, v[8 * K + 7] + y.w));
+}
+
+// Maxima of the four units from unit u on, whose columns are in v, with the
+// columns past a document's end dropped.
+__device__ __forceinline__ void unit_maxima_counted(const float (&v)[32], float (&um)[4], uint32_t partial,
+                                                    const uint8_t* valid, const float* bias) {
+    unit_maxima(v, um);
+    if (partial != 0u) {
+        const float4* b = reinterpret_cast<const float4*>(bias);
+        if (partial & 1u) um[0] = unit_max_bias<0>(v, b + 2 * valid[0]);
+        if (partial & 2u) um[1] = unit_max_bias<1>(v, b + 2 * valid[1]);
+        if (partial & 4u) um[2] = unit_max_bias<2>(v, b + 2 * valid[2]);
+        if (partial & 8u) um[3] = unit_max_bias<3>(v, b + 2 * valid[3]);
+    }
 }
 
 // Tensor maps of one launch.  doc[h] covers document rows with a box of
@@ -332,8 +408,11 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
     constexpr int KACC = acc_count(STR, CTAS);
     constexpr uint32_t TCOLS = KACC * STR;
     constexpr int kEpiWarps = epi_warps(H);
-    constexpr int kLoaderWarp = 2 + kEpiWarps;
-    constexpr int kFinWarp = kLoaderWarp + 1;              // the first of them
+    constexpr int kLoaderWarp = 1 + kMmaWarps;
+    constexpr int kEpiWarp = kLoaderWarp + 1;  // the first of them
+    static_assert(kEpiWarp % 4 == 0, "epilogue warp w reads the tensor-memory lanes of quarter w % 4");
+    constexpr int kFinWarp = kEpiWarp + kEpiWarps;         // the first of them
+    constexpr int kHelpers = help_warps(KIND);
     constexpr int kHelpWarp = kFinWarp + fin_warps(SH);    // TF / kPQ: the first splitter / decompressor
     constexpr int kStRing = st_ring(STR);
     static_assert(KACC >= 2 && TCOLS * CTAS <= 512, "tensor memory of one SM");
@@ -345,15 +424,15 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
     const int NCH = a.nchunks;
     const int qslot_bytes = NCH * a.rows_alloc * 128;
     const bool QSTREAM = QS == 0;  // the query rows come with every chunk stage
-    const Layout L = make_layout(S, QS, NCH, a.rows_alloc, STR, KIND, KACC, a.bpc, fin_warps(SH), QSTREAM ? 128 * H : 0);
-    const int UMS = um_slots(NCH);
+    const Layout L = make_layout(S, QS, NCH, a.rows_alloc, STR, KIND, KACC, a.bpc, SH, QSTREAM ? 128 * H : 0, H);
     const int SSTRIDE = L.stage_stride;  // bytes between stages (TF: hi, then lo)
 
     uint8_t* q_base = smem + L.q_off;
     uint8_t* qlo_base = smem + L.qlo_off;  // TF: the lo twin of the query region
     uint8_t* stage_base = smem + L.stage_off;
-    uint8_t* um_base = smem + L.um_off;    // [UMS][unit][block][row] unit maxima
-    uint8_t* fin_base = smem + L.fin_off;  // [finisher warp] finished-document rows
+    uint8_t* um_base = smem + L.um_off;    // per-query lists: [kUmSlots][unit][block][row] row maxima
+    uint8_t* fin_base = smem + L.fin_off;  // finished-document rows
+    float* bias = reinterpret_cast<float*>(smem + L.bias_off);  // [8][8]: entry [n][j] 0 for j < n, else -inf
     float* sc = reinterpret_cast<float*>(smem + L.sc_off);      // F8: [kStRing][STR] scale of each column
     StSlot* slots = reinterpret_cast<StSlot*>(smem + L.st_off);
     uint8_t* cb = smem + L.cb_off;           // kPQ: fp16 codebook, entry (code, m) at (code * 16 + m) * 16
@@ -367,11 +446,11 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
     uint64_t* qempty = qfull + QS;
     uint64_t* xfull = qempty + QS;          // [kStRing]
     uint64_t* xempty = xfull + kStRing;     // [kStRing]
-    uint64_t* umfull = xempty + kStRing;    // [UMS <= 2] unit maxima written
-    uint64_t* umempty = umfull + 2;         // [UMS <= 2] unit maxima read
-    uint64_t* scfull = umempty + 2;          // F8: [kStRing] a record slot's column scales landed
+    uint64_t* umfull = xempty + kStRing;    // [kUmSlots] row maxima written
+    uint64_t* umempty = umfull + kUmSlots;         // [kUmSlots] row maxima read
+    uint64_t* scfull = umempty + kUmSlots;          // F8: [kStRing] a record slot's column scales landed
     uint64_t* mdone = scfull + kStRing;
-    uint64_t* conv = mdone + 1;   // TF: [S] stage split
+    uint64_t* conv = mdone + kMmaWarps;   // TF: [S] stage split
     uint64_t* qconv = conv + S;   // TF: [QS] query tile split
     uint64_t* codefull = qconv + QS;            // kPQ: [kCodeRing] code rows landed
     uint64_t* codeempty = codefull + kCodeRing;  // kPQ: [kCodeRing] code rows consumed
@@ -383,35 +462,35 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < S; ++i) {
-            mbar_init(&full[i], PQ ? kSplitWarps : 1);  // kPQ: every decompressor warp wrote its rows
-            mbar_init(&empty[i], 1);
+            mbar_init(&full[i], PQ ? kHelpers : 1);  // kPQ: every decompressor warp wrote its rows
+            mbar_init(&empty[i], kMmaWarps);  // the MMAs that read it, and the other MMA warps passing it
         }
         for (int i = 0; i < KACC; ++i) {
             mbar_init(&tfull[i], 1);
-            // the epilogue warps of a half whose row block belongs to a copy
-            mbar_init(&tempty[i], a.reps * a.bpc < 4 ? a.reps * a.bpc : 4);
+            // the epilogue warps of a half whose row block belongs to a copy, and the
+            // other MMA warps passing it
+            mbar_init(&tempty[i], (H == 1 && a.reps * a.bpc < 4 ? a.reps * a.bpc : 4) + kMmaWarps - 1);
         }
         for (int i = 0; i < QS; ++i) {
             mbar_init(&qfull[i], 1);
-            mbar_init(&qempty[i], 1);
+            mbar_init(&qempty[i], kMmaWarps);
         }
         for (int i = 0; i < kStRing; ++i) {
             mbar_init(&xfull[i], 1);
             // loader, MMA, epilogue, finishers, splitters
-            mbar_init(&xempty[i], 2 + kEpiWarps + fin_warps(SH) + ((TF || PQ) ? kSplitWarps : 0));
+            mbar_init(&xempty[i], 1 + kMmaWarps + kEpiWarps + fin_warps(SH) + ((TF || PQ) ? kHelpers : 0));
         }
-        for (int i = 0; i < 2; ++i) {
-            // the epilogue warps whose row block belongs to a copy
-            mbar_init(&umfull[i], H == 2 ? 8 : (a.reps * a.bpc < 4 ? a.reps * a.bpc : 4));
-            mbar_init(&umempty[i], fin_warps(SH));
+        for (int i = 0; i < kUmSlots; ++i) {
+            mbar_init(&umfull[i], a.reps * a.bpc < 4 ? a.reps * a.bpc : 4);
+            mbar_init(&umempty[i], 1);
         }
         for (int i = 0; i < kStRing; ++i) mbar_init(&scfull[i], 32);  // one cp.async arrival per loader lane
-        mbar_init(mdone, 1);
-        for (int i = 0; i < S; ++i) mbar_init(&conv[i], kSplitWarps);
-        for (int i = 0; i < QS; ++i) mbar_init(&qconv[i], kSplitWarps);
+        for (int i = 0; i < kMmaWarps; ++i) mbar_init(&mdone[i], 1);
+        for (int i = 0; i < S; ++i) mbar_init(&conv[i], kHelpers);
+        for (int i = 0; i < QS; ++i) mbar_init(&qconv[i], kHelpers);
         for (int i = 0; i < kCodeRing; ++i) {
             mbar_init(&codefull[i], 1);
-            mbar_init(&codeempty[i], kSplitWarps);
+            mbar_init(&codeempty[i], kHelpers);
         }
         *abort_flag = 0;
         fence_mbar_init();
@@ -420,6 +499,10 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
         if (lane < kBoxKinds) prefetch_tensormap(&maps.doc[lane]);
     }
     if (warp == 0 && lane == 0) prefetch_tensormap(&maps.q);
+    if (warp == 0) {
+        bias[lane] = (lane & 7) < lane >> 3 ? 0.f : -INFINITY;
+        bias[32 + lane] = (lane & 7) < 4 + (lane >> 3) ? 0.f : -INFINITY;
+    }
     if (warp == 1) {
         tmem_alloc(tmem_slot, TCOLS);
         tmem_relinquish();
@@ -451,7 +534,6 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = *tmem_slot;
-
     if (warp == 0) {
         // ------------------------------------------------------- planner
         const uint64_t pol_keep = policy_evict_last();
@@ -461,6 +543,9 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
         // The open super-tile, written into its record slot as it fills.
         int used = 0, nseg = 0, nfin = 0, st_q = 0;  // units, tiles, documents ended, query
         unsigned ends = 0, partial = 0;
+        uint32_t shares = 0x80000000u >> (32 - STR / 8);  // last units of the shares
+        if (a.reps >= 2) shares |= shares >> (STR / 16);
+        if (a.reps >= 4) shares |= shares >> (STR / 32);
 
         // Publish the open super-tile: the record, and the query tile if the
         // query changed.
@@ -475,7 +560,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                 h.rows = 8 * used;
                 h.ends = ends;
                 h.partial = partial;
-                h.pad = 0;
+                h.values = (shares & (used == 32 ? 0xffffffffu : (1u << used) - 1u)) | ends;
                 slots[xs].h = h;
             }
             __syncwarp();
@@ -494,16 +579,9 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                     uint8_t* qdst = q_base + slot * qslot_bytes;
                     for (int kc = 0; kc < NCH; ++kc) {
                         uint8_t* cdst = qdst + kc * a.rows_alloc * 128;
-                        for (int rp = 0; rp < a.reps; ++rp) {
-                            if (SH) {  // one 32-row box per query of the group
-                                for (int g = 0; g < a.bpc; ++g)
-                                    tma_load_2d(cdst + (rp * a.bpc + g) * 32 * 128, &maps.q, kc * CE,
-                                                (st_q * a.group + g) * a.nq, &qfull[slot], pol_keep);
-                            } else {
-                                tma_load_2d(cdst + rp * a.qbox * 128, &maps.q, kc * CE, st_q * a.nq, &qfull[slot],
-                                            pol_keep);
-                            }
-                        }
+                        for (int rp = 0; rp < a.reps; ++rp)
+                            tma_load_3d(cdst + rp * a.bpc * 32 * 128, &maps.q, kc * CE, 0, st_q * (SH ? a.group : 1),
+                                        &qfull[slot], pol_keep);
                     }
                 }
                 ++qi;
@@ -521,29 +599,25 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
         }
         // three-window metadata pipeline: ids two windows ahead, offsets
         // and lengths one window ahead, the current window in registers.
-        int id_next = load_id(a, 32 + lane);
-        Meta cur = load_meta(a, load_id(a, lane));
+        const Work<SH> work(a);
+        int id_next = work.load_id(a, 32 + lane);
+        Meta cur = load_meta(a, work.load_id(a, lane));
         Meta nxt = load_meta(a, id_next);
-        int id_next2 = load_id(a, 64 + lane);
+        int id_next2 = work.load_id(a, 64 + lane);
 
         for (int64_t k0 = 0;; k0 += 32) {
-            if (static_cast<int64_t>(blockIdx.x) + k0 * gridDim.x >= a.n_flat) break;
+            if (k0 >= work.n) break;
             // lane = one candidate of the window
-            const int64_t f = static_cast<int64_t>(blockIdx.x) + (k0 + lane) * gridDim.x;
-            const bool valid = f < a.n_flat;
-            const int status = valid ? meta_status(a, cur.id, cur.off, cur.len) : 3;
+            const bool valid = k0 + lane < work.n;
             int ql = 0;
-            int64_t pos = f;  // shared mode: position in the candidate list
-            if (SH) {
-                if (valid) {
-                    ql = static_cast<int>(f / a.n_cand);
-                    pos = f - static_cast<int64_t>(ql) * a.n_cand;
-                }
-            } else {
+            int64_t pos = 0;  // entry of the list (per-query lists: flat index)
+            if (valid) work.at(a, k0 + lane, &ql, &pos);
+            const int status = valid ? meta_status(a, cur.id, cur.off, cur.len) : 3;
+            if (!SH) {
                 ql = qw;
                 int64_t qe = qw_end;
                 if (valid) {
-                    while (f >= qe && ql < a.n_queries - 1) {
+                    while (pos >= qe && ql < a.n_queries - 1) {
                         ++ql;
                         qe = __ldg(a.cand_offsets + ql + 1);
                     }
@@ -559,7 +633,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                         if (ql * a.group + g < a.n_queries)
                             a.out[static_cast<int64_t>(ql * a.group + g) * a.n_cand + pos] = v;
                 } else {
-                    a.out[f] = v;
+                    a.out[pos] = v;
                 }
                 if (status != 0) atomicOr(a.err, status == 1 ? TMS_DEVERR_BAD_ID : TMS_DEVERR_BAD_RANGE);
             }
@@ -581,7 +655,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                 const int x = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += x;
             }
-            const int fi = static_cast<int>(SH ? pos : f);
+            const int fi = static_cast<int>(pos);
             const int row = static_cast<int>(cur.off);
             constexpr int C = STR / 8;  // units of a super-tile
             unsigned docs = __ballot_sync(0xffffffffu, nu > 0);
@@ -654,7 +728,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
             if (aborted) break;
             cur = nxt;
             nxt = load_meta(a, id_next2);
-            id_next2 = load_id(a, k0 + 96 + lane);
+            id_next2 = work.load_id(a, k0 + 96 + lane);
         }
         if (!aborted && used > 0 && !close_st()) aborted = true;
         if (!aborted) {
@@ -668,7 +742,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                 h.rows = 0;
                 h.ends = 0;
                 h.partial = 0;
-                h.pad = 0;
+                h.values = 0;
                 slots[xs].h = h;
                 mbar_arrive(&xfull[xs]);
             }
@@ -778,15 +852,9 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                         // the query (group) rows of this chunk, laid out as one
                         // chunk of the resident query region
                         uint8_t* qdst = stage_base + s * SSTRIDE + STR * 128;
-                        for (int rp = 0; rp < a.reps; ++rp) {
-                            if (SH) {
-                                for (int g = 0; g < a.bpc; ++g)
-                                    tma_load_2d(qdst + (rp * a.bpc + g) * 32 * 128, &maps.q, kc * CE,
-                                                (h.q * a.group + g) * a.nq, &full[s], pol_keep);
-                            } else {
-                                tma_load_2d(qdst + rp * a.qbox * 128, &maps.q, kc * CE, h.q * a.nq, &full[s], pol_keep);
-                            }
-                        }
+                        for (int rp = 0; rp < a.reps; ++rp)
+                            tma_load_3d(qdst + rp * a.bpc * 32 * 128, &maps.q, kc * CE, 0, h.q * (SH ? a.group : 1),
+                                        &full[s], pol_keep);
                     }
                 }
                 __syncwarp();
@@ -831,7 +899,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
         // row: eight subspaces, eight distinct codebook bank groups, one
         // 128-byte store.
         const int tid = (warp - kHelpWarp) * 32 + lane;
-        constexpr int kDecThreads = 32 * kSplitWarps;
+        constexpr int kDecThreads = 32 * kHelpers;
         int s = 0;
         uint32_t ph = 0;
         for (int t = 0;; ++t) {
@@ -895,14 +963,20 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
         // Elements are independent, so the 128-byte swizzle needs no
         // decoding: x and lo keep the same byte positions.
         const int tid = (warp - kHelpWarp) * 32 + lane;
-        constexpr int kSplitThreads = 32 * kSplitWarps;
+        constexpr int kSplitThreads = 32 * kHelpers;
         auto split = [&](uint8_t* hi_p, uint8_t* lo_p, int bytes) {
             float4* hv = reinterpret_cast<float4*>(hi_p);
             float4* lv = reinterpret_cast<float4*>(lo_p);
-            for (int v = tid; v < bytes / 16; v += kSplitThreads) {
+#pragma unroll 1
+            for (int v = tid; v < bytes / 16; v += 2 * kSplitThreads) {
+                const bool two = v + kSplitThreads < bytes / 16;
                 const float4 x = hv[v];
+                const float4 y = hv[two ? v + kSplitThreads : v];
                 lv[v] = make_float4(x.x - tf32_trunc(x.x), x.y - tf32_trunc(x.y), x.z - tf32_trunc(x.z),
                                     x.w - tf32_trunc(x.w));
+                if (two)
+                    lv[v + kSplitThreads] = make_float4(y.x - tf32_trunc(y.x), y.y - tf32_trunc(y.y),
+                                                        y.z - tf32_trunc(y.z), y.w - tf32_trunc(y.w));
             }
             fence_proxy_async_smem();  // generic-proxy writes, read next by the tensor cores
             __syncwarp();
@@ -940,18 +1014,26 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
             }
             if (!ok) break;
         }
-    } else if (warp == 1) {
+    } else if (warp <= kMmaWarps) {
         // ---------------------------------------------------------- MMA
         // The whole warp runs this role, so that its control flow and the
         // descriptors are uniform -- kept in uniform registers, where the
         // MMA takes them from; a loop that one lane runs alone moves each
         // of them there for every MMA -- and one elected lane issues.
         // Descriptors advance by adding the 16-byte-unit offset of each
-        // K-step to a per-stage base.
+        // K-step to a per-stage base.  Warp w issues super-tiles w,
+        // w + kMmaWarps, ...; past the others it goes through the same waits,
+        // and its arrivals are part of their stages' and accumulators' next
+        // phases: a wait can tell a phase only from the one before it, so no
+        // phase may complete before every MMA warp has seen its predecessor
+        // (a warp that came 1 us late, on a cold instruction cache, waited
+        // for a phase that needed its own next super-tile).
+        const int mw = warp - 1;
         int s = 0;
         uint32_t ph = 0;
         int qi = 0, cur_q = -1, qslot = 0;
         bool any = false;
+        const bool half_major = H == 2 && !QSTREAM && 2 * NCH <= S;
         const uint32_t stage_sa = smem_u32(stage_base);
         for (int t = 0;; ++t) {
             const int xs = t % kStRing;
@@ -969,97 +1051,142 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                 cur_q = xq;
             }
             bool ok = true;
-            const uint64_t q_desc = desc_sw128(smem_u32(q_base) + static_cast<uint32_t>(qslot * qslot_bytes));
-            const uint64_t qlo_desc = desc_sw128(smem_u32(qlo_base) + static_cast<uint32_t>(qslot * qslot_bytes));
+            const uint32_t q_desc = desc_sw128(smem_u32(q_base) + static_cast<uint32_t>(qslot * qslot_bytes));
+            const uint32_t qlo_desc = desc_sw128(smem_u32(qlo_base) + static_cast<uint32_t>(qslot * qslot_bytes));
             const uint32_t idesc = a.idesc | (static_cast<uint32_t>(xn >> 3) << 17);
-            for (int kc = 0; kc < NCH; ++kc) {
-                if (!warp_wait(TF ? &conv[s] : &full[s], ph, abort_flag, a.err, a.budget)) {
-                    ok = false;
-                    break;
+            // K-steps of chunk kc, half hq (its operands in the current stage).
+            auto issue = [&](int kc, int hq, bool last_use) {
+                const int ab = (H * t + hq) % KACC;
+                const uint32_t d_tmem = tbase + static_cast<uint32_t>(ab * STR);
+                const uint32_t b_desc = desc_sw128(stage_sa + static_cast<uint32_t>(s * SSTRIDE));
+                const uint32_t blo_desc = desc_sw128(stage_sa + static_cast<uint32_t>(s * SSTRIDE + STAGE_BYTES));
+                const uint32_t qoff = QSTREAM ? 0u : static_cast<uint32_t>(((kc * a.rows_alloc + hq * 128) * 128) >> 4);
+                const uint32_t a_desc =
+                    QSTREAM ? desc_sw128(stage_sa + static_cast<uint32_t>(s * SSTRIDE + (STR + hq * 128) * 128))
+                            : q_desc + qoff;
+                if (elect_one()) {
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) {
+                        const uint32_t accumulate = (kc > 0 || kk > 0) ? 1u : 0u;
+                        if (TF) {  // hi.hi + hi.lo + lo.hi
+                            mma_tf32(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
+                            mma_tf32(d_tmem, a_desc + 2 * kk, blo_desc + 2 * kk, idesc, 1u);
+                            mma_tf32(d_tmem, qlo_desc + qoff + 2 * kk, b_desc + 2 * kk, idesc, 1u);
+                        } else if (F8)
+                            mma_f8(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
+                        else
+                            mma_f16(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
+                    }
+                    if (kc == NCH - 1 && (a.fault != kFaultHoldAccumulator || blockIdx.x != 0 || t != 0))
+                        mma_commit(&tfull[ab]);
+                    if (last_use) mma_commit(&empty[s]);
                 }
+            };
+            auto acc_free = [&](int hq) {
+                const int use = H * t + hq;
+                const bool got = warp_wait(&tempty[use % KACC], ((use / KACC) & 1) ^ 1, abort_flag, a.err, a.budget);
                 tc_fence_after();
-                const uint64_t b_desc = desc_sw128(stage_sa + static_cast<uint32_t>(s * SSTRIDE));
-                const uint64_t blo_desc = desc_sw128(stage_sa + static_cast<uint32_t>(s * SSTRIDE + STAGE_BYTES));
-#pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    const int use = H * t + h;
-                    const int ab = use % KACC;
-                    const uint32_t d_tmem = tbase + static_cast<uint32_t>(ab * STR);
-                    if (kc == 0) {
-                        if (!warp_wait(&tempty[ab], ((use / KACC) & 1) ^ 1, abort_flag, a.err, a.budget)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                    }
-                    const uint64_t qoff =
-                        QSTREAM ? 0 : static_cast<uint64_t>(((kc * a.rows_alloc + h * 128) * 128) >> 4);
-                    const uint64_t a_desc =
-                        QSTREAM ? desc_sw128(stage_sa + static_cast<uint32_t>(s * SSTRIDE + (STR + h * 128) * 128))
-                                : q_desc + qoff;
-                    if (elect_one()) {
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
-                            const uint32_t accumulate = (kc > 0 || kk > 0) ? 1u : 0u;
-                            if (TF) {  // hi.hi + hi.lo + lo.hi
-                                mma_tf32(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
-                                mma_tf32(d_tmem, a_desc + 2 * kk, blo_desc + 2 * kk, idesc, 1u);
-                                mma_tf32(d_tmem, qlo_desc + qoff + 2 * kk, b_desc + 2 * kk, idesc, 1u);
-                            } else if (F8)
-                                mma_f8(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
-                            else
-                                mma_f16(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
-                        }
-                        if (kc == NCH - 1 && (a.fault != kFaultHoldAccumulator || blockIdx.x != 0 || t != 0))
-                            mma_commit(&tfull[ab]);
-                    }
-                    any = true;
-                }
-                if (!ok) break;
-                if (elect_one()) mma_commit(&empty[s]);
+                return got;
+            };
+            auto stage_full = [&]() {
+                const bool got = warp_wait(TF ? &conv[s] : &full[s], ph, abort_flag, a.err, a.budget);
+                tc_fence_after();
+                return got;
+            };
+            auto advance = [&]() {
                 if (++s == S) {
                     s = 0;
                     ph ^= 1;
                 }
+            };
+            if (t % kMmaWarps != mw) {
+#pragma unroll
+                for (int hq = 0; hq < H; ++hq) {
+                    ok = ok && acc_free(hq);
+                    if (ok && elect_one()) mbar_arrive(&tempty[(H * t + hq) % KACC]);
+                }
+                for (int kc = 0; kc < NCH && ok; ++kc) {
+                    ok = stage_full();
+                    if (ok && elect_one()) mbar_arrive(&empty[s]);
+                    advance();
+                }
+                if (!ok) break;
+                continue;
             }
-            if (!ok) break;
+            any = true;
+            if (H == 2 && STR == 256 && half_major) {
+                // Half by half, where the ring holds the chunks of two
+                // super-tiles: the first half's accumulator is ready, and
+                // free again, half a super-tile earlier.
+                const int s0 = s;
+                const uint32_t ph0 = ph;
+                ok = acc_free(0);
+                for (int kc = 0; kc < NCH && ok; ++kc) {
+                    ok = stage_full();
+                    if (!ok) break;
+                    issue(kc, 0, false);
+                    advance();
+                }
+                if (!ok || !acc_free(H - 1)) break;
+                s = s0;
+                ph = ph0;
+                for (int kc = 0; kc < NCH; ++kc) {
+                    issue(kc, H - 1, true);
+                    advance();
+                }
+            } else {
+                for (int kc = 0; kc < NCH; ++kc) {
+                    ok = stage_full();
+                    if (!ok) break;
+#pragma unroll
+                    for (int hq = 0; hq < H; ++hq) {
+                        if (kc == 0 && !acc_free(hq)) {
+                            ok = false;
+                            break;
+                        }
+                        issue(kc, hq, hq == H - 1);
+                    }
+                    if (!ok) break;
+                    advance();
+                }
+                if (!ok) break;
+            }
         }
         // Every MMA this warp issued must finish before TMEM is freed.
         if (any && elect_one()) {
-            mma_commit(mdone);
-            drain_wait(mdone, 0);
+            mma_commit(&mdone[mw]);
+            drain_wait(&mdone[mw], 0);
         }
         __syncwarp();
-    } else if (warp >= kFinWarp) {
-        // ----------------------------------------------------- finishers
-        // lane = row of a 32-row block (a query token); warp w takes blocks
-        // w, w + fin_warps, ...  m[b] is the running max of the lane's row
-        // of block b over the current document's columns, carried from one
-        // super-tile to the next when a document is cut at a super-tile's
-        // end.
-        constexpr int FB = fin_blocks(H, SH);
-        constexpr int FW = fin_warps(SH);
-        const int fw = warp - kFinWarp;
-        const int nb = fw < a.bpc ? (a.bpc - fw + FW - 1) / FW : 0;  // its blocks, <= FB
-        float m[FB], qsc[FB];  // qsc, F8: the row's query-token scale, reloaded when the query changes
-#pragma unroll
-        for (int b = 0; b < FB; ++b) m[b] = -INFINITY, qsc[b] = 1.f;
-        int qsc_q = -1;
-        // Row r of block b of a document of query (group) q, if it counts.
-        auto row_value = [&](int b) {
-            const int tok = SH ? lane : b * 32 + lane;
-            return tok < a.nq ? (F8 ? m[b] * qsc[b] : m[b]) : 0.f;
-        };
+    } else {
+        // ---------------------------------------- epilogue and finisher
+        // Epilogue: thread = query row 128 hh + 32 qd + lane of the warp's
+        // half hh (TMEM lane 32 qd + lane).  A warp reduces its columns, in
+        // groups of four units, to a running max that starts again after
+        // each document's end.
+        //   * Shared lists: a warp owns one query of the group and sees all
+        //     columns, so the value at a document's end is the row's
+        //     maximum; a document that goes on keeps it in a register.
+        //   * Per-query lists: row block qd is copy qd / bpc of token block
+        //     qd % bpc; the copies hold the same sums, so each takes its
+        //     share of the columns and leaves its values -- at documents'
+        //     ends and at its last unit -- to the finisher warp, which
+        //     combines them.
+        // What counts here is the number of instructions: the warps of the
+        // SM issue 1.7 a cycle between them, whatever their number (walking
+        // the documents in every warp took 500-600 instructions per 128
+        // columns; values and finishers for shared lists too, 7,600 per
+        // 256-row super-tile over all warps).
+        //
         // Documents are finished in batches: their 32 row maxima (times the
-        // query-token scales, F8; 0 past nq) go to this warp's rows in
-        // shared memory, and when they are full lane r sums row r in token
-        // order and stores the score -- the same fixed order for every
-        // document, wherever it sits in a batch.  With several 32-token
-        // blocks per query (nq > 32) each block is summed across the warp
-        // and the blocks are added in order instead.
-        const bool batched = SH || a.bpc == 1;
-        float* fin_rows = reinterpret_cast<float*>(fin_base + fw * kFinWarpBytes);
-        int* fin_ids = reinterpret_cast<int*>(fin_base + fw * kFinWarpBytes + kFinRows * 33 * 4);
+        // query-token scales, F8; 0 past nq) go to the warp's rows in shared
+        // memory, and when they are full lane r sums row r in token order
+        // and stores the score -- the same fixed order for every document,
+        // wherever it sits in a batch.
+        const bool finisher = !SH && warp >= kFinWarp;
+        const int ew = finisher || !SH ? 0 : warp - kEpiWarp;
+        float* fin_rows = reinterpret_cast<float*>(fin_base + ew * kFinWarpBytes);
+        int* fin_ids = reinterpret_cast<int*>(fin_base + ew * kFinWarpBytes + kFinRows * 33 * 4);
         int nfin = 0;  // rows in use
         auto flush = [&]() {
             __syncwarp();
@@ -1071,7 +1198,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
 #pragma unroll
                 for (int i = 0; i < 32; ++i) sum += x[i];
                 const int f = fin_ids[2 * lane];
-                const int qq = fin_ids[2 * lane + 1];  // shared mode: the row's query
+                const int qq = fin_ids[2 * lane + 1];  // shared lists: the row's query
                 if (SH) {
                     if (qq < a.n_queries) a.out[static_cast<int64_t>(qq) * a.n_cand + f] = sum;
                 } else {
@@ -1081,158 +1208,235 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
             __syncwarp();
             nfin = 0;
         };
-        for (int t = 0;; ++t) {
-            const int xs = t % kStRing;
-            if (!warp_wait(&xfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
-            const StHdr xh = slots[xs].h;
-            if (xh.flags & kEnd) break;
-            if (F8 && xh.q != qsc_q) {
-                qsc_q = xh.q;
+        if (finisher) {
+            // lane = row of a token block; m[b] is the running max of block
+            // b's row over the current document's columns, carried from one
+            // super-tile to the next when a document is cut at a
+            // super-tile's end.  With several blocks per query (nq > 32)
+            // each block is summed across the warp and the blocks are added
+            // in order.
+            float m[kMaxBlocks], qsc[kMaxBlocks];  // qsc, F8: the row's query-token scale
 #pragma unroll
-                for (int b = 0; b < FB; ++b) {
-                    const int blk = fw + b * FW;
-                    const int qq = SH ? xh.q * a.group + blk : xh.q;
-                    const int tok = SH ? lane : blk * 32 + lane;
-                    qsc[b] = (b < nb && tok < a.nq && qq < a.n_queries)
-                                 ? __ldg(a.q_scales + static_cast<int64_t>(qq) * a.nq + tok)
-                                 : 0.f;
+            for (int b = 0; b < kMaxBlocks; ++b) m[b] = -INFINITY, qsc[b] = 1.f;
+            int qsc_q = -1;
+            auto row_value = [&](int b) {
+                return b * 32 + lane < a.nq ? (F8 ? m[b] * qsc[b] : m[b]) : 0.f;
+            };
+            for (int t = 0;; ++t) {
+                const int xs = t % kStRing;
+                if (!warp_wait(&xfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
+                const StHdr xh = slots[xs].h;
+                if (xh.flags & kEnd) break;
+                if (F8 && xh.q != qsc_q) {
+                    qsc_q = xh.q;
+#pragma unroll
+                    for (int b = 0; b < kMaxBlocks; ++b)
+                        qsc[b] = b * 32 + lane < a.nq
+                                     ? __ldg(a.q_scales + static_cast<int64_t>(xh.q) * a.nq + b * 32 + lane)
+                                     : 0.f;
                 }
-            }
-            const int us = t % UMS;
-            if (!warp_wait(&umfull[us], (t / UMS) & 1, abort_flag, a.err, a.budget)) break;
-            const float* um = reinterpret_cast<const float*>(um_base + us * L.um_stride) + fw * 32 + lane;
-            // Units with a value: a document's last one, and the last one of
-            // a copy's share of the columns, where its document goes on.
-            uint32_t shares = 0x80000000u >> (32 - STR / 8);
-            if (a.reps >= 2) shares |= shares >> (STR / 16);
-            if (a.reps >= 4) shares |= shares >> (STR / 32);
-            const int units = xh.rows >> 3;
-            uint32_t todo = (shares & (units == 32 ? 0xffffffffu : (1u << units) - 1u)) | xh.ends;
-            int e = 0;  // documents ended so far in this super-tile
+                const int us = t % kUmSlots;
+                if (!warp_wait(&umfull[us], (t / kUmSlots) & 1, abort_flag, a.err, a.budget)) break;
+                const float* um = reinterpret_cast<const float*>(um_base + us * L.um_stride) + lane;
+                uint32_t todo = xh.values;
+                int e = 0;  // documents ended so far in this super-tile
 #pragma unroll 1
-            while (todo != 0u) {
-                const int u = __ffs(todo) - 1;
-                todo &= todo - 1u;
+                while (todo != 0u) {
+                    const int u = __ffs(todo) - 1;
+                    todo &= todo - 1u;
+                    m[0] = fmaxf(m[0], um[u * a.bpc * 32]);
+                    if (a.bpc > 1) {
 #pragma unroll
-                for (int b = 0; b < FB; ++b)
-                    if (b < nb) m[b] = fmaxf(m[b], um[(u * a.bpc + b * FW) * 32]);
-                if ((xh.ends >> u) & 1u) {
+                        for (int b = 1; b < kMaxBlocks; ++b)
+                            if (b < a.bpc) m[b] = fmaxf(m[b], um[(u * a.bpc + b) * 32]);
+                    }
+                    if (((xh.ends >> u) & 1u) == 0u) continue;
                     const int f = slots[xs].f[e++];
-                    if (batched) {
-#pragma unroll
-                        for (int b = 0; b < (SH ? FB : 1); ++b) {
-                            if (b < nb) {
-                                fin_rows[nfin * 33 + lane] = row_value(b);
-                                if (lane == 0) {
-                                    fin_ids[2 * nfin] = f;
-                                    fin_ids[2 * nfin + 1] = xh.q * a.group + fw + b * FW;
-                                }
-                                ++nfin;
-                            }
-                        }
-                        if (nfin > kFinRows - FB) flush();
+                    if (a.bpc == 1) {
+                        fin_rows[nfin * 33 + lane] = row_value(0);
+                        if (lane == 0) fin_ids[2 * nfin] = f;
+                        if (++nfin == kFinRows) flush();
                     } else {
-                        float tot = 0.f;
+                        float tot = warp_sum(row_value(0));
 #pragma unroll
-                        for (int b = 0; b < FB; ++b) {
-                            if (b < nb) {
-                                const float sum = warp_sum(row_value(b));
-                                tot = b == 0 ? sum : tot + sum;
-                            }
+                        for (int b = 1; b < kMaxBlocks; ++b) {
+                            if (b < a.bpc) tot += warp_sum(row_value(b));
+                            m[b] = -INFINITY;
                         }
                         if (lane == 0) a.out[f] = tot;
                     }
-#pragma unroll
-                    for (int b = 0; b < FB; ++b) m[b] = -INFINITY;
+                    m[0] = -INFINITY;
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&umempty[us]);
+                    mbar_arrive(&xempty[xs]);
                 }
             }
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(&umempty[us]);
-                mbar_arrive(&xempty[xs]);
+        } else {
+            const int qd = warp & 3;
+            const int hh = H == 2 ? (warp - kEpiWarp) >> 2 : 0;
+            const int copy = SH ? 0 : qd / a.bpc;
+            const int blk = 4 * hh + qd - copy * a.bpc;  // token block, or query of the group
+            const bool active = SH ? blk < a.bpc : copy < a.reps;
+            const int share = SH ? STR / 8 : STR / 8 / a.reps;  // units per copy, a multiple of 4
+            const int ua = copy * share;                        // the warp's first
+            // F8: columns are read in blocks, two columns of four rows per
+            // thread and unit, so that a thread needs two row scales per unit
+            // and not eight: broadcast to every lane, 32 scales per group
+            // took more of the shared-memory pipe than the MMAs left (with
+            // 256-column MMAs running, 42-61 cycles per group and SM against
+            // 11 for the load and the maxima; measured).  m[i] is then the
+            // running max of row lane / 4 + 8 (i % 2) + 16 (i / 2) over this
+            // thread's columns, and `row` the row it speaks for once the four
+            // threads of a row are combined.
+            constexpr int MR = F8 ? 4 : 1;
+            const int row = F8 ? (lane >> 2) + 8 * (lane & 1) + 16 * ((lane >> 1) & 1) : lane;
+            float m[MR], qsc = 1.f;  // qsc, F8, shared lists: the row's query-token scale
+#pragma unroll
+            for (int i = 0; i < MR; ++i) m[i] = -INFINITY;
+            // The row's running max; it starts again.
+            auto take_max = [&]() -> float {
+                float x = m[0];
+                if constexpr (F8) {
+                    const bool b0 = (lane & 1) != 0, b1 = (lane & 2) != 0;
+                    const float y0 = fmaxf(b0 ? m[1] : m[0], __shfl_xor_sync(0xffffffffu, b0 ? m[0] : m[1], 1));
+                    const float y1 = fmaxf(b0 ? m[3] : m[2], __shfl_xor_sync(0xffffffffu, b0 ? m[2] : m[3], 1));
+                    x = fmaxf(b1 ? y1 : y0, __shfl_xor_sync(0xffffffffu, b1 ? y0 : y1, 2));
+                }
+#pragma unroll
+                for (int i = 0; i < MR; ++i) m[i] = -INFINITY;
+                return x;
+            };
+            int qsc_q = -1;
+            for (int t = 0;; ++t) {
+                const int xs = t % kStRing;
+                if (!warp_wait(&xfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
+                const StHdr xh = slots[xs].h;
+                if (xh.flags & kEnd) break;
+                if (!active) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&xempty[xs]);
+                    continue;
+                }
+                const int units = xh.rows >> 3;
+                const int u1 = min(units, ua + share);
+                const int us = t % kUmSlots;
+                float* um_out = reinterpret_cast<float*>(um_base + us * L.um_stride) + blk * 32 + row;
+                const float* scol = sc + xs * STR;  // F8: scale of each column's document row
+                const int use = H * t + hh;
+                const int ab = use % KACC;
+                const uint32_t tacc = tbase + (static_cast<uint32_t>(qd * 32) << 16) + static_cast<uint32_t>(ab * STR);
+                const int qq = SH ? xh.q * a.group + blk : 0;
+                if (SH && F8 && xh.q != qsc_q) {
+                    qsc_q = xh.q;
+                    qsc = row < a.nq && qq < a.n_queries
+                              ? __ldg(a.q_scales + static_cast<int64_t>(qq) * a.nq + row)
+                              : 0.f;
+                }
+                if (!SH && !warp_wait(&umempty[us], ((t / kUmSlots) & 1) ^ 1, abort_flag, a.err, a.budget)) break;
+                if (F8 && !warp_wait(&scfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
+                if (!warp_wait(&tfull[ab], (use / KACC) & 1, abort_flag, a.err, a.budget)) break;
+                tc_fence_after();
+                const int* ended = slots[xs].f;  // SH: the documents that end here
+                // Unit u ends a document: its row maximum is x.
+                auto end_doc = [&](int u, float x) {
+                    if (SH) {
+                        fin_rows[nfin * 33 + row] = row < a.nq ? (F8 ? x * qsc : x) : 0.f;
+                        ++nfin;
+                    } else {
+                        um_out[u * a.bpc * 32] = x;
+                    }
+                };
+#pragma unroll 1
+                for (int u = ua; u < u1; u += 4) {  // a group of four units: 32 columns
+                    const uint32_t eg = (xh.ends >> u) & 15u;
+                    const uint32_t taddr = tacc + static_cast<uint32_t>(8 * u);
+                    auto landed = [&]() {  // after the last load: hand the accumulator back
+                        if (u + 4 >= u1) {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(&tempty[ab]);
+                        }
+                    };
+                    auto list_ended = [&]() {
+                        if (SH) {
+                            const int n = __popc(eg);
+                            if (lane < n) {
+                                fin_ids[2 * (nfin + lane)] = ended[lane];
+                                fin_ids[2 * (nfin + lane) + 1] = qq;
+                            }
+                            ended += n;
+                        }
+                    };
+                    if constexpr (F8) {
+                        uint32_t r[2][16];
+                        tmem_ld_blocks(taddr, r);
+                        landed();
+                        const float2* scales = reinterpret_cast<const float2*>(scol + 8 * u) + (lane & 3);
+                        float v[4][MR][2];  // [unit][row][column], scaled; columns past a document's end are NaN
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const float2 sc2 = scales[4 * k];
+#pragma unroll
+                            for (int i = 0; i < MR; ++i) {
+                                v[k][i][0] = __uint_as_float(r[i >> 1][4 * k + 2 * (i & 1)]);
+                                v[k][i][1] = __uint_as_float(r[i >> 1][4 * k + 2 * (i & 1) + 1]);
+                                mul_f32x2(v[k][i][0], v[k][i][1], sc2.x, sc2.y);
+                            }
+                        }
+                        if (eg == 0u) {
+#pragma unroll
+                            for (int i = 0; i < MR; ++i)
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) m[i] = fmax3(m[i], v[k][i][0], v[k][i][1]);
+                            continue;
+                        }
+                        list_ended();
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+#pragma unroll
+                            for (int i = 0; i < MR; ++i) m[i] = fmax3(m[i], v[k][i][0], v[k][i][1]);
+                            if ((eg >> k) & 1u) end_doc(u + k, take_max());
+                        }
+                    } else {
+                        float v[32], um[4];
+                        tmem_ld32(taddr, v);
+                        landed();
+                        unit_maxima_counted(v, um, (xh.partial >> u) & 15u, slots[xs].valid + u, bias);
+                        if (eg == 0u) {
+                            m[0] = fmax3(m[0], fmax3(um[0], um[1], um[2]), um[3]);
+                            continue;
+                        }
+                        list_ended();
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            m[0] = fmaxf(m[0], um[k]);
+                            if ((eg >> k) & 1u) end_doc(u + k, take_max());
+                        }
+                    }
+                    if (SH && nfin > kFinRows - 4) flush();
+                }
+                if (ua >= u1) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&tempty[ab]);
+                }
+                // the share's last unit, unless a document (or the super-tile) ended before or there
+                if (!SH && ua + share <= units && ((xh.ends >> (ua + share - 1)) & 1u) == 0u)
+                    end_doc(ua + share - 1, take_max());
+                // nothing goes on; m may hold columns past the super-tile's last unit
+                if (!SH || ((xh.ends >> (units - 1)) & 1u) != 0u) {
+#pragma unroll
+                    for (int i = 0; i < MR; ++i) m[i] = -INFINITY;
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    if (!SH) mbar_arrive(&umfull[us]);
+                    mbar_arrive(&xempty[xs]);
+                }
             }
         }
         if (nfin > 0) flush();
-    } else {
-        // ----------------------------------------------------- epilogue
-        // Thread = query row 128 hh + 32 qd + lane of the warp's half hh (TMEM
-        // lane 32 qd + lane).  Row block 4 hh + qd is copy (4 hh + qd) / bpc
-        // of block (4 hh + qd) % bpc; the copies hold the same sums, so each
-        // copy's warps take their share of the columns.  A warp reduces its
-        // columns to a running max that starts again after each document's
-        // end, and leaves its value at every end and at its last unit to the
-        // finishers, which know whose columns they are: the code is short
-        // and nearly free of branches, and every warp has the same work.
-        // (Walking the documents and summing their rows here took 500-600
-        // instructions per warp for 128 columns of a shared list.)
-        const int qd = warp & 3;
-        const int hh = (warp - 2) >> 2;  // 0 for H = 1
-        const int copy = H == 1 ? qd / a.bpc : 0;
-        const int blk = 4 * hh + qd - copy * a.bpc;  // block of the copy: token block, or query of the group
-        const bool active = copy < a.reps;
-        const int share = STR / 8 / a.reps;  // units per copy, a multiple of 4
-        for (int t = 0;; ++t) {
-            const int xs = t % kStRing;
-            if (!warp_wait(&xfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
-            const StHdr xh = slots[xs].h;
-            if (xh.flags & kEnd) break;
-            if (!active) {
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&xempty[xs]);
-                continue;
-            }
-            const int units = xh.rows >> 3;
-            const int u1 = min(units, (copy + 1) * share);
-            const int us = t % UMS;
-            float* um_out = reinterpret_cast<float*>(um_base + us * L.um_stride) + blk * 32 + lane;
-            const float* scol = sc + xs * STR;  // F8: scale of each column's document row
-            const int use = H * t + hh;
-            const int ab = use % KACC;
-            const uint32_t tacc = tbase + (static_cast<uint32_t>(qd * 32) << 16) + static_cast<uint32_t>(ab * STR);
-            if (!warp_wait(&umempty[us], ((t / UMS) & 1) ^ 1, abort_flag, a.err, a.budget)) break;
-            if (F8 && !warp_wait(&scfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
-            if (!warp_wait(&tfull[ab], (use / KACC) & 1, abort_flag, a.err, a.budget)) break;
-            tc_fence_after();
-            float m = -INFINITY;
-#pragma unroll 1
-            for (int u = copy * share; u < u1; u += 4) {  // a group of four units: 32 columns
-                float v[32], um[4];
-                tmem_ld32(tacc + static_cast<uint32_t>(8 * u), v);
-                if (F8) scale32(v, scol + 8 * u);  // columns past a document's end have scale NaN
-                unit_maxima(v, um);
-                if (!F8 && ((xh.partial >> u) & 15u) != 0u) {
-                    const uint8_t* valid = slots[xs].valid + u;
-                    if ((xh.partial >> u) & 1u) um[0] = unit_max_n<0>(v, valid[0]);
-                    if ((xh.partial >> u) & 2u) um[1] = unit_max_n<1>(v, valid[1]);
-                    if ((xh.partial >> u) & 4u) um[2] = unit_max_n<2>(v, valid[2]);
-                    if ((xh.partial >> u) & 8u) um[3] = unit_max_n<3>(v, valid[3]);
-                }
-                const uint32_t eg = (xh.ends >> u) & 15u;
-                if (eg == 0u) {
-                    m = fmax3(m, fmax3(um[0], um[1], um[2]), um[3]);
-                } else {
-                    float* o = um_out + u * a.bpc * 32;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        m = fmaxf(m, um[k]);
-                        if ((eg >> k) & 1u) {
-                            o[k * a.bpc * 32] = m;
-                            m = -INFINITY;
-                        }
-                    }
-                }
-            }
-            // the share's last unit, unless a document (or the whole super-tile) ended before or there
-            const int ul = (copy + 1) * share - 1;
-            if (ul < units && ((xh.ends >> ul) & 1u) == 0u) um_out[ul * a.bpc * 32] = m;
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(&tempty[ab]);
-                mbar_arrive(&umfull[us]);
-                mbar_arrive(&xempty[xs]);
-            }
-        }
     }
 
     tc_fence_before();
@@ -1292,6 +1496,11 @@ inline TuneKey group_key(int device, int kind, int nchunks, int n_queries) {
 // The configurations an instantiation has kernels for.
 template <int H, bool SH, int KIND>
 inline int config_shapes(Config* out) {
+    if (H == 2 && KIND != kPQ) {
+        out[0] = {256, 1, 0, 0, 0, 0};
+        out[1] = {128, 1, 0, 0, 0, 0};
+        return 2;
+    }
     if (H == 2 || KIND == kTF32) {
         out[0] = {128, 1, 0, 0, 0, 0};
         return 1;
@@ -1315,8 +1524,7 @@ inline int config_shapes(Config* out) {
 // stages twice the size) take one CTA with 128-row super-tiles.  KIND
 // selects the row type; kE4M3 ignores `dtype` (rows are E4M3 codes;
 // t_scales in `a`).  The caller sets a.nchunks = ceil(d / chunk_elems(KIND)),
-// and a.bpc / a.qbox: per-query ceil(nq / 32) and 32 bpc, shared mode the
-// group size and 32.  `force` (the autotuner's) overrides the choice;
+// and a.bpc: per-query ceil(nq / 32), shared mode the group size.  `force` (the autotuner's) overrides the choice;
 // TMS_ERR_UNSUPPORTED when it does not fit.
 // The resolved launch configuration: every field of Config set (qslots 0:
 // the query is streamed).
@@ -1339,10 +1547,11 @@ tms_status plan_tc(const DeviceInfo& dev, const Args& a, const Config* force, Pl
     // Shared-memory plan for (rows per super-tile, CTAs per SM, copies):
     // the query-slot count (2, else 1) that gives the most stages; the
     // plan fits with at least 4 chunk stages (2 with one CTA per SM).
-    const int max_reps = H == 2 ? 1 : (a.bpc == 3 ? 1 : 4 / a.bpc);
+    const int max_reps = SH ? 1 : (a.bpc == 3 ? 1 : 4 / a.bpc);
     auto fits = [&](int str, int ctas, int rp, int need, int& stages, int& qslots, int cap = 0, int want_qs = 0,
                     bool stream = false) {
         if (rp < 1 || rp > max_reps) return false;
+        if (H == 2 && PQ && str != 128) return false;
         if (stream && (TF || PQ)) return false;  // their query tiles are split / decompressed in place
         const int limit = ctas == 2 ? dev.smem_per_sm / 2 - dev.smem_reserved - 1024
                                     : std::min(kSmemLimit, dev.max_smem_optin) - 1024;
@@ -1350,7 +1559,7 @@ tms_status plan_tc(const DeviceInfo& dev, const Args& a, const Config* force, Pl
         for (int qs = stream ? 0 : 2; qs >= (stream ? 0 : 1); --qs) {
             if (!stream && want_qs && qs != want_qs) continue;
             const Layout L0 = make_layout(0, qs, a.nchunks, 32 * a.bpc * rp, str, KIND, acc_count(str, ctas),
-                                          a.bpc, fin_warps(SH), stream ? 128 * H : 0);
+                                          a.bpc, SH, stream ? 128 * H : 0, H);
             int sts = std::min(kMaxStages, (limit - L0.total) / (L0.stage_stride + 24));
             if (cap > 0 && sts > cap) sts = cap;
             if (sts > best) {
@@ -1391,6 +1600,8 @@ tms_status plan_tc(const DeviceInfo& dev, const Args& a, const Config* force, Pl
     if (ctas == 0) {
         if (PQ && H == 1) {
             if (plan(256, 1, stages, qslots, reps)) str = 256, ctas = 1;
+        } else if (H == 2 && !PQ && fits(256, 1, 1, 3, stages, qslots)) {
+            str = 256, ctas = 1, reps = 1;
         } else if (H == 2 || TF) {
             if (plan(128, 1, stages, qslots, reps)) str = 128, ctas = 1;
         } else if (!SH && a.nchunks == 1) {
@@ -1410,7 +1621,7 @@ tms_status plan_tc(const DeviceInfo& dev, const Args& a, const Config* force, Pl
     if (ctas == 0 && !TF && !PQ) {
         // the resident query tile leaves no room: stream it with every chunk
         // stage (the copies a 128-row half needs, at least two stages)
-        const int sh[2][2] = {{H == 2 ? 128 : 256, 1}, {128, 1}};
+        const int sh[2][2] = {{256, 1}, {128, 1}};
         for (int i = 0; i < 2 && ctas == 0; ++i)
             for (int rp = max_reps; rp >= 1 && ctas == 0; rp /= 2)
                 if (fits(sh[i][0], sh[i][1], rp, 2, stages, qslots, 0, 0, true)) {
@@ -1422,6 +1633,30 @@ tms_status plan_tc(const DeviceInfo& dev, const Args& a, const Config* force, Pl
     if (ctas == 0) return TMS_ERR_UNSUPPORTED;
     *out = Plan{str, ctas, reps, stages, qslots};
     return TMS_OK;
+}
+
+// Shared lists: the rounds in which `groups` groups share `grid` CTAs (see
+// Work).  A round of g groups gives each floor(grid / g) CTAs, so few rounds
+// (few passes over the documents) are weighed against CTAs left over: the
+// fewest rounds that keep 97% of the CTAs busy, else those that keep most.
+// At most 16 groups at a time, so that they stay close to one another.
+inline void plan_rounds(int grid, int groups, Args* a) {
+    double best = 0;
+    for (int rounds = (groups + 15) / 16; rounds <= groups; ++rounds) {
+        const int full = (groups + rounds - 1) / rounds;
+        if ((rounds - 1) * full >= groups) continue;
+        const int last = groups - (rounds - 1) * full;
+        if (grid / full == 0) continue;
+        const double time = static_cast<double>(rounds - 1) / (grid / full) + 1.0 / (grid / last);
+        const double busy = groups / (grid * time);
+        if (busy > best) {
+            best = busy;
+            a->rounds = rounds;
+            a->round_groups = full;
+            a->last_groups = last;
+        }
+        if (best >= 0.97) break;
+    }
 }
 
 template <int H, bool SH, int KIND>
@@ -1445,8 +1680,9 @@ tms_status launch_tc(const DeviceInfo& dev, const void* queries, tms_dtype dtype
     // maps; describe the query buffer so that they still encode.
     const void* dbase = n_tokens > 0 ? doc_tokens : queries;
     Maps maps;
-    st = encode_tmap_2d(&maps.q, tdt, queries, d, static_cast<uint64_t>(n_queries) * nq, row_bytes, CE,
-                        static_cast<uint32_t>(a.qbox));
+    // one query's token blocks, or a group's queries of 32 rows each: rows past nq are zeros
+    st = encode_tmap_3d(&maps.q, tdt, queries, d, static_cast<uint64_t>(nq), static_cast<uint64_t>(n_queries), row_bytes,
+                        CE, static_cast<uint32_t>(SH ? 32 : 32 * a.bpc), static_cast<uint32_t>(SH ? a.bpc : 1));
     if (st != TMS_OK) return st;
     a.reps = reps;
     a.rows_alloc = 32 * a.bpc * reps;
@@ -1463,10 +1699,12 @@ tms_status launch_tc(const DeviceInfo& dev, const void* queries, tms_dtype dtype
     a.stages = stages;
     a.qslots = qslots;
     const Layout L = make_layout(stages, qslots, a.nchunks, a.rows_alloc, str, KIND, acc_count(str, ctas),
-                                 a.bpc, fin_warps(SH), qslots == 0 ? 128 * H : 0);
+                                 a.bpc, SH, qslots == 0 ? 128 * H : 0, H);
     const int smem = L.total + 1024;
     void (*kern)(const Maps, const Args);
-    if constexpr (H == 2) {
+    if constexpr (H == 2 && !PQ) {
+        kern = str == 256 ? dense_tc_kernel<2, 256, 1, SH, KIND> : dense_tc_kernel<2, 128, 1, SH, KIND>;
+    } else if constexpr (H == 2) {
         kern = dense_tc_kernel<2, 128, 1, SH, KIND>;
     } else if constexpr (PQ) {
         kern = dense_tc_kernel<1, 256, 1, true, kPQ>;  // H == 2 took the first branch
@@ -1479,6 +1717,7 @@ tms_status launch_tc(const DeviceInfo& dev, const void* queries, tms_dtype dtype
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return launch_status(cudaErrorInvalidValue);
     const int64_t grid = std::min<int64_t>(static_cast<int64_t>(dev.sm_count) * ctas, a.n_flat);
+    if (SH) plan_rounds(static_cast<int>(grid), static_cast<int>(a.n_flat / a.n_cand), &a);
     return launch_status(launch_dependent(kern, dim3(static_cast<unsigned>(grid)), dim3(kernel_threads(KIND, H, SH)),
                                           static_cast<size_t>(smem), stream, maps, a));
 }
@@ -1577,7 +1816,6 @@ inline tms_status shared_group_launch(const DeviceInfo& dev, const void* queries
     a.n_flat = n_groups * a.n_cand;
     a.group = group;
     a.bpc = group;
-    a.qbox = 32;
     if (tune)
         return group == 8 ? tune_tc<2, true, KIND>(dev, queries, dtype, n_queries, nq, d, doc_tokens, n_tokens, a,
                                                     stream, n_timed, ms, false)

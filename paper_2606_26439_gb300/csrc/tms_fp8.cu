@@ -237,7 +237,6 @@ tms_status score(const uint8_t* q_codes, const float* q_scales, int n_queries, i
     a.n_flat = n_cand;
     a.group = 0;
     a.bpc = (nq + 31) / 32;
-    a.qbox = 32 * a.bpc;
     if (tune)
         return dense::tune_tc<1, false, dense::kE4M3>(dev, q_codes, TMS_F16, n_queries, nq, d, doc_codes, n_tokens, a,
                                                       stream, n_configs);

@@ -31,6 +31,11 @@ tms_status current_device(DeviceInfo* out);
 tms_status encode_tmap_2d(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, uint64_t cols,
                           uint64_t rows, uint64_t row_bytes, uint32_t box_cols, uint32_t box_rows);
 
+// The same for `planes` planes of `rows` rows each, one after another, and a
+// box of box_cols x box_rows x box_planes; rows past a plane's end are zeros.
+tms_status encode_tmap_3d(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, uint64_t cols,
+                          uint64_t rows, uint64_t planes, uint64_t row_bytes, uint32_t box_cols, uint32_t box_rows,
+                          uint32_t box_planes);
 
 // Diagnostics set by tms_debug_set, read when a launch is prepared: the
 // bound of every pipeline wait in SM cycles (0 = the kernels' default) and

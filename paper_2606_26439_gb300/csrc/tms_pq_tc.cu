@@ -62,7 +62,6 @@ extern "C" tms_status tms_score_pq_tc_shared(const void* queries, tms_dtype qdty
         a.n_flat = n_groups * n_cand;
         a.group = group;
         a.bpc = group;
-        a.qbox = 32;
         st = group == 8
                  ? dense::launch_tc<2, true, dense::kPQ>(dev, queries, TMS_F16, n_queries, nq, d, codes, n_tokens, a,
                                                          stream)

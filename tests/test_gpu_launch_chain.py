@@ -104,3 +104,29 @@ def test_pq_table_scoring_topk_chain_matches_synchronised_runs(cuda_lib):
         if i == n_iter - 1:
             assert torch.equal(out.view(torch.int32), alone.view(torch.int32))
         assert torch.equal(tp[i], a_p) and torch.equal(ts[i].view(torch.int32), a_s.view(torch.int32)), i
+
+
+@pytest.mark.parametrize("dtype,n_docs,nd,d", [("f16", 10_000, 128, 128), ("f16", 2_000, 33, 64), ("f32", 3_000, 128, 128)])
+def test_many_chained_passes_never_wait_out(cuda_lib, dtype, n_docs, nd, d):
+    """Hundreds of back-to-back score -> top-k passes, each starting on SMs
+    whose instruction caches hold the other kernel: no wait of the scoring
+    pipeline may run out (the roles of a CTA may start late by microseconds,
+    in any order), and every pass gives the same bits."""
+    import torch
+    from paper_2606_26439_gb300 import tms
+    tok, off, ln = synth.device_dense_corpus(synth.lengths_fixed(n_docs, nd), d, dtype, 3)
+    q = synth.device_unit_rows(32, d, dtype, 3, 9).view(1, 32, d)
+    cand = synth.device_candidates(n_docs, n_docs, 3, 0)
+    co = torch.tensor([0, n_docs], dtype=torch.int64, device="cuda")
+    ws = torch.empty(max(16, tms.topk_workspace_size(1, 10, n_docs)), dtype=torch.uint8, device="cuda")
+    outs = torch.empty((8, n_docs), dtype=torch.float32, device="cuda")
+    tms.device_error()
+    for i in range(400):
+        tms.score_dense(q, tok, off, ln, cand, co, out=outs[i % 8])
+        top = tms.topk_split(outs[i % 8], co, 10, n_docs, workspace=ws)
+    torch.cuda.synchronize()
+    assert tms.device_error() == 0
+    want = outs[0].cpu().numpy().view(np.uint32)
+    for o in outs[1:]:
+        assert np.array_equal(o.cpu().numpy().view(np.uint32), want)
+    assert np.array_equal(top[1].cpu().numpy()[0], np.argsort(-outs[0].cpu().numpy(), kind="stable")[:10])
