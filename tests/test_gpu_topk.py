@@ -136,3 +136,26 @@ def test_topk_bad_csr_is_flagged_not_read(cuda_lib):
         assert list(tp[0]) == [-1, -1, -1]          # negative start: empty
         assert list(tp[1]) == [-1, -1, -1]          # 40 > 30: clamped to empty
         assert list(tp[2]) == [69, 68, 67]          # [30, 100): positions within the list
+
+
+@pytest.mark.parametrize("k", [1, 16, 17, 32, 33, 255, 256, 257])
+def test_topk_bounded_selection_edges(cuda_lib, k):
+    """Around the sizes where the selection changes form: lists held 4 or 20
+    keys per thread or re-read, fewer elements than threads or warps, k at the
+    steps of the per-warp rounds and on both sides of its limit; scores with
+    exactly as many ties at the cut as the survivor buffer holds, one more,
+    and sorted both ways (the top in one warp's share)."""
+    g = np.random.default_rng(1000 + k)
+    lists = [g.standard_normal(n).astype(np.float32)
+             for n in (31, 32, 33, 1023, 1024, 1025, 4095, 4096, 4097, 20_479, 20_480, 20_481)]
+    lists += [np.arange(6000, dtype=np.float32), -np.arange(21_000, dtype=np.float32)]
+    for ties in (1023, 1024, 1025, 3000):
+        x = -1.0 - g.random(9000).astype(np.float32)
+        x[g.permutation(9000)[:ties]] = 2.0
+        lists.append(x)
+    x = np.full(5000, np.nan, np.float32)
+    x[g.permutation(5000)[:k // 2]] = -np.inf
+    lists.append(x)
+    _check(lists, k)
+    for y in lists:  # each alone: the split form cuts by its own length
+        _check([y], k)
