@@ -86,8 +86,9 @@ constexpr int kMaxSeg = 32;                   // tiles per super-tile (each >= 8
 // Super-tile records in flight.  A record slot is republished only after
 // every role has passed it, so the ring also bounds how far the loader can
 // run ahead of the epilogue: with HBM latencies of a few microseconds under
-// load, the loads of many super-tiles must be in flight at once.
-__host__ __device__ constexpr int st_ring(int) { return 16; }
+// load, the loads of many super-tiles must be in flight at once: 16 of 128
+// rows, 8 of 256.
+__host__ __device__ constexpr int st_ring(int str) { return str == 256 ? 8 : 16; }
 // Epilogue warps: one per tensor-memory lane quarter and query half.
 __host__ __device__ constexpr int epi_warps(int h) { return 4 * h; }
 // Warps that prepare every chunk stage.  TF: splitters -- four of them took
@@ -106,11 +107,20 @@ constexpr int kMmaWarps = 2;
 __host__ __device__ constexpr int kernel_threads(int kind, int h, bool sh) {
     return 32 * (2 + kMmaWarps + epi_warps(h) + fin_warps(sh) + ((kind == kTF32 || kind == kPQ) ? help_warps(kind) : 0));
 }
+// Split TF32 with the query's hi and lo parts in tensor memory as the MMA's A
+// operand, where they fit (QT: 32 columns each per 32-element chunk, up to
+// kQueryCols): the MMAs, three per K-step over 128 columns, then read 64 B of
+// shared memory a cycle instead of 128, beside the fills and the splits of the
+// stages (32 B each); the query tile needs no copies and no lo twin in shared
+// memory, which leaves room for two more stages.
+constexpr int kQueryCols = 256;
+constexpr int kQueryChunks = kQueryCols / 64;
 // Accumulator buffers of STR tensor-memory columns -- one holds one query
 // half of a super-tile -- as many as the SM's 512 columns give the CTAs
 // sharing it, at most four.
-__host__ __device__ constexpr int acc_count(int str, int ctas) {
-    return 512 / (str * ctas) < 4 ? 512 / (str * ctas) : 4;
+__host__ __device__ constexpr int acc_count(int str, int ctas, bool qt) {
+    const int n = (512 - (qt ? kQueryCols : 0)) / (str * ctas);
+    return n < 4 ? n : 4;
 }
 constexpr int kMaxStages = 16;
 constexpr int kSmemLimit = 232448;            // 227 KB opt-in maximum per CTA
@@ -196,8 +206,13 @@ struct Layout {
         misc_off, total;
 };
 
-// Per-query lists: super-tiles whose row maxima may wait for the finisher.
-constexpr int kUmSlots = 2;
+// Per-query lists: super-tiles whose row maxima (up to 16 KB each) may wait for
+// the finisher.  One leaves room for another chunk stage, and is enough where
+// a super-tile takes three or more of them: 10 queries of 125 tokens x 2,948
+// documents on the FP8 store at d = 768 took 467 us with two, and so two
+// stages, 432 before there was a finisher, 381 with one.
+constexpr int kMaxUmSlots = 2;
+__host__ __device__ constexpr int um_slots(int nchunks) { return nchunks >= 3 ? 1 : kMaxUmSlots; }
 // Finished documents waiting for their sum over query tokens, per epilogue warp
 // (shared lists) or the finisher: kFinRows rows of 32 row maxima (one row per document and 32-row
 // block), padded to 33 floats so that lane r reading row r walks distinct
@@ -218,24 +233,24 @@ constexpr int kFinWarpBytes = kFinRows * 33 * 4 + kFinRows * 8;
 // each chunk stage holds the str document rows, then the qrows query rows
 // of the same dimension chunk.
 __host__ __device__ inline Layout make_layout(int stages, int qslots, int nchunks, int rows_alloc, int str, int kind,
-                                              int kacc, int blocks, bool sh, int qrows, int h) {
+                                              int kacc, int blocks, bool sh, int qrows, int h, bool qt) {
     const bool f8 = kind == kE4M3;
     const int twin = kind == kTF32 ? 2 : 1;
     Layout L;
     L.q_off = 0;
     L.qlo_off = qslots * nchunks * rows_alloc * 128;
-    L.stage_off = (twin * L.qlo_off + 1023) & ~1023;
+    L.stage_off = ((qt ? 1 : twin) * L.qlo_off + 1023) & ~1023;
     L.stage_stride = twin * (str + qrows) * 128;
     L.um_off = L.stage_off + stages * L.stage_stride;
     L.um_stride = sh ? 0 : (str / 8) * blocks * 128;  // [unit][32-row block][row] row maxima
-    L.fin_off = L.um_off + kUmSlots * L.um_stride;
+    L.fin_off = L.um_off + um_slots(nchunks) * L.um_stride;
     L.bias_off = (L.fin_off + (sh ? epi_warps(h) : 1) * kFinWarpBytes + 127) & ~127;
     L.sc_off = L.bias_off + 256;
     L.cb_off = L.sc_off + (f8 ? st_ring(str) * str * 4 : 0);  // F8: [st_ring][str] column scales
     L.code_off = L.cb_off + (kind == kPQ ? kPqCbBytes : 0);                        // kPQ: fp16 codebook
     L.st_off = L.code_off + (kind == kPQ ? kCodeRing * str * kPqM : 0);  // kPQ: code-row ring
     L.bar_off = L.st_off + st_ring(str) * static_cast<int>(sizeof(StSlot));
-    const int nbar = 3 * stages + 2 * kacc + 3 * qslots + 3 * st_ring(str) + 2 * kUmSlots + kMmaWarps + 2 * kCodeRing;
+    const int nbar = 3 * stages + 2 * kacc + 3 * qslots + 3 * st_ring(str) + 2 * kMaxUmSlots + 1 + kMmaWarps + 2 * kCodeRing;
     L.misc_off = L.bar_off + nbar * 8;
     L.total = L.misc_off + 16;
     return L;
@@ -389,7 +404,7 @@ struct Maps {
 
 // H: 128-row halves of the query tile (2 for a shared group of 8 queries).
 // STR: rows per super-tile (MMA N at most), 256 or 128.  CTAS: CTAs per SM
-// (1 or 2); the CTA holds KACC = acc_count(STR, CTAS) accumulators of STR
+// (1 or 2); the CTA holds KACC = acc_count(...) accumulators of STR
 // tensor-memory columns; half h of super-tile t is accumulator use H t + h.
 // SH (shared mode): the launch's queries all score one candidate list; a
 // "query" of the pipeline is then a group of up to 4 H queries stacked in
@@ -397,7 +412,8 @@ struct Maps {
 // writes one score per query of the group.
 // F8: rows are E4M3 codes; similarities are scaled by the document row's
 // scale before the max and by the query token's scale before the sum.
-template <int H, int STR, int CTAS, bool SH, int KIND>
+// QT (TF): the query in tensor memory, see kQueryCols.
+template <int H, int STR, int CTAS, bool SH, int KIND, bool QT = false>
 __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
     dense_tc_kernel(const __grid_constant__ Maps maps, const Args a) {
     constexpr bool F8 = KIND == kE4M3;
@@ -405,8 +421,8 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
     constexpr bool PQ = KIND == kPQ;
     constexpr int CE = chunk_elems(KIND);
     constexpr int STAGE_BYTES = STR * 128;
-    constexpr int KACC = acc_count(STR, CTAS);
-    constexpr uint32_t TCOLS = KACC * STR;
+    constexpr int KACC = acc_count(STR, CTAS, QT);
+    constexpr uint32_t TCOLS = KACC * STR + (QT ? kQueryCols : 0);
     constexpr int kEpiWarps = epi_warps(H);
     constexpr int kLoaderWarp = 1 + kMmaWarps;
     constexpr int kEpiWarp = kLoaderWarp + 1;  // the first of them
@@ -424,13 +440,14 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
     const int NCH = a.nchunks;
     const int qslot_bytes = NCH * a.rows_alloc * 128;
     const bool QSTREAM = QS == 0;  // the query rows come with every chunk stage
-    const Layout L = make_layout(S, QS, NCH, a.rows_alloc, STR, KIND, KACC, a.bpc, SH, QSTREAM ? 128 * H : 0, H);
+    const Layout L = make_layout(S, QS, NCH, a.rows_alloc, STR, KIND, KACC, a.bpc, SH, QSTREAM ? 128 * H : 0, H, QT);
+    const int UMS = um_slots(NCH);
     const int SSTRIDE = L.stage_stride;  // bytes between stages (TF: hi, then lo)
 
     uint8_t* q_base = smem + L.q_off;
     uint8_t* qlo_base = smem + L.qlo_off;  // TF: the lo twin of the query region
     uint8_t* stage_base = smem + L.stage_off;
-    uint8_t* um_base = smem + L.um_off;    // per-query lists: [kUmSlots][unit][block][row] row maxima
+    uint8_t* um_base = smem + L.um_off;    // per-query lists: [UMS][unit][block][row] row maxima
     uint8_t* fin_base = smem + L.fin_off;  // finished-document rows
     float* bias = reinterpret_cast<float*>(smem + L.bias_off);  // [8][8]: entry [n][j] 0 for j < n, else -inf
     float* sc = reinterpret_cast<float*>(smem + L.sc_off);      // F8: [kStRing][STR] scale of each column
@@ -446,10 +463,11 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
     uint64_t* qempty = qfull + QS;
     uint64_t* xfull = qempty + QS;          // [kStRing]
     uint64_t* xempty = xfull + kStRing;     // [kStRing]
-    uint64_t* umfull = xempty + kStRing;    // [kUmSlots] row maxima written
-    uint64_t* umempty = umfull + kUmSlots;         // [kUmSlots] row maxima read
-    uint64_t* scfull = umempty + kUmSlots;          // F8: [kStRing] a record slot's column scales landed
-    uint64_t* mdone = scfull + kStRing;
+    uint64_t* umfull = xempty + kStRing;    // [UMS] row maxima written
+    uint64_t* umempty = umfull + kMaxUmSlots;         // [UMS] row maxima read
+    uint64_t* scfull = umempty + kMaxUmSlots;          // F8: [kStRing] a record slot's column scales landed
+    uint64_t* qready = scfull + kStRing;     // QT: the query is in tensor memory
+    uint64_t* mdone = qready + 1;
     uint64_t* conv = mdone + kMmaWarps;   // TF: [S] stage split
     uint64_t* qconv = conv + S;   // TF: [QS] query tile split
     uint64_t* codefull = qconv + QS;            // kPQ: [kCodeRing] code rows landed
@@ -473,18 +491,20 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
         }
         for (int i = 0; i < QS; ++i) {
             mbar_init(&qfull[i], 1);
-            mbar_init(&qempty[i], kMmaWarps);
+            // the MMAs of every MMA warp, or (QT) the copies to tensor memory
+            mbar_init(&qempty[i], QT ? (a.reps * a.bpc < 4 ? a.reps * a.bpc : 4) : kMmaWarps);
         }
         for (int i = 0; i < kStRing; ++i) {
             mbar_init(&xfull[i], 1);
             // loader, MMA, epilogue, finishers, splitters
             mbar_init(&xempty[i], 1 + kMmaWarps + kEpiWarps + fin_warps(SH) + ((TF || PQ) ? kHelpers : 0));
         }
-        for (int i = 0; i < kUmSlots; ++i) {
+        for (int i = 0; i < kMaxUmSlots; ++i) {
             mbar_init(&umfull[i], a.reps * a.bpc < 4 ? a.reps * a.bpc : 4);
             mbar_init(&umempty[i], 1);
         }
         for (int i = 0; i < kStRing; ++i) mbar_init(&scfull[i], 32);  // one cp.async arrival per loader lane
+        mbar_init(qready, (a.reps * a.bpc < 4 ? a.reps * a.bpc : 4) + kMmaWarps);
         for (int i = 0; i < kMmaWarps; ++i) mbar_init(&mdone[i], 1);
         for (int i = 0; i < S; ++i) mbar_init(&conv[i], kHelpers);
         for (int i = 0; i < QS; ++i) mbar_init(&qconv[i], kHelpers);
@@ -579,7 +599,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                     uint8_t* qdst = q_base + slot * qslot_bytes;
                     for (int kc = 0; kc < NCH; ++kc) {
                         uint8_t* cdst = qdst + kc * a.rows_alloc * 128;
-                        for (int rp = 0; rp < a.reps; ++rp)
+                        for (int rp = 0; rp < (QT ? 1 : a.reps); ++rp)
                             tma_load_3d(cdst + rp * a.bpc * 32 * 128, &maps.q, kc * CE, 0, st_q * (SH ? a.group : 1),
                                         &qfull[slot], pol_keep);
                     }
@@ -992,7 +1012,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
             __syncwarp();
             if (lane == 0) mbar_arrive(&xempty[xs]);
             bool ok = true;
-            if (h.q != cur_q) {
+            if (!QT && h.q != cur_q) {
                 const int slot = qi % QS;
                 if (!warp_wait(&qfull[slot], (qi / QS) & 1, abort_flag, a.err, a.budget)) break;
                 split(q_base + slot * qslot_bytes, qlo_base + slot * qslot_bytes, qslot_bytes);
@@ -1044,9 +1064,18 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
             const int xn = __reduce_max_sync(0xffffffffu, x->n);
             if (elect_one()) mbar_arrive(&xempty[xs]);
             if (!QSTREAM && xq != cur_q) {
-                if (cur_q >= 0 && elect_one()) mma_commit(&qempty[qslot]);
-                qslot = qi % QS;
-                if (!warp_wait(TF ? &qconv[qslot] : &qfull[qslot], (qi / QS) & 1, abort_flag, a.err, a.budget)) break;
+                if (QT) {
+                    // this warp's arrival is part of the phase, so that it
+                    // cannot complete before the last one was seen here
+                    if (elect_one()) mbar_arrive(qready);
+                    if (!warp_wait(qready, qi & 1, abort_flag, a.err, a.budget)) break;
+                    tc_fence_after();
+                } else {
+                    if (cur_q >= 0 && elect_one()) mma_commit(&qempty[qslot]);
+                    qslot = qi % QS;
+                    if (!warp_wait(TF ? &qconv[qslot] : &qfull[qslot], (qi / QS) & 1, abort_flag, a.err, a.budget))
+                        break;
+                }
                 ++qi;
                 cur_q = xq;
             }
@@ -1064,11 +1093,16 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                 const uint32_t a_desc =
                     QSTREAM ? desc_sw128(stage_sa + static_cast<uint32_t>(s * SSTRIDE + (STR + hq * 128) * 128))
                             : q_desc + qoff;
+                const uint32_t q_tmem = tbase + static_cast<uint32_t>(KACC * STR + kc * 64);  // QT: hi, then lo
                 if (elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
                         const uint32_t accumulate = (kc > 0 || kk > 0) ? 1u : 0u;
-                        if (TF) {  // hi.hi + hi.lo + lo.hi
+                        if (QT) {  // the three products below, A in tensor memory
+                            mma_tf32_ta(d_tmem, q_tmem + 8 * kk, b_desc + 2 * kk, idesc, accumulate);
+                            mma_tf32_ta(d_tmem, q_tmem + 8 * kk, blo_desc + 2 * kk, idesc, 1u);
+                            mma_tf32_ta(d_tmem, q_tmem + 32 + 8 * kk, b_desc + 2 * kk, idesc, 1u);
+                        } else if (TF) {  // hi.hi + hi.lo + lo.hi
                             mma_tf32(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
                             mma_tf32(d_tmem, a_desc + 2 * kk, blo_desc + 2 * kk, idesc, 1u);
                             mma_tf32(d_tmem, qlo_desc + qoff + 2 * kk, b_desc + 2 * kk, idesc, 1u);
@@ -1235,8 +1269,8 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                                      ? __ldg(a.q_scales + static_cast<int64_t>(xh.q) * a.nq + b * 32 + lane)
                                      : 0.f;
                 }
-                const int us = t % kUmSlots;
-                if (!warp_wait(&umfull[us], (t / kUmSlots) & 1, abort_flag, a.err, a.budget)) break;
+                const int us = t % UMS;
+                if (!warp_wait(&umfull[us], (t / UMS) & 1, abort_flag, a.err, a.budget)) break;
                 const float* um = reinterpret_cast<const float*>(um_base + us * L.um_stride) + lane;
                 uint32_t todo = xh.values;
                 int e = 0;  // documents ended so far in this super-tile
@@ -1309,6 +1343,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                 return x;
             };
             int qsc_q = -1;
+            int qi = 0, cur_q = -1;  // QT
             for (int t = 0;; ++t) {
                 const int xs = t % kStRing;
                 if (!warp_wait(&xfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
@@ -1321,7 +1356,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                 }
                 const int units = xh.rows >> 3;
                 const int u1 = min(units, ua + share);
-                const int us = t % kUmSlots;
+                const int us = t % UMS;
                 float* um_out = reinterpret_cast<float*>(um_base + us * L.um_stride) + blk * 32 + row;
                 const float* scol = sc + xs * STR;  // F8: scale of each column's document row
                 const int use = H * t + hh;
@@ -1334,7 +1369,44 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                               ? __ldg(a.q_scales + static_cast<int64_t>(qq) * a.nq + row)
                               : 0.f;
                 }
-                if (!SH && !warp_wait(&umempty[us], ((t / kUmSlots) & 1) ^ 1, abort_flag, a.err, a.budget)) break;
+                if (QT && xh.q != cur_q) {
+                    // The new query's rows of this warp's block, split, from
+                    // the swizzled tile to its lanes.  The MMAs on the old
+                    // ones are done: this warp has seen all their commits.
+                    const int slot = qi % QS;
+                    if (!warp_wait(&qfull[slot], (qi / QS) & 1, abort_flag, a.err, a.budget)) break;
+                    const int r = 32 * blk + lane;
+#pragma unroll 1
+                    for (int half = 0; half < 2 * NCH; ++half) {  // 16 elements
+                        const uint4* src = reinterpret_cast<const uint4*>(
+                            q_base + slot * qslot_bytes + ((half >> 1) * a.rows_alloc + r) * 128);
+                        const uint32_t qaddr = tbase + (static_cast<uint32_t>(qd * 32) << 16) +
+                                               static_cast<uint32_t>(KACC * STR + (half >> 1) * 64 + (half & 1) * 16);
+                        uint32_t w[16];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const uint4 x = src[(4 * (half & 1) + i) ^ (r & 7)];
+                            w[4 * i] = x.x, w[4 * i + 1] = x.y, w[4 * i + 2] = x.z, w[4 * i + 3] = x.w;
+                        }
+                        tmem_st16(qaddr, w);  // the MMA reads x as hi
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            const float x = __uint_as_float(w[i]);
+                            w[i] = __float_as_uint(x - tf32_trunc(x));
+                        }
+                        tmem_st16(qaddr + 32, w);
+                    }
+                    tmem_st_wait();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive(&qempty[slot]);
+                        mbar_arrive(qready);
+                    }
+                    ++qi;
+                    cur_q = xh.q;
+                }
+                if (!SH && !warp_wait(&umempty[us], ((t / UMS) & 1) ^ 1, abort_flag, a.err, a.budget)) break;
                 if (F8 && !warp_wait(&scfull[xs], (t / kStRing) & 1, abort_flag, a.err, a.budget)) break;
                 if (!warp_wait(&tfull[ab], (use / KACC) & 1, abort_flag, a.err, a.budget)) break;
                 tc_fence_after();
@@ -1535,6 +1607,12 @@ struct Plan {
     }
 };
 
+// Whether a launch keeps its query in tensor memory (see kQueryCols).
+template <int KIND>
+inline bool query_in_tmem(const Args& a) {
+    return KIND == kTF32 && a.nchunks <= kQueryChunks;
+}
+
 // The configuration a launch of this instantiation takes: `force` if it
 // fits (else TMS_ERR_UNSUPPORTED), else the autotuner's for this shape if
 // one fits, else the default below.
@@ -1548,6 +1626,11 @@ tms_status plan_tc(const DeviceInfo& dev, const Args& a, const Config* force, Pl
     // the query-slot count (2, else 1) that gives the most stages; the
     // plan fits with at least 4 chunk stages (2 with one CTA per SM).
     const int max_reps = SH ? 1 : (a.bpc == 3 ? 1 : 4 / a.bpc);
+    const bool qt = query_in_tmem<KIND>(a);
+    // Which shapes take split TF32 is a rule of its own, not what happens to
+    // fit: the exact fp32 kernel takes the others, and the two differ in the
+    // last bits.
+    if (TF && (a.bpc * a.nchunks > 18 || a.nchunks > 17)) return TMS_ERR_UNSUPPORTED;
     auto fits = [&](int str, int ctas, int rp, int need, int& stages, int& qslots, int cap = 0, int want_qs = 0,
                     bool stream = false) {
         if (rp < 1 || rp > max_reps) return false;
@@ -1558,8 +1641,8 @@ tms_status plan_tc(const DeviceInfo& dev, const Args& a, const Config* force, Pl
         int best = -1;
         for (int qs = stream ? 0 : 2; qs >= (stream ? 0 : 1); --qs) {
             if (!stream && want_qs && qs != want_qs) continue;
-            const Layout L0 = make_layout(0, qs, a.nchunks, 32 * a.bpc * rp, str, KIND, acc_count(str, ctas),
-                                          a.bpc, SH, stream ? 128 * H : 0, H);
+            const Layout L0 = make_layout(0, qs, a.nchunks, 32 * a.bpc * (qt ? 1 : rp), str, KIND,
+                                          acc_count(str, ctas, qt), a.bpc, SH, stream ? 128 * H : 0, H, qt);
             int sts = std::min(kMaxStages, (limit - L0.total) / (L0.stage_stride + 24));
             if (cap > 0 && sts > cap) sts = cap;
             if (sts > best) {
@@ -1685,7 +1768,8 @@ tms_status launch_tc(const DeviceInfo& dev, const void* queries, tms_dtype dtype
                         CE, static_cast<uint32_t>(SH ? 32 : 32 * a.bpc), static_cast<uint32_t>(SH ? a.bpc : 1));
     if (st != TMS_OK) return st;
     a.reps = reps;
-    a.rows_alloc = 32 * a.bpc * reps;
+    const bool qt = query_in_tmem<KIND>(a);
+    a.rows_alloc = 32 * a.bpc * (qt ? 1 : reps);
     for (int h = 0; h < kBoxKinds; ++h) {
         if (PQ) {  // rows are decompressed in shared memory, never loaded by TMA
             maps.doc[h] = maps.q;
@@ -1698,8 +1782,8 @@ tms_status launch_tc(const DeviceInfo& dev, const void* queries, tms_dtype dtype
     a.idesc = make_idesc(128, 0, TF ? 2u : ((!F8 && dtype == TMS_BF16) ? 1u : 0u));
     a.stages = stages;
     a.qslots = qslots;
-    const Layout L = make_layout(stages, qslots, a.nchunks, a.rows_alloc, str, KIND, acc_count(str, ctas),
-                                 a.bpc, SH, qslots == 0 ? 128 * H : 0, H);
+    const Layout L = make_layout(stages, qslots, a.nchunks, a.rows_alloc, str, KIND, acc_count(str, ctas, qt), a.bpc, SH,
+                                 qslots == 0 ? 128 * H : 0, H, qt);
     const int smem = L.total + 1024;
     void (*kern)(const Maps, const Args);
     if constexpr (H == 2 && !PQ) {
@@ -1709,7 +1793,7 @@ tms_status launch_tc(const DeviceInfo& dev, const void* queries, tms_dtype dtype
     } else if constexpr (PQ) {
         kern = dense_tc_kernel<1, 256, 1, true, kPQ>;  // H == 2 took the first branch
     } else if constexpr (TF) {
-        kern = dense_tc_kernel<1, 128, 1, false, kTF32>;
+        kern = qt ? dense_tc_kernel<1, 128, 1, false, kTF32, true> : dense_tc_kernel<1, 128, 1, false, kTF32>;
     } else {
         kern = str == 256 ? dense_tc_kernel<1, 256, 1, SH, KIND>
                           : (ctas == 2 ? dense_tc_kernel<1, 128, 2, SH, KIND> : dense_tc_kernel<1, 128, 1, SH, KIND>);
