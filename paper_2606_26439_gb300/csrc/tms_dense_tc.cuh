@@ -1654,9 +1654,9 @@ tms_status plan_tc(const DeviceInfo& dev, const Args& a, const Config* force, Pl
         return best >= std::max(need, ctas == 2 ? 4 : 2);
     };
     // default: as many copies as fit with 4 stages, else (one CTA) with 2
-    auto plan = [&](int str, int ctas, int& stages, int& qslots, int& reps) {
+    auto plan = [&](int str, int ctas, int& stages, int& qslots, int& reps, int most = 4) {
         for (int need = 4; need >= (ctas == 2 ? 4 : 2); need -= 2)
-            for (int rp = max_reps; rp >= 1; rp /= 2)
+            for (int rp = std::min(max_reps, most); rp >= 1; rp /= 2)
                 if (fits(str, ctas, rp, need, stages, qslots)) {
                     reps = rp;
                     return true;
@@ -1683,15 +1683,33 @@ tms_status plan_tc(const DeviceInfo& dev, const Args& a, const Config* force, Pl
     if (ctas == 0) {
         if (PQ && H == 1) {
             if (plan(256, 1, stages, qslots, reps)) str = 256, ctas = 1;
-        } else if (H == 2 && !PQ && fits(256, 1, 1, 3, stages, qslots)) {
+        } else if (H == 2 && !PQ && a.nchunks <= 2 && fits(256, 1, 1, 3, stages, qslots)) {
             str = 256, ctas = 1, reps = 1;
+        } else if (H == 2 && !PQ && a.nchunks >= 5) {
+            // streamed, below: what the resident tile of eight queries leaves
+            // is two or three 128-row stages (61 queries x 12,000 documents,
+            // fp16, d = 320: 1,192 us resident, 1,117 streamed; 16 queries,
+            // FP8, d = 640: 348 and 316)
         } else if (H == 2 || TF) {
+            // eight queries of three or four chunks: 128-row super-tiles,
+            // four accumulators and four stages or more (as above, fp16, d =
+            // 192: 731 us against 772 with 256 rows and three stages; FP8, d
+            // = 384: 203 and 229)
             if (plan(128, 1, stages, qslots, reps)) str = 128, ctas = 1;
-        } else if (!SH && a.nchunks == 1) {
-            // 128-byte rows (FP8 at d <= 128, fp16 / bf16 at d <= 64): a
-            // super-tile carries few bytes for its fixed pipeline costs, so
-            // two CTAs per SM run two pipelines side by side
-            if (plan(128, 2, stages, qslots, reps)) str = 128, ctas = 2;
+        } else if (SH ? a.nchunks <= 2 : (a.nchunks == 1 || (a.nchunks == 2 && a.bpc >= 2))) {
+            // Short rows (one chunk: FP8 at d <= 128, fp16 / bf16 at d <= 64;
+            // two where each warp has all of a super-tile's columns or half
+            // of them): a super-tile carries few bytes for its fixed pipeline
+            // costs, so two CTAs per SM run two pipelines side by side.
+            // Over 20,000 documents of 32..180 tokens, one CTA and two:
+            // shared by 2..4 queries, d = 64, fp16 91 and 69 us, FP8 116 and
+            // 87; d = 128, 94 and 85, 113 and 85.  Lists, 4 x 10,000, 64
+            // query tokens: fp16 d = 64 152 and 121 us, d = 96 156 and 141,
+            // d = 128 157 and 152; but with 32 tokens and d = 128 591 and 595
+            // (8 x 20,000), and shared d = 256 167 and 168.  Two copies are
+            // enough for one chunk of fp16: 359 us at 8 x 20,000, d = 64,
+            // against 383 with four (FP8: 445 against 431).
+            if (plan(128, 2, stages, qslots, reps, !SH && KIND == kF16 && a.nchunks == 1 ? 2 : 4)) str = 128, ctas = 2;
             else if (plan(256, 1, stages, qslots, reps)) str = 256, ctas = 1;
             else if (plan(128, 1, stages, qslots, reps)) str = 128, ctas = 1;
         } else {

@@ -74,3 +74,27 @@ def test_shared_rounds_equal_per_query_lists(cuda_lib, n_queries, n_cand):
     lists = tms.score_fp8(qc, qs, tc, ts, o, l, cc, co).view(n_queries, n_cand)
     assert torch.equal(shared.view(torch.int32), lists.view(torch.int32))
     assert tms.device_error() & ~tms.TMS_DEVERR_BAD_ID == 0
+
+
+@pytest.mark.parametrize("n_queries", [2, 4, 7])
+@pytest.mark.parametrize("d", [64, 96, 192, 256, 320, 640])
+def test_shared_row_lengths_equal_per_query_lists(cuda_lib, n_queries, d):
+    """Both sides of each row length at which the super-tile, the CTAs per SM
+    or the query tile (resident, streamed) changes: the same bits as
+    per-query lists, fp16 and FP8."""
+    import torch
+    from paper_2606_26439_gb300 import tms
+    tok, off, ln = _corpus(d, "f16", 500 + d)
+    cand = np.random.default_rng(d).permutation(len(ln)).astype(np.int32)
+    Q = synth.queries(n_queries, 32, d, "f16", 501 + d)
+    q, t, o, l, c, cc, co = gc.to_dev(Q, tok, off, ln, cand, np.tile(cand, n_queries),
+                                      np.arange(n_queries + 1, dtype=np.int64) * len(cand))
+    shared = tms.score_dense_shared(q, t, o, l, c)
+    lists = tms.score_dense(q, t, o, l, cc, co).view(n_queries, -1)
+    assert torch.equal(shared.view(torch.int32), lists.view(torch.int32))
+    qc, qs = tms.quantize_e4m3(q)
+    tc, ts = tms.quantize_e4m3(t)
+    shared = tms.score_fp8_shared(qc, qs, tc, ts, o, l, c)
+    lists = tms.score_fp8(qc, qs, tc, ts, o, l, cc, co).view(n_queries, -1)
+    assert torch.equal(shared.view(torch.int32), lists.view(torch.int32))
+    assert tms.device_error() == 0
