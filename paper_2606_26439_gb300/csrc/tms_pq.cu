@@ -298,6 +298,12 @@ __device__ __forceinline__ void add_f16x2(float& acc0, float& acc1, uint32_t w) 
         : "r"(w));
 }
 
+// Two fp32 rounded to nearest fp16, x in the low half.
+__device__ __forceinline__ uint32_t pack_f16x2(float x, float y) {
+    const __half2 h = __floats2half2_rn(x, y);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+
 // 16-byte shared-memory load at shared-window address addr + OFF
 template <int OFF>
 __device__ __forceinline__ uint4 lds128(uint32_t addr) {
@@ -331,7 +337,8 @@ __device__ __forceinline__ void gather_groups(const CodeRow<M>& c, uint32_t tbl,
 }
 
 struct PendingMeta {
-    int64_t li;  // local candidate index (>= n_local: none)
+    int64_t f;  // candidate, -1: none
+    bool done;  // no cells left
     int id;
     int64_t off;
     int len;
@@ -340,6 +347,65 @@ struct PendingMeta {
 // Table bytes of the staged variant: the last block holds 256 rows so that
 // a code >= k still reads inside the allocation.
 __host__ __device__ constexpr int staged_table_bytes(int M) { return ((M / 8 - 1) * (4096 / M) + 256) * 256; }
+
+// One CTA's share of the candidates.  The flat list of all queries' candidates
+// is cut into gridDim.x equal parts; a CTA works on the queries its part
+// meets, so it stages the table of one or two queries and not of every one (at
+// 17 us a chunk then, and 152 CTAs, 16 queries x 50,000 candidates spent 1.1
+// of 6.7 ms on it and 16 x 1,000 with 100 query tokens 3.4 of 4.1 ms).  Within
+// a query, the W CTAs that meet it take its candidates in turn, so that
+// neighbours in the list, often alike in length, are spread over them: cell
+// u = col R + t of a W x R grid is candidate t W + col, and the CTAs take
+// consecutive cells in proportion to their parts (the last row's cells past
+// the list's end are empty).
+struct Share {
+    int64_t c0;    // the query's first candidate
+    int len;       // its candidates
+    int n;         // cells of this CTA; 0: it does not meet the query
+    int w, rows;   // W and R
+    int col0, t0;  // the first cell's column and row
+
+    __device__ __forceinline__ Share(const Args& a, int q) : n(0) {
+        c0 = __ldg(a.cand_offsets + q);
+        int64_t c1 = __ldg(a.cand_offsets + q + 1);
+        c0 = c0 < 0 ? 0 : (c0 > a.n_cand ? a.n_cand : c0);
+        c1 = c1 < c0 ? c0 : (c1 > a.n_cand ? a.n_cand : c1);
+        const int64_t grid = gridDim.x, b = blockIdx.x;
+        const int64_t lo = max(a.n_cand * b / grid, c0), hi = min(a.n_cand * (b + 1) / grid, c1);
+        if (lo >= hi) return;
+        len = static_cast<int>(c1 - c0);
+        w = static_cast<int>((c1 * grid - 1) / a.n_cand - ((c0 + 1) * grid - 1) / a.n_cand) + 1;
+        rows = (len + w - 1) / w;
+        const int64_t cells = static_cast<int64_t>(rows) * w;
+        const int64_t u0 = (lo - c0) * cells / len, u1 = (hi - c0) * cells / len;
+        n = static_cast<int>(u1 - u0);
+        col0 = static_cast<int>(u0 / rows);
+        t0 = static_cast<int>(u0 - static_cast<int64_t>(col0) * rows);
+    }
+    // Candidate of cell li, or -1 (an empty cell).
+    __device__ __forceinline__ int64_t at(int li) const {
+        int64_t t = static_cast<int64_t>(t0) + li;
+        int col = col0;
+        while (t >= rows) {
+            t -= rows;
+            ++col;
+        }
+        const int64_t j = t * w + col;
+        return j < len ? c0 + j : -1;
+    }
+};
+
+// Words (.x .y .z .w: four codes) of four subspaces, rotated by kq.
+__device__ __forceinline__ void rotate4(uint4 (&v)[4], int kq) {
+    if (kq & 1) {
+        const uint4 x = v[0];
+        v[0] = v[1], v[1] = v[2], v[2] = v[3], v[3] = x;
+    }
+    if (kq & 2) {
+        const uint4 x = v[0], y = v[1];
+        v[0] = v[2], v[1] = v[3], v[2] = x, v[3] = y;
+    }
+}
 
 template <int M, bool H16>
 __global__ void __launch_bounds__(kWarps * 32, 1) score_kernel_staged(const Args a, int lut_bytes) {
@@ -389,21 +455,61 @@ __global__ void __launch_bounds__(kWarps * 32, 1) score_kernel_staged(const Args
     uint32_t issued = 0, consumed = 0;  // pieces of this warp (buffer = count & 1)
 
     for (int q = 0; q < a.n_queries; ++q) {
-        int64_t c0 = __ldg(a.cand_offsets + q), c1 = __ldg(a.cand_offsets + q + 1);
-        c0 = c0 < 0 ? 0 : (c0 > a.n_cand ? a.n_cand : c0);
-        c1 = c1 < c0 ? c0 : (c1 > a.n_cand ? a.n_cand : c1);
-        if (c0 + blockIdx.x >= c1) continue;
-        const int64_t n_local = (c1 - c0 - blockIdx.x + gridDim.x - 1) / gridDim.x;
+        const Share share(a, q);
+        const int n_local = share.n;
+        if (n_local == 0) continue;
         for (int ch = 0; ch < nchunks; ++ch) {
             __syncthreads();
-            // Table chunk -> shared memory.  A warp fills 8 rows x one 128-byte
-            // half (slo) per task; lane (ii, ml) reads 8 consecutive codes of
-            // table row (query token, subspace) -- whole sectors -- and each
-            // store instruction writes 32 consecutive words.  Rows of codes >= k
-            // and query tokens >= nq are filled with zeros.
-            {
-                const float* src = a.lut + static_cast<int64_t>(q) * a.nq * M * K;
-                const int ii = lane & 7;
+            // Table chunk -> shared memory, zeros for codes >= k and query
+            // tokens >= nq.  A warp fills 16 rows x one 128-byte half (slo) per
+            // task: lane (ii, kq) loads four codes from 4 kq on of each of the
+            // half's four subspaces of query token ii -- 64 bytes of eight
+            // table rows per instruction -- and stores them in an order that
+            // kq rotates over the subspaces, so that a store's 32 words fall
+            // in 32 banks.  A 128 KB chunk took 17 us with scalar loads of 32
+            // rows each (32,768 lines looked up in L1, one a cycle) and takes
+            // 5.3 with these (2,048): 3.7 TB/s from L2 over all SMs, whether
+            // two or four tasks of a warp are in flight.
+            const float* src = a.lut + static_cast<int64_t>(q) * a.nq * M * K;
+            const int ii = lane & 7;
+            if ((K & 3) == 0) {
+                constexpr int kTasks = staged_table_bytes(M) / 256 / 16 * 2;
+                const int kq = lane >> 3;
+#pragma unroll 2
+                for (int task = warp; task < kTasks; task += kWarps) {
+                    const int slo = task & 1;
+                    const int rho0 = (task >> 1) * 16;  // KS is a multiple of 16
+                    const int shi = min(rho0 / KS, M / 8 - 1);
+                    const int kk = rho0 - shi * KS + 4 * kq;
+                    const int mb = 4 * (2 * shi + slo);
+                    uint4 v[4];
+#pragma unroll
+                    for (int ml = 0; ml < 4; ++ml) {
+                        auto load = [&](int qi) {
+                            return qi < a.nq && kk < K
+                                       ? __ldg(reinterpret_cast<const float4*>(
+                                             src + (static_cast<int64_t>(qi) * M + mb + ml) * K + kk))
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+                        };
+                        if constexpr (H16) {  // query tokens 2 ii and 2 ii + 1, rounded to nearest fp16
+                            const float4 x = load(ch * QC + 2 * ii), y = load(ch * QC + 2 * ii + 1);
+                            v[ml] = make_uint4(pack_f16x2(x.x, y.x), pack_f16x2(x.y, y.y), pack_f16x2(x.z, y.z),
+                                               pack_f16x2(x.w, y.w));
+                        } else {
+                            const float4 x = load(ch * QC + ii);
+                            v[ml] = make_uint4(__float_as_uint(x.x), __float_as_uint(x.y), __float_as_uint(x.z),
+                                               __float_as_uint(x.w));
+                        }
+                    }
+                    rotate4(v, kq);
+                    uint32_t* dst = reinterpret_cast<uint32_t*>(lut_s) + (rho0 + 4 * kq) * 64 + slo * 32 + ii;
+#pragma unroll
+                    for (int st = 0; st < 4; ++st) {
+                        uint32_t* d = dst + ((st + kq) & 3) * 8;
+                        d[0] = v[st].x, d[64] = v[st].y, d[128] = v[st].z, d[192] = v[st].w;
+                    }
+                }
+            } else {  // rows of any alignment: a lane reads 8 consecutive codes of one
                 const int ml = lane >> 3;
                 const int tasks = (lut_bytes / 256 / 8) * 2;
                 for (int task = warp; task < tasks; task += kWarps) {
@@ -441,20 +547,20 @@ __global__ void __launch_bounds__(kWarps * 32, 1) score_kernel_staged(const Args
             if (threadIdx.x == 0) next_local = 0;
             __syncthreads();
 
-            auto grab = [&]() -> int64_t {
+            auto grab = [&]() -> int {
                 int li = 0;
                 if (lane == 0) li = atomicAdd(&next_local, 1);
                 return __shfl_sync(0xffffffffu, li, 0);
             };
-            auto fetch = [&](int64_t li) {  // issue the metadata loads of candidate li
+            auto fetch = [&](int li) {  // issue the metadata loads of cell li's candidate
                 PendingMeta m;
-                m.li = li;
+                m.done = li >= n_local;
+                m.f = m.done ? -1 : share.at(li);
                 m.id = -1;
                 m.off = 0;
                 m.len = 0;
-                if (li < n_local) {
-                    const int64_t f = c0 + blockIdx.x + li * gridDim.x;
-                    m.id = __ldg(a.cand_ids + f);
+                if (m.f >= 0) {
+                    m.id = __ldg(a.cand_ids + m.f);
                     if (m.id >= 0 && m.id < a.n_docs) {
                         m.off = __ldg(a.offsets + m.id);
                         m.len = __ldg(a.lengths + m.id);
@@ -467,13 +573,14 @@ __global__ void __launch_bounds__(kWarps * 32, 1) score_kernel_staged(const Args
             PendingMeta pend = fetch(grab());
             auto take = [&](int64_t& f, int64_t& off, int& len) {
                 for (;;) {
-                    if (pend.li >= n_local) {
+                    if (pend.done) {
                         f = -1;
                         return;
                     }
                     const PendingMeta cur = pend;
                     pend = fetch(grab());
-                    f = c0 + blockIdx.x + cur.li * gridDim.x;
+                    f = cur.f;
+                    if (f < 0) continue;
                     int status = 0;
                     if (cur.id < 0 || cur.id >= a.n_docs)
                         status = 1;

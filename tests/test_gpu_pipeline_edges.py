@@ -98,3 +98,36 @@ def test_shared_row_lengths_equal_per_query_lists(cuda_lib, n_queries, d):
     lists = tms.score_fp8(qc, qs, tc, ts, o, l, cc, co).view(n_queries, -1)
     assert torch.equal(shared.view(torch.int32), lists.view(torch.int32))
     assert tms.device_error() == 0
+
+
+@pytest.mark.parametrize("M,K", [(16, 256), (16, 255), (16, 252), (16, 3), (32, 128), (32, 126), (32, 20)])
+@pytest.mark.parametrize("lists", [(1,), (0, 1, 0, 2), (700, 1, 0, 3, 150, 151, 152, 153), (5, 1500), (1,) * 200],
+                         ids=["one", "few", "uneven", "two", "many"])
+@pytest.mark.parametrize("f16", [False, True])
+def test_pq_shares_and_table_rows_exact(cuda_lib, M, K, lists, f16):
+    """Lists of every size cut over the CTAs, tables whose rows are and are
+    not 16-byte aligned: an integer-valued table (exact in fp16 and in every
+    partial sum) must give the exact scores, every candidate written once."""
+    import torch
+    from paper_2606_26439_gb300 import tms
+    g = np.random.default_rng(M + K + len(lists))
+    nq, nd = 19, 60
+    T = g.integers(-1000, 1001, size=(len(lists), nq, M, K)).astype(np.float32)
+    ln = g.integers(0, 40, nd).astype(np.int32)
+    off = np.concatenate([[0], np.cumsum(ln)[:-1]]).astype(np.int64)
+    codes = g.integers(0, K, size=(int(ln.sum()), M)).astype(np.uint8)
+    cands = [g.integers(0, nd, n).astype(np.int32) for n in lists]
+    flat, co = gc.csr(cands)
+    t_d, c_d, o_d, l_d, f_d, co_d = gc.to_dev(T, codes, off, ln, flat, co)
+    out = torch.full((len(flat),), 12345.5, dtype=torch.float32, device="cuda")
+    tms.score_pq(t_d, c_d, o_d, l_d, f_d, co_d, out=out, f16_table=f16)
+    got = out.cpu().numpy()
+    assert tms.device_error() == 0
+    for q, c in enumerate(cands):
+        per_doc = np.full(nd, -np.inf)
+        for x in set(c.tolist()):
+            if ln[x]:
+                rows = codes[off[x]:off[x] + ln[x]].astype(int)
+                dots = T[q][:, np.arange(M), rows].sum(-1)  # (nq, tokens)
+                per_doc[x] = dots.max(1).sum()
+        assert np.array_equal(got[co[q]:co[q + 1]], per_doc[c].astype(np.float32))
