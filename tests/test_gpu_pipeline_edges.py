@@ -131,3 +131,38 @@ def test_pq_shares_and_table_rows_exact(cuda_lib, M, K, lists, f16):
                 dots = T[q][:, np.arange(M), rows].sum(-1)  # (nq, tokens)
                 per_doc[x] = dots.max(1).sum()
         assert np.array_equal(got[co[q]:co[q + 1]], per_doc[c].astype(np.float32))
+
+
+@pytest.mark.parametrize("dtype", ["f16", "f32", "fp8"])
+@pytest.mark.parametrize("lists", [(0, 0, 5), (1,) * 70, (0, 1, 0, 2, 0), (400, 1, 0, 3, 150, 151, 152, 153, 304),
+                                   (2,) * 1100, (1, 3000, 1)], ids=["last", "ones", "few", "uneven", "many", "long"])
+def test_lists_cut_over_ctas(cuda_lib, dtype, lists):
+    """Lists of every size, empty ones between, cut over the CTAs: each
+    candidate is written once, with the bits that its query and document give
+    in a list of all documents."""
+    import torch
+    from paper_2606_26439_gb300 import tms
+    tok, off, ln = _corpus(64, "f32" if dtype == "f32" else "f16", 88)
+    g = np.random.default_rng(len(lists))
+    Q = synth.queries(len(lists), 9, 64, "f32" if dtype == "f32" else "f16", 89)
+    cands = [g.integers(0, len(ln), n).astype(np.int32) for n in lists]
+    flat, co = gc.csr(cands)
+    every = np.arange(len(ln), dtype=np.int32)
+    q, t, o, l, f, c, e = gc.to_dev(Q, tok, off, ln, flat, co, every)
+    out = torch.full((len(flat),), 12345.0, dtype=torch.float32, device="cuda")
+    if dtype == "fp8":
+        qc, qs = tms.quantize_e4m3(q)
+        tc, ts = tms.quantize_e4m3(t)
+        tms.score_fp8(qc, qs, tc, ts, o, l, f, c, out=out)
+        full = tms.score_fp8_shared(qc, qs, tc, ts, o, l, e)
+    else:
+        tms.score_dense(q, t, o, l, f, c, out=out)
+        if dtype == "f32":  # no shared lists: one call for each query
+            whole = torch.tensor([0, len(ln)], dtype=torch.int64, device="cuda")
+            full = torch.stack([tms.score_dense(q[i:i + 1], t, o, l, e, whole) for i in range(len(lists))])
+        else:
+            full = tms.score_dense_shared(q, t, o, l, e)
+    got, full = out.cpu().numpy(), full.cpu().numpy()
+    assert tms.device_error() == 0
+    want = np.concatenate([full[i][x] for i, x in enumerate(cands)])
+    assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
