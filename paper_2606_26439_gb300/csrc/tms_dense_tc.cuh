@@ -35,25 +35,27 @@
 //     by parallel lanes (128-byte swizzle).  Each token is read from HBM
 //     once (Theorem 1 with BQ = Nq, or the whole group of queries in the
 //     shared schedule).
-//   * TF only -- four splitter warps: split every landed chunk stage (hi in
-//     place, lo beside it) and every new query tile before the MMA reads
-//     them.
-//   * MMA warp: one thread issues tcgen05.mma (M = 128 query rows, K = 32
-//     bytes: 16 fp16/bf16 elements with kind::f16, 32 E4M3 elements with
-//     kind::f8f6f4, 8 TF32 elements -- three products -- with kind::tf32)
-//     over every dimension chunk of a super-tile,
-//     accumulating the partial dot products in tensor memory before any
-//     max is taken -- the paper's dimension tiling (Section 3), with the K
-//     loop running through TMEM.
-//   * Epilogue warps: thread = query row (TMEM lane).  Each warp takes its
-//     share of a super-tile's columns with tcgen05.ld, multiplies column j
-//     by document row j's scale (F8), and reduces them to a running max
-//     that starts again after each document's end; the values at documents'
-//     ends and at the end of its share go to shared memory.
-//   * Finisher warps: combine those values into each document's row maxima
-//     and sum them over the query tokens (times their scales, F8).  Each
-//     score is written once; the Nq x Nd similarity matrix never reaches
-//     HBM and no atomics or memset are needed.
+//   * TF only -- eight splitter warps: split every landed chunk stage (hi in
+//     place, lo beside it) before the MMA reads it, and every new query tile
+//     that does not lie in tensor memory (see kQueryCols).
+//   * Two MMA warps, super-tiles in turn: an elected lane issues tcgen05.mma
+//     (M = 128 query rows, K = 32 bytes: 16 fp16/bf16 elements with
+//     kind::f16, 32 E4M3 elements with kind::f8f6f4, 8 TF32 elements --
+//     three products -- with kind::tf32) over every dimension chunk of a
+//     super-tile, accumulating the partial dot products in tensor memory
+//     before any max is taken -- the paper's dimension tiling (Section 3),
+//     with the K loop running through TMEM.
+//   * Epilogue warps (four for each 128-row half): thread = query row (TMEM
+//     lane).  Each warp takes its columns of a super-tile with tcgen05.ld,
+//     multiplies column j by document row j's scale (F8), and reduces them to
+//     a running max that starts again after each document's end.
+//   * Shared lists: a warp sees all columns of its query and sums each
+//     document's row maxima over the query tokens (times their scales, F8)
+//     itself.  Per-query lists: the copies share the columns and leave their
+//     values at documents' ends, and at the end of their share, in shared
+//     memory; a finisher warp combines and sums them.  Each score is written
+//     once; the Nq x Nd similarity matrix never reaches HBM and no atomics or
+//     memset are needed.
 //
 // Every wait is bounded (see tms_common.cuh); a timeout sets
 // TMS_DEVERR_TIMEOUT and the CTA drains its in-flight copies and MMAs,
@@ -1649,14 +1651,13 @@ inline int config_shapes(Config* out) {
 
 // Plan shared memory, encode the tensor maps and launch dense_tc_kernel.
 // Without a tuned or forced configuration: one CTA per SM with 256-row
-// super-tiles (about two documents per MMA run) by default; per-query lists
-// on the FP8 store prefer two CTAs per SM with 128-row super-tiles (two of
-// every pipeline role per SM; measured faster for its 128-byte rows, slower
-// for fp16/bf16); a shared group of 8 (H = 2) and split TF32 (fp32 rows,
-// stages twice the size) take one CTA with 128-row super-tiles.  KIND
-// selects the row type; kE4M3 ignores `dtype` (rows are E4M3 codes;
-// t_scales in `a`).  The caller sets a.nchunks = ceil(d / chunk_elems(KIND)),
-// and a.bpc: per-query ceil(nq / 32), shared mode the group size.  `force` (the autotuner's) overrides the choice;
+// super-tiles (about two documents per MMA run); two CTAs with 128-row ones
+// for short rows; one CTA with 128-row ones for eight queries of three or four
+// chunks, split TF32 and what leaves no room for more (plan_tc has the lines
+// and the figures).  KIND selects the row type; kE4M3 ignores `dtype` (rows
+// are E4M3 codes; t_scales in `a`).  The caller sets a.nchunks =
+// ceil(d / chunk_elems(KIND)), and a.bpc: per-query ceil(nq / 32), shared mode
+// the group size.  `force` (the autotuner's) overrides the choice;
 // TMS_ERR_UNSUPPORTED when it does not fit.
 // The resolved launch configuration: every field of Config set (qslots 0:
 // the query is streamed).
