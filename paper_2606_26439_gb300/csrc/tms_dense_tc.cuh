@@ -141,7 +141,7 @@ struct SegInfo {
     uint16_t rows;  // rows that count (8 nu but for a partial last unit)
 };
 
-// One super-tile record (planner -> loader, MMA thread and epilogue).
+// One super-tile record (planner -> loader, MMA warps and epilogue).
 struct StHdr {
     int q;            // query (group) whose tile it is scored against
     int n;            // MMA N: packed rows rounded up to 16
@@ -185,7 +185,7 @@ struct Args {
     int stages;      // chunk stages in the ring
     int qslots;      // resident query-tile slots; 0: the query is streamed with each chunk stage
     int bpc;         // 32-row query blocks per copy: ceil(nq / 32) token blocks, or the group's queries
-    int reps;        // copies of the blocks stacked in M (1, 2 or 4); documents are dealt round-robin to them
+    int reps;        // copies of the blocks stacked in M (1, 2 or 4); they share a super-tile's columns
     int rows_alloc;  // query rows held per dimension chunk: 32 * bpc * reps
     uint32_t idesc;  // instruction descriptor, N field left 0 (set per super-tile)
     const uint8_t* pq_codes;    // kPQ: [n_tokens][16] uint8
@@ -198,7 +198,7 @@ struct Args {
 // Stands in for the row scale of a column past its document's end.
 static __device__ const float kNanScale = __builtin_nanf("");
 
-// Diagnostics (tms_debug_set): the MMA thread of CTA 0 never signals its
+// Diagnostics (tms_debug_set): the MMA warp of CTA 0 never signals its
 // first accumulator, so that CTA's epilogue wait runs out of budget and the
 // timeout path -- flag, abort, drain, tensor-memory release -- runs.
 constexpr int kFaultHoldAccumulator = TMS_FAULT_HOLD_ACCUMULATOR;
@@ -658,8 +658,8 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
             used = nseg = nfin = 0;
             ends = partial = 0;
             // A new query's rows go to the next query slot.  The record is
-            // published first: the MMA thread releases the old slot only
-            // once it sees the new query.
+            // published first: the MMA warps release the old slot only
+            // once they see the new query.
             if (!QSTREAM && st_q != cur_q) {
                 const int slot = qi % QS;
                 if (!warp_wait(&qempty[slot], ((qi / QS) & 1) ^ 1, abort_flag, a.err, a.budget)) return false;
@@ -1041,7 +1041,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
         // Split each new query tile and every landed chunk stage: the MMA
         // reads an fp32 element as hi = tf32_trunc(x), so x stays in place
         // as its own hi part and lo = x - hi (exact, |lo| < 2^-10 |x|) goes
-        // to the twin region; then publish the split to the MMA thread.
+        // to the twin region; then publish the split to the MMA warps.
         // Elements are independent, so the 128-byte swizzle needs no
         // decoding: x and lo keep the same byte positions.
         const int tid = (warp - kHelpWarp) * 32 + lane;
