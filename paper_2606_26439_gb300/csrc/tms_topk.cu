@@ -24,8 +24,10 @@
 // block barriers instead of some thirty: the kernels are bound by those and
 // by launch and load latency, not by bytes (top-10 of one list of 1,000 /
 // 10,000 scores: 7.8 / 13.6 -> 3.3 / 5.7 us; top-100 of 16 x 20,000: 29.4 ->
-// 9.6 us; back to back in a graph).  A list with more than kCand keys at or
-// above the bound (many equal scores) takes the radix path.
+// 9.6 us; back to back in a graph).  More than kCand keys at or above the
+// bound are equal keys, most often, and then the bound is the k-th largest
+// (take_tied); only a list with k or more keys above such a bound takes the
+// radix path.
 //
 // tms_topk: one CTA per query selects from the whole list.
 // tms_topk_split: S CTAs per query each select the top-k of one contiguous
@@ -302,8 +304,53 @@ __device__ int select_sorted(int n, int k, KeyAt key_at, PosAt pos_at, Smem& sm)
     return cnt;
 }
 
+// select_fast where more keys than the survivor buffer holds are at or above
+// its bound: the keys above it and, if those are fewer than k -- so that the
+// bound is the k-th largest key itself -- its lowest positions up to k go to
+// sm.fast.cand.  Returns k, or -1 (for the whole CTA) if k or more keys exceed
+// the bound.  Out of line, so that the usual path stays as short as it was.
+// 10,000 equal scores, top-10: 9.3 us, and 22.8 when they went on to the radix
+// passes (which alone took 19.1).
+template <class KeyAt, class PosAt>
+__device__ __noinline__ int take_tied(int n, int k, uint32_t bound, KeyAt key_at, PosAt pos_at, Smem& sm) {
+    __syncthreads();  // sm.count is read by all before it is reset
+    sm.fast.cand[threadIdx.x] = 0ull;
+    if (threadIdx.x == 0) sm.count = 0;
+    __syncthreads();
+    for (int base = 0; base < n; base += kAhead * kThreads) {
+        uint32_t keys[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int i = base + u * kThreads + threadIdx.x;
+            keys[u] = i < n ? key_at(i) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int i = base + u * kThreads + threadIdx.x;
+            if (i < n && keys[u] > bound) {
+                const int slot = atomicAdd(&sm.count, 1);
+                if (slot < kCand) sm.fast.cand[slot] = pack(keys[u], pos_at(i));
+            }
+        }
+    }
+    __syncthreads();
+    int c = sm.count;
+    __syncthreads();  // as above, for the radix path
+    if (c >= k) return -1;
+    for (int base = 0; base < n && c < k; base += kThreads) {
+        const int i = base + threadIdx.x;
+        const bool tied = i < n && key_at(i) == bound;
+        int total;
+        const int slot = c + block_exclusive_scan(tied ? 1 : 0, sm.scan_buf, &total);
+        if (tied && slot < k) sm.fast.cand[slot] = pack(bound, pos_at(i));
+        c += total;
+    }
+    __syncthreads();
+    return k;
+}
+
 // The select step for k <= kFastK: same arguments and result as
-// select_sorted, or -1 (for the whole CTA) if too many keys reach the bound.
+// select_sorted, or -1 (for the whole CTA) if too many keys exceed the bound.
 // A: keys a thread loads together; RES: n <= A * kThreads, so that they stay in
 // registers for both passes.
 template <int A, bool RES, class KeyAt, class PosAt>
@@ -360,10 +407,10 @@ __device__ int select_fast(int n, int k, KeyAt key_at, PosAt pos_at, Smem& sm) {
         }
     }
     __syncthreads();
-    const int c = sm.count;
-    if (c > kCand) {
-        __syncthreads();  // sm.count is read by all before the radix path resets it
-        return -1;
+    int c = sm.count;
+    if (__builtin_expect(c > kCand, 0)) {
+        c = take_tied(n, k, bound, key_at, pos_at, sm);
+        if (c < 0) return -1;
     }
     // A survivor's place: how many are larger.  Entries are distinct, but for
     // the zero padding of a workspace, which ranks below every other and is
