@@ -340,12 +340,13 @@ tms_status tms_topk(const float *scores, const int64_t *cand_offsets, int n_quer
                     float *out_scores, int32_t *out_pos, cudaStream_t stream);
 
 /*
- * tms_topk on the whole GPU: each query's list is cut into S contiguous
- * slices, one CTA selects each slice's top-k into `workspace`, and one CTA
- * per query selects the final top-k from its S x topk entries.  The result
+ * tms_topk on the whole GPU: each query's list is cut into up to S contiguous
+ * slices, by its own length (one, if one CTA is as fast), one CTA selects each
+ * slice's top-k into `workspace`, and one CTA per query selects the final
+ * top-k from its slices' entries.  The result
  * is bit-identical to tms_topk (same order, same ties, same padding); only
- * the work is spread over S times more CTAs, which matters when there are
- * few queries with long lists (e.g. 16 lists of 100,000 scores).
+ * the work is spread over up to S times more CTAs, which matters when there
+ * are few queries with long lists (e.g. 16 lists of 100,000 scores).
  *
  *   n_cand         cand_offsets[n_queries] (HOST value): fixes S with
  *                  n_queries, topk and the device's SM count.

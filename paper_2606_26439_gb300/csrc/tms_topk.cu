@@ -30,7 +30,7 @@
 // radix path.
 //
 // tms_topk: one CTA per query selects from the whole list.
-// tms_topk_split: S CTAs per query each select the top-k of one contiguous
+// tms_topk_split: up to S CTAs per query each select the top-k of one contiguous
 // slice of the list into the caller's workspace (k sorted entries, padded
 // with key 0), then one CTA per query selects from the S x k entries.  The
 // order (key desc, position asc) is total, so every member of the list's
@@ -53,8 +53,10 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kMaxK = 1024;
 constexpr int kMaxSlices = 64;
 constexpr int kFastK = 256;          // select_fast: r = ceil(k / 16) rounds per warp
+constexpr int kMergeSteps = 6;       // merge_fast: 2 k / n doubled so often is k or more, for any n <= kMaxSlices
 constexpr int kCand = kThreads;      // select_fast: survivors it can rank, one per thread
 constexpr int kFastResident = 20;    // select_fast: keys per thread of a list read once
+constexpr int kSliceLen = 8192;      // list_slices: scores of a slice, at least
 
 __device__ __forceinline__ uint32_t score_key(float x) {
     if (x != x) return 1u;  // NaN: after every number (the smallest number's key is 0x007fffff)
@@ -349,6 +351,52 @@ __device__ __noinline__ int take_tied(int n, int k, uint32_t bound, KeyAt key_at
     return k;
 }
 
+// The last steps of select_fast and merge_fast: the keys at or above `bound`
+// (k or more of them) collected and put in their places.  RES: they lie in
+// `keys` already.
+template <int A, bool RES, class KeyAt, class PosAt>
+__device__ __forceinline__ int take_above(uint32_t bound, uint32_t (&keys)[A], int n, int k, KeyAt key_at,
+                                          PosAt pos_at, Smem& sm) {
+    for (int base = 0; base < n; base += A * kThreads) {
+        if constexpr (!RES) {
+#pragma unroll
+            for (int u = 0; u < A; ++u) {
+                const int i = base + u * kThreads + threadIdx.x;
+                keys[u] = i < n ? key_at(i) : 0u;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < A; ++u) {
+            const int i = base + u * kThreads + threadIdx.x;
+            if (i < n && keys[u] >= bound) {
+                const int slot = atomicAdd(&sm.count, 1);
+                if (slot < kCand) sm.fast.cand[slot] = pack(keys[u], pos_at(i));
+            }
+        }
+    }
+    __syncthreads();
+    int c = sm.count;
+    if (__builtin_expect(c > kCand, 0)) {
+        c = take_tied(n, k, bound, key_at, pos_at, sm);
+        if (c < 0) return -1;
+    }
+    // A survivor's place: how many are larger.  Entries are distinct, but for
+    // the zero padding of a workspace, which ranks below every other and is
+    // in place already.
+    const unsigned long long e = sm.fast.cand[threadIdx.x];
+    if (e != 0ull) {
+        const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(sm.fast.cand);
+        int place = 0;
+        for (int j = 0; j < c; j += 4) {
+            const ulonglong2 x = c2[j >> 1], y = c2[(j >> 1) + 1];
+            place += (x.x > e) + (x.y > e) + (y.x > e) + (y.y > e);
+        }
+        if (place < k) sm.sel[place] = e;
+    }
+    __syncthreads();
+    return min(c, k);
+}
+
 // The select step for k <= kFastK: same arguments and result as
 // select_sorted, or -1 (for the whole CTA) if too many keys exceed the bound.
 // A: keys a thread loads together; RES: n <= A * kThreads, so that they stay in
@@ -389,44 +437,44 @@ __device__ int select_fast(int n, int k, KeyAt key_at, PosAt pos_at, Smem& sm) {
         rank += (y > mine || (y == mine && j < lane)) ? 1 : 0;
     }
     const uint32_t bound = __reduce_max_sync(0xffffffffu, rank == q - 1 ? mine : 0u);
-    for (int base = 0; base < n; base += A * kThreads) {
-        if constexpr (!RES) {
-#pragma unroll
-            for (int u = 0; u < A; ++u) {
-                const int i = base + u * kThreads + threadIdx.x;
-                keys[u] = i < n ? key_at(i) : 0u;
+    return take_above<A, RES>(bound, keys, n, k, key_at, pos_at, sm);
+}
+
+// select_any for the merge: n slices' entries, k sorted ones each, k <= kFastK.
+// If the j-th entries of m = ceil(k / j) slices are v or more, so are k entries
+// at least; warp w finds the largest such v for j = 2 k / n, doubled w times,
+// and the largest of those is the bound -- a close one whether all slices hold
+// their share of the largest (j = 2 k / n) or one of them all (j = k).  The
+// bound of select_fast was not: sorted runs of a length that is a power of two
+// give their first entries to the same few warps, and more entries than can be
+// ranked reached it (k = 128, 2 x 400,000 scores: 27.8 us by it, now 16.8).
+template <class KeyAt, class PosAt>
+__device__ int merge_fast(int n, int k, KeyAt key_at, PosAt pos_at, Smem& sm) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    sm.fast.cand[threadIdx.x] = 0ull;
+    if (static_cast<int>(threadIdx.x) < k) sm.sel[threadIdx.x] = 0ull;
+    if (warp < kMergeSteps) {
+        const int j = min(k, ((2 * k + n - 1) / n) << warp), m = (k + j - 1) / j;
+        uint32_t a = lane < n ? key_at(lane * k + j - 1) : 0u;
+        uint32_t b = lane + 32 < n ? key_at((lane + 32) * k + j - 1) : 0u;
+        uint32_t v = 0;
+        for (int i = 0; i < m; ++i) {  // the m-th largest of a and b over the warp
+            v = __reduce_max_sync(0xffffffffu, max(a, b));
+            const unsigned who = __ballot_sync(0xffffffffu, a == v || b == v);
+            if (lane == __ffs(who) - 1) {
+                if (a == v) a = 0u;
+                else b = 0u;
             }
         }
+        if (lane == 0) sm.fast.bound[warp] = v;
+    }
+    if (threadIdx.x == 0) sm.count = 0;
+    __syncthreads();
+    uint32_t bound = 0;
 #pragma unroll
-        for (int u = 0; u < A; ++u) {
-            const int i = base + u * kThreads + threadIdx.x;
-            if (i < n && keys[u] >= bound) {
-                const int slot = atomicAdd(&sm.count, 1);
-                if (slot < kCand) sm.fast.cand[slot] = pack(keys[u], pos_at(i));
-            }
-        }
-    }
-    __syncthreads();
-    int c = sm.count;
-    if (__builtin_expect(c > kCand, 0)) {
-        c = take_tied(n, k, bound, key_at, pos_at, sm);
-        if (c < 0) return -1;
-    }
-    // A survivor's place: how many are larger.  Entries are distinct, but for
-    // the zero padding of a workspace, which ranks below every other and is
-    // in place already.
-    const unsigned long long e = sm.fast.cand[threadIdx.x];
-    if (e != 0ull) {
-        const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(sm.fast.cand);
-        int place = 0;
-        for (int j = 0; j < c; j += 4) {
-            const ulonglong2 x = c2[j >> 1], y = c2[(j >> 1) + 1];
-            place += (x.x > e) + (x.y > e) + (y.x > e) + (y.y > e);
-        }
-        if (place < k) sm.sel[place] = e;
-    }
-    __syncthreads();
-    return min(c, k);
+    for (int w = 0; w < kMergeSteps; ++w) bound = max(bound, sm.fast.bound[w]);
+    uint32_t keys[kAhead];
+    return take_above<kAhead, false>(bound, keys, n * k, k, key_at, pos_at, sm);
 }
 
 // select_fast where it applies, else (or where it gives up) select_sorted;
@@ -496,29 +544,50 @@ __global__ void __launch_bounds__(kThreads, 1)
     write_out(sm, cnt, k, s, out_scores + static_cast<int64_t>(q) * k, out_pos + static_cast<int64_t>(q) * k);
 }
 
-// Slice `blockIdx.x % S` of query `blockIdx.x / S`: its top-k (sorted,
-// padded with zero entries to k) at ws[(q * S + slice) * k ...].
+// How many of the S slices there is room for a list of `len` scores takes.
+// k <= kFastK: a list that one CTA holds in registers is not cut (one CTA 5.2
+// us for 10,000 scores, slices and a merge 7.9; k = 100, 16 lists of 20,000:
+// 12.9 against 18.0), a longer one into slices of kSliceLen or more.  Larger k
+// (radix passes): all of them.
+__host__ __device__ inline int list_slices(int64_t len, int k, int S) {
+    if (k > kFastK) return S;
+    if (len <= kFastResident * kThreads) return 1;
+    const int64_t n = len / kSliceLen;
+    return static_cast<int>(n < S ? n : S);
+}
+
+// Slice `blockIdx.x / n_queries` of query `blockIdx.x % n_queries`: its top-k
+// (sorted, padded with zero entries to k) at ws[(q * S + slice) * k ...].
+// A list in one slice is finished here; the CTAs of slices that a list does
+// not take have nothing to do, and come last.
 __global__ void __launch_bounds__(kThreads, 1)
-    topk_slice_kernel(const float* __restrict__ scores, const int64_t* __restrict__ cand_offsets, int k, int S,
-                      unsigned long long* __restrict__ ws, unsigned int* err) {
+    topk_slice_kernel(const float* __restrict__ scores, const int64_t* __restrict__ cand_offsets, int n_queries,
+                      int k, int S, unsigned long long* __restrict__ ws, float* __restrict__ out_scores,
+                      int32_t* __restrict__ out_pos, unsigned int* err) {
     __shared__ Smem sm;
     griddep_wait();
     griddep_launch_dependents();
-    const int q = blockIdx.x / S;
-    const int sl = blockIdx.x - q * S;
+    const int sl = blockIdx.x / n_queries;
+    const int q = blockIdx.x - sl * n_queries;
     int64_t c0, c1;
     query_list(cand_offsets, q, sl == 0 ? err : nullptr, &c0, &c1);
     const int64_t len = list_len(c0, c1);
-    const int64_t a = len * sl / S, b = len * (sl + 1) / S;  // slice [a, b) of the list
+    const int n = list_slices(len, k, S);
+    if (sl >= n) return;
+    const int64_t a = len * sl / n, b = len * (sl + 1) / n;  // slice [a, b) of the list
     const float* s = scores + c0 + a;
     const int cnt = select_any(
         static_cast<int>(b - a), k, [&](int i) { return score_key(s[i]); },
         [&](int i) { return static_cast<uint32_t>(a + i); }, sm);
-    unsigned long long* dst = ws + static_cast<int64_t>(blockIdx.x) * k;
+    if (n == 1) {
+        write_out(sm, cnt, k, s, out_scores + static_cast<int64_t>(q) * k, out_pos + static_cast<int64_t>(q) * k);
+        return;
+    }
+    unsigned long long* dst = ws + (static_cast<int64_t>(q) * S + sl) * k;
     for (int r = threadIdx.x; r < k; r += kThreads) dst[r] = r < cnt ? sm.sel[r] : 0ull;
 }
 
-// Query blockIdx.x: the top-k of its S x k slice entries.
+// Query blockIdx.x: the top-k of its slices' entries.
 __global__ void __launch_bounds__(kThreads, 1)
     topk_merge_kernel(const float* __restrict__ scores, const int64_t* __restrict__ cand_offsets, int k, int S,
                       const unsigned long long* __restrict__ ws, float* __restrict__ out_scores,
@@ -529,25 +598,37 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int q = blockIdx.x;
     int64_t c0, c1;
     query_list(cand_offsets, q, nullptr, &c0, &c1);
+    const int n = list_slices(list_len(c0, c1), k, S);
+    if (n == 1) return;
     const unsigned long long* e = ws + static_cast<int64_t>(q) * S * k;
-    const int cnt = select_any(
-        S * k, k, [&](int i) { return key_of(e[i]); }, [&](int i) { return pos_of(e[i]); }, sm);
+    auto key_at = [&](int i) { return key_of(e[i]); };
+    auto pos_at = [&](int i) { return pos_of(e[i]); };
+    int cnt = k <= kFastK ? merge_fast(n, k, key_at, pos_at, sm) : -1;
+    if (cnt < 0) cnt = n * k <= kResident * kThreads ? select_sorted<true>(n * k, k, key_at, pos_at, sm)
+                                                     : select_sorted<false>(n * k, k, key_at, pos_at, sm);
     write_out(sm, cnt, k, scores + c0, out_scores + static_cast<int64_t>(q) * k,
               out_pos + static_cast<int64_t>(q) * k);
 }
 
-// Slices per query of tms_topk_split: about two CTAs per SM in all, at most
-// kMaxSlices.  k <= kFastK: lists that one CTA holds in registers are not cut
-// (one CTA 5.2 us for 10,000 scores, slices and a merge 7.9; k = 100, 16 lists
-// of 20,000: 12.9 against 18.0), longer ones into slices of 8,192 or more;
-// larger k (radix passes): slices of a few thousand scores.
+// Room per query for slices in tms_topk_split: about two CTAs per SM in all,
+// at most kMaxSlices.  The host knows the lists' lengths only in sum, so for
+// several of them (k <= kFastK) it makes room by their average and list_slices
+// settles each list's number on the device: one number for all, by the average,
+// left 31 lists of 600 scores and one of 600,000 with one CTA each, 237 us, now
+// 34.  Room that equal lists of up to 20,480 do not use costs a second launch
+// and CTAs that leave at once (16 x 20,000, k = 100: 9.9 us without, 11.5
+// with).  So there is none for up to three slices, which gain little over one
+// CTA of select_fast (15 x 1,000 and one of 100,000: 42 us; three slices by
+// radix passes took 47), nor where no list can be longer than two CTAs hold.
 int slices(int sm_count, int n_queries, int k, int64_t n_cand) {
     const int64_t avg = n_cand / n_queries;
     const int64_t by_grid = (2 * static_cast<int64_t>(sm_count) + n_queries - 1) / n_queries;
-    const int64_t by_len = k > kFastK ? avg / std::max<int64_t>(2048, 4 * static_cast<int64_t>(k))
-                           : avg <= kFastResident * kThreads ? 1
-                                                             : avg / 8192;
-    return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({static_cast<int64_t>(kMaxSlices), by_grid, by_len})));
+    const int64_t most = std::min<int64_t>(kMaxSlices, by_grid);
+    const int64_t room = std::min(most, avg / std::max<int64_t>(2048, 4 * static_cast<int64_t>(k)));
+    if (k > kFastK) return static_cast<int>(std::max<int64_t>(1, room));
+    if (n_queries == 1) return list_slices(n_cand, k, static_cast<int>(most));
+    if (avg > kFastResident * kThreads) return static_cast<int>(room);
+    return room > 3 && n_cand > 2 * kFastResident * kThreads ? static_cast<int>(room) : 1;
 }
 
 bool args_ok(const float* scores, const int64_t* cand_offsets, int n_queries, int k, const float* out_scores,
@@ -603,7 +684,8 @@ extern "C" tms_status tms_topk_split(const float* scores, const int64_t* cand_of
     if (workspace == nullptr || !aligned16(workspace) || workspace_bytes < need) return TMS_ERR_INVALID_ARG;
     auto* ws = static_cast<unsigned long long*>(workspace);
     st = launch_status(launch_dependent(topk::topk_slice_kernel, dim3(static_cast<unsigned>(n_queries * S)),
-                                        dim3(topk::kThreads), 0, stream, scores, cand_offsets, topk, S, ws, dev.err));
+                                        dim3(topk::kThreads), 0, stream, scores, cand_offsets, n_queries, topk, S, ws,
+                                        out_scores, out_pos, dev.err));
     if (st != TMS_OK) return st;
     return launch_status(launch_dependent(topk::topk_merge_kernel, dim3(static_cast<unsigned>(n_queries)),
                                           dim3(topk::kThreads), 0, stream, scores, cand_offsets, topk, S, ws,
@@ -666,10 +748,11 @@ extern "C" tms_status tms_topk_split_noalloc(const float* scores, const int64_t*
     unsigned long long* ws = nullptr;
     st = topk::noalloc_scratch(dev.ordinal, &ws);
     if (st != TMS_OK) return st;
-    // Every slice writes all k of its entries (padding included), so nothing
-    // from an earlier call is ever read.
+    // Every slice that a list takes writes all k of its entries (padding
+    // included), so nothing from an earlier call is ever read.
     st = launch_status(launch_dependent(topk::topk_slice_kernel, dim3(static_cast<unsigned>(n_queries * S)),
-                                        dim3(topk::kThreads), 0, stream, scores, cand_offsets, topk, S, ws, dev.err));
+                                        dim3(topk::kThreads), 0, stream, scores, cand_offsets, n_queries, topk, S, ws,
+                                        out_scores, out_pos, dev.err));
     if (st != TMS_OK) return st;
     return launch_status(launch_dependent(topk::topk_merge_kernel, dim3(static_cast<unsigned>(n_queries)),
                                           dim3(topk::kThreads), 0, stream, scores, cand_offsets, topk, S, ws,
