@@ -1714,9 +1714,17 @@ tms_status plan_tc(const DeviceInfo& dev, const Args& a, const Config* force, Pl
         }
         return best >= std::max(need, ctas == 2 ? 4 : 2);
     };
-    // default: as many copies as fit with 4 stages, else (one CTA) with 2
+    // default: as many copies as fit with 4 stages, else (one CTA) with 2 --
+    // with 3 of 256 rows where the query can be streamed instead.  The streamed
+    // tile leaves four of those, and two are too few to cover HBM: 4 x 8,000
+    // documents, fp16, 128 query tokens, d = 448: 547 us resident, 473 streamed
+    // (509 when the row maxima took no room and three stages were left); 96,
+    // d = 640: 795 and 642 (691); 64, d = 960: 1,168 and 953 (1,081); FP8, 128,
+    // d = 1,024: 627 and 511; shared by 4, fp16, d = 512: 251 and 197.  Three
+    // resident stages are as good (96, d = 512: 511 and 512).
     auto plan = [&](int str, int ctas, int& stages, int& qslots, int& reps, int most = 4) {
-        for (int need = 4; need >= (ctas == 2 ? 4 : 2); need -= 2)
+        const int least = ctas == 2 ? 4 : (str == 256 && !TF && !PQ ? 3 : 2);
+        for (int need : {4, least})
             for (int rp = std::min(max_reps, most); rp >= 1; rp /= 2)
                 if (fits(str, ctas, rp, need, stages, qslots)) {
                     reps = rp;
@@ -1773,11 +1781,8 @@ tms_status plan_tc(const DeviceInfo& dev, const Args& a, const Config* force, Pl
             if (plan(128, 2, stages, qslots, reps, !SH && KIND == kF16 && a.nchunks == 1 ? 2 : 4)) str = 128, ctas = 2;
             else if (plan(256, 1, stages, qslots, reps)) str = 256, ctas = 1;
             else if (plan(128, 1, stages, qslots, reps)) str = 128, ctas = 1;
-        } else {
-            // 256-row super-tiles unless the query tile leaves no room for
-            // their stages; then 128-row ones
-            if (plan(256, 1, stages, qslots, reps)) str = 256, ctas = 1;
-            else if (plan(128, 1, stages, qslots, reps)) str = 128, ctas = 1;
+        } else if (plan(256, 1, stages, qslots, reps)) {
+            str = 256, ctas = 1;
         }
     }
     if (ctas == 0 && !TF && !PQ) {
