@@ -1353,10 +1353,24 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
                         if (lane == 0) fin_ids[2 * nfin] = f;
                         if (++nfin == kFinRows) flush();
                     } else {
-                        float tot = warp_sum(row_value(0));
+                        // the blocks' sums over the warp, each as warp_sum
+                        // has it, with the blocks dealt to quarters of the
+                        // warp on the way: one at a time, four blocks'
+                        // twenty shuffles in a row bounded short documents
+                        // (8 x 10,000 of 16 tokens, 128 query tokens, d = 128:
+                        // FP8 281 us, now 156; fp16 272, now 151)
+                        const bool up16 = (lane & 16) != 0, up8 = (lane & 8) != 0;
+                        const float x0 = row_value(0), x1 = row_value(1), x2 = row_value(2), x3 = row_value(3);
+                        const float s0 = (up16 ? x2 : x0) + __shfl_xor_sync(0xffffffffu, up16 ? x0 : x2, 16);
+                        const float s1 = (up16 ? x3 : x1) + __shfl_xor_sync(0xffffffffu, up16 ? x1 : x3, 16);
+                        float sum = (up8 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, up8 ? s0 : s1, 8);
+#pragma unroll
+                        for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                        float tot = sum;  // lane 0: block 0; block b in lanes 8 b on
 #pragma unroll
                         for (int b = 1; b < kMaxBlocks; ++b) {
-                            if (b < a.bpc) tot += warp_sum(row_value(b));
+                            const float x = __shfl_sync(0xffffffffu, sum, 8 * b);
+                            if (b < a.bpc) tot += x;
                             m[b] = -INFINITY;
                         }
                         if (lane == 0) a.out[f] = tot;
