@@ -90,6 +90,19 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     return mbar_wait_slow(bar, parity, abort_flag, err, budget);
 }
 
+// Barrier `ID` (1 .. 15) of `THREADS` threads, whole warps: producers arrive
+// and go on, consumers wait for all of them.
+template <int ID, int THREADS>
+__device__ __forceinline__ void named_barrier_arrive() {
+    __syncwarp();
+    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(THREADS) : "memory");
+}
+template <int ID, int THREADS>
+__device__ __forceinline__ void named_barrier_sync() {
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(THREADS) : "memory");
+}
+
 // True in one lane of a converged warp, always the same one.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;

@@ -67,6 +67,7 @@
 #include <mutex>
 
 #include "tms_common.cuh"
+#include "tms_deal.cuh"
 #include "tms_internal.h"
 
 namespace tms {
@@ -125,6 +126,11 @@ __host__ __device__ constexpr int acc_count(int str, int ctas, bool qt) {
     return n < 4 ? n : 4;
 }
 constexpr int kMaxStages = 16;
+// Per-query lists: candidates per CTA from which their lengths are sampled (one
+// list of 180-token and fifteen of 32-token documents, 1,000 each, FP8, 52 per
+// CTA: 64.6 us not sampled, 29.2 sampled; 16 like lists of 650, 34 per CTA: 38.3
+// and 39.5).
+constexpr int kMinSampled = 24;
 constexpr int kSmemLimit = 232448;            // 227 KB opt-in maximum per CTA
 
 enum : int { kEnd = 1 };
@@ -181,6 +187,7 @@ struct Args {
     int last_groups;   // groups of the last round
     int n_queries;
     int nq;
+    int sampled;     // per-query lists: parts by estimated work (tms_deal.cuh); set by launch_tc
     int nchunks;     // ceil(d / chunk_elems)
     int stages;      // chunk stages in the ring
     int qslots;      // resident query-tile slots; 0: the query is streamed with each chunk stage
@@ -193,6 +200,10 @@ struct Args {
     int pq_k;                   // kPQ: centroids per subspace (codes >= pq_k read zeros)
     long long budget;           // SM cycles a pipeline wait may last (<= 0: kWaitBudgetCycles)
     int fault;                  // diagnostics: kFaultHoldAccumulator, else 0
+
+    __device__ __forceinline__ deal::Lists lists() const {
+        return deal::Lists{cand_offsets, cand_ids, lengths, n_docs, n_queries, static_cast<int>(n_flat)};
+    }
 };
 
 // Stands in for the row scale of a column past its document's end.
@@ -204,7 +215,7 @@ static __device__ const float kNanScale = __builtin_nanf("");
 constexpr int kFaultHoldAccumulator = TMS_FAULT_HOLD_ACCUMULATOR;
 
 struct Layout {
-    int q_off, qlo_off, stage_off, stage_stride, um_off, um_stride, fin_off, bias_off, sc_off, cb_off, code_off, st_off, bar_off,
+    int q_off, qlo_off, stage_off, stage_stride, um_off, um_stride, fin_off, bias_off, deal_off, sc_off, cb_off, code_off, st_off, bar_off,
         misc_off, total;
 };
 
@@ -247,7 +258,8 @@ __host__ __device__ inline Layout make_layout(int stages, int qslots, int nchunk
     L.um_stride = sh ? 0 : (str / 8) * blocks * 128;  // [unit][32-row block][row] row maxima
     L.fin_off = L.um_off + um_slots(nchunks) * L.um_stride;
     L.bias_off = (L.fin_off + (sh ? epi_warps(h) : 1) * kFinWarpBytes + 127) & ~127;
-    L.sc_off = L.bias_off + 256;
+    L.deal_off = L.bias_off + 256;
+    L.sc_off = L.deal_off + (sh ? 0 : deal::kSums * 4);
     L.cb_off = L.sc_off + (f8 ? st_ring(str) * str * 4 : 0);  // F8: [st_ring][str] column scales
     L.code_off = L.cb_off + (kind == kPQ ? kPqCbBytes : 0);                        // kPQ: fp16 codebook
     L.st_off = L.code_off + (kind == kPQ ? kCodeRing * str * kPqM : 0);  // kPQ: code-row ring
@@ -270,14 +282,10 @@ struct Meta {
 
 // The work items of one CTA, numbered k = 0, 1, ..., in the order in which
 // each lane takes its own: k = lane, lane + 32, ...
-// Per-query lists: the flat list is cut into gridDim.x equal parts, so a CTA
-// meets a few queries only, and loads few query tiles and leaves few
-// super-tiles part empty.  Within a query, the w or so CTAs that meet it take
-// its candidates in turn -- place x of the list is candidate t w + col, the
-// t-th of column col -- so that neighbours in the list, often alike in
-// length, are spread over them.  Score and top-k of 24 queries x 100 and 16 x
-// 1,000 candidates, every query dealt to every CTA: 42 and 92 us (fp16), 38 and
-// 84 (FP8), 82 and 235 (fp32); now 28 and 79, 27 and 64, 49 and 212.
+// Per-query lists: one part of the flat list (tms_deal.cuh).  Score and top-k
+// of 24 queries x 100 and 16 x 1,000 candidates, every query dealt to every
+// CTA: 42 and 92 us (fp16), 38 and 84 (FP8), 82 and 235 (fp32); in parts 28 and
+// 79, 27 and 64, 49 and 212.
 // Shared lists: the groups are taken in rounds of `round_groups` (the last
 // round `last_groups`); in a round the CTAs are dealt to its groups in turn
 // and a group's candidates to its CTAs in turn, so CTAs of different groups
@@ -324,70 +332,58 @@ struct Work<true> {
 
 template <>
 struct Work<false> {
-    int64_t n;                   // items of this CTA
-    int lo;                      // its first place in the flat list
-    int q, c0, end;              // this lane's query and its list
-    int w, wide, tall, rem;      // its columns: the first `rem` of `tall` entries (`wide` together), then of tall - 1
-    float parts;                 // parts (CTAs) per candidate
+    deal::Lists lists;
+    const int* sums;  // see deal::per_candidate
+    deal::Part part;
+    int64_t n;  // items of this CTA
+    int q;      // this lane's query
+    deal::Columns cols;
+    float parts;  // parts (CTAs) per candidate, equal parts
 
-    __device__ __forceinline__ explicit Work(const Args& a) {
-        const int total = static_cast<int>(a.n_flat), grid = gridDim.x;
-        const int each = total / grid, more = total - each * grid;
-        auto start = [&](int b) { return each * b + more * b / grid; };  // total * b / grid
-        lo = start(blockIdx.x);
-        n = start(blockIdx.x + 1) - lo;
-        parts = static_cast<float>(grid) / static_cast<float>(total);
+    __device__ __forceinline__ explicit Work(const Args& a)
+        : lists(a.lists()), sums(nullptr), part(deal::equal_part(lists)) {
+        parts = static_cast<float>(static_cast<int>(gridDim.x)) / static_cast<float>(lists.total);
+        begin();
+    }
+    // The sampled lengths are in `s`: whether the part is another one for them.
+    __device__ __forceinline__ bool recut(int* s) {
+        sums = s;
+        if (!deal::uneven_part(lists, s, &part)) return false;
+        begin();
+        return true;
+    }
+    __device__ __forceinline__ void begin() {
+        n = part.hi - part.lo;
         // the first query that ends past lo, 32 candidates for it at a time
         const int lane = threadIdx.x & 31;
         int base = 0;
-        for (int span = a.n_queries - 1; span > 0;) {
+        for (int span = lists.n_queries - 1; span > 0;) {
             const int step = (span + 31) / 32;
             const int last = min((lane + 1) * step, span) - 1;  // of this lane's piece
-            const bool before = lane * step < span && __ldg(a.cand_offsets + base + last + 1) <= lo;
+            const bool before = lane * step < span && __ldg(lists.offsets + base + last + 1) <= part.lo;
             const int pieces = __popc(__ballot_sync(0xffffffffu, before));
             base += min(pieces * step, span);
             span = min(step, span - min(pieces * step, span)) - 1;
         }
-        enter(a, base);
+        enter(base);
     }
-    __device__ __forceinline__ int bound(const Args& a, int i) const {
-        const int64_t x = __ldg(a.cand_offsets + i);
-        return static_cast<int>(x < 0 ? 0 : (x > a.n_flat ? a.n_flat : x));
-    }
-    __device__ __forceinline__ void enter(const Args& a, int query) {
+    __device__ __forceinline__ void enter(int query) {
         q = query;
-        c0 = 0, end = static_cast<int>(a.n_flat);  // one query: the first ids need not wait for its bounds
-        if (a.n_queries > 1) c0 = bound(a, q), end = bound(a, q + 1);
-        if (c0 >= end) return;
-        // about the CTAs that meet it (any number that all of them agree on will do)
-        w = min(max(__float2int_rn(static_cast<float>(end - c0) * parts), 1), end - c0);
-        tall = (end - c0 + w - 1) / w;
-        rem = end - c0 - (tall - 1) * w;
-        wide = rem * tall;
+        // one query: the first ids need not wait for its bounds
+        const bool one = lists.n_queries == 1;
+        cols.enter(one ? 0 : deal::bound(lists, q), one ? lists.total : deal::bound(lists, q + 1),
+                   part.uneven ? deal::per_candidate(lists, sums, q) : parts);
     }
     // Item k < n: its query and its flat index.
     __device__ __forceinline__ void at(const Args& a, int64_t k, int* query, int* pos) {
-        const int p = lo + static_cast<int>(k);
-        if (p >= end && q < a.n_queries - 1) {
+        const int p = part.lo + static_cast<int>(k);
+        if (p >= cols.end && q < a.n_queries - 1) {
             int next = q + 1;
-            while (next < a.n_queries - 1 && p >= bound(a, next + 1)) ++next;
-            enter(a, next);
+            while (next < a.n_queries - 1 && p >= deal::bound(lists, next + 1)) ++next;
+            enter(next);
         }
         *query = q;
-        int x = p - c0;
-        *pos = p;
-        if (x < 0 || p >= end) return;  // not a valid list
-        int col, t;
-        if (x < wide) {
-            col = x / tall;
-            t = x - col * tall;
-        } else {
-            x -= wide;
-            col = x / (tall - 1);
-            t = x - col * (tall - 1);
-            col += rem;
-        }
-        *pos = c0 + t * w + col;
+        *pos = p < cols.c0 || p >= cols.end ? p : cols.at(p);  // outside: not a valid list
     }
 };
 
@@ -500,6 +496,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
     constexpr int kHelpers = help_warps(KIND);
     constexpr int kHelpWarp = kFinWarp + fin_warps(SH);    // TF / kPQ: the first splitter / decompressor
     constexpr int kStRing = st_ring(STR);
+    constexpr int kDealThreads = 32 * (1 + kEpiWarps + fin_warps(SH));  // the planner and the warps that sample for it
     static_assert(KACC >= 2 && TCOLS * CTAS <= 512, "tensor memory of one SM");
 
     extern __shared__ uint8_t smem_raw[];
@@ -519,6 +516,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
     uint8_t* um_base = smem + L.um_off;    // per-query lists: [UMS][unit][block][row] row maxima
     uint8_t* fin_base = smem + L.fin_off;  // finished-document rows
     float* bias = reinterpret_cast<float*>(smem + L.bias_off);  // [8][8]: entry [n][j] 0 for j < n, else -inf
+    int* deal_sums = reinterpret_cast<int*>(smem + L.deal_off);  // per-query lists: see tms_deal.cuh
     float* sc = reinterpret_cast<float*>(smem + L.sc_off);      // F8: [kStRing][STR] scale of each column
     StSlot* slots = reinterpret_cast<StSlot*>(smem + L.st_off);
     uint8_t* cb = smem + L.cb_off;           // kPQ: fp16 codebook, entry (code, m) at (code * 16 + m) * 16
@@ -695,11 +693,23 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
             }
             return x;
         };
-        Item now = item(lane);
-        Meta cur = load_meta(a, now.id);
-        Item then = item(32 + lane);
-        Meta nxt = load_meta(a, then.id);
-        Item later = item(64 + lane);
+        Item now, then, later;
+        Meta cur, nxt;
+        auto first_windows = [&]() {
+            now = item(lane);
+            cur = load_meta(a, now.id);
+            then = item(32 + lane);
+            nxt = load_meta(a, then.id);
+            later = item(64 + lane);
+        };
+        first_windows();
+        if constexpr (!SH) {
+            // the samples' loads ran beside these
+            if (a.sampled) {
+                named_barrier_sync<1, kDealThreads>();
+                if (work.recut(deal_sums)) first_windows();
+            }
+        }
 
         for (int64_t k0 = 0;; k0 += 32) {
             if (k0 >= work.n) break;
@@ -1279,6 +1289,14 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
         // memory, and when they are full lane r sums row r in token order
         // and stores the score -- the same fixed order for every document,
         // wherever it sits in a batch.
+        if constexpr (!SH) {
+            // nothing to do here yet: the lists' lengths for the planner
+            if (a.sampled) {
+                deal::sample<8>(a.lists(), deal_sums, warp - kEpiWarp, kEpiWarps + fin_warps(SH));
+                __threadfence_block();
+                named_barrier_arrive<1, kDealThreads>();
+            }
+        }
         const bool finisher = !SH && warp >= kFinWarp;
         const int ew = finisher || !SH ? 0 : warp - kEpiWarp;
         float* fin_rows = reinterpret_cast<float*>(fin_base + ew * kFinWarpBytes);
@@ -1909,6 +1927,7 @@ tms_status launch_tc(const DeviceInfo& dev, const void* queries, tms_dtype dtype
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return launch_status(cudaErrorInvalidValue);
     const int64_t grid = std::min<int64_t>(static_cast<int64_t>(dev.sm_count) * ctas, a.n_flat);
+    a.sampled = !SH && a.n_queries > 1 && a.n_flat / grid >= kMinSampled;
     if (SH) plan_rounds(static_cast<int>(grid), static_cast<int>(a.n_flat / a.n_cand), a.n_cand, &a);
     return launch_status(launch_dependent(kern, dim3(static_cast<unsigned>(grid)), dim3(kernel_threads(KIND, H, SH)),
                                           static_cast<size_t>(smem), stream, maps, a));

@@ -56,3 +56,87 @@ def test_one_shared_candidate_uses_every_cta(cuda_lib):
     one = best_time(lambda: tms.score_dense_shared(q, tok, off, ln, ids[:1], out=out))
     few = best_time(lambda: tms.score_dense_shared(q[:256], tok, off, ln, ids, out=out.view(256, 16)))
     assert one < 3 * few, (one, few)
+
+
+def _uneven(kind, n_long, n_short, seed):
+    """Lists over a store of long (180 tokens) and short (32) documents: `apart`
+    in lists of their own, `mixed` in equal parts in every list -- the same
+    candidates in all."""
+    import torch
+    n_lists = 16
+    ln = synth.lengths_fixed(n_long + (n_lists - 1) * n_short, 32)
+    ln[:n_long] = 180
+    long_ids, short_ids = np.arange(n_long), n_long + np.arange((n_lists - 1) * n_short)
+    if kind == "apart":
+        lists = [long_ids] + list(short_ids.reshape(n_lists - 1, n_short))
+    else:
+        lists = [np.concatenate([long_ids[i::n_lists], short_ids[i::n_lists]]) for i in range(n_lists)]
+    g = np.random.default_rng(seed)
+    flat = np.concatenate([g.permutation(x) for x in lists]).astype(np.int32)
+    co = np.concatenate([[0], np.cumsum([len(x) for x in lists])]).astype(np.int64)
+    return ln, torch.from_numpy(flat).cuda(), torch.from_numpy(co).cuda()
+
+
+@pytest.mark.parametrize("dtype", ["f16", "fp8", "f32"])
+def test_lists_of_unlike_lengths_are_balanced(cuda_lib, dtype):
+    """One list of 180-token documents beside fifteen of 32-token ones, against
+    the same documents mixed in every list: about the same time (1.8 to 2.3
+    times in parts of equal count)."""
+    import torch
+    from paper_2606_26439_gb300 import tms
+    n = 4000 if dtype == "f32" else 10_000
+    t = []
+    for kind in ("apart", "mixed"):
+        ln, ids, co = _uneven(kind, n, n, 85)
+        tok, off, lens = synth.device_dense_corpus(ln, 128, "f32" if dtype == "f32" else "f16", 85)
+        q = synth.device_unit_rows(16 * 32, 128, "f32" if dtype == "f32" else "f16", 85, 1).view(16, 32, 128)
+        out = torch.empty(len(ids), device="cuda")
+        if dtype == "fp8":
+            (qc, qs), (tc, ts) = tms.quantize_e4m3(q), tms.quantize_e4m3(tok)
+            t.append(best_time(lambda: tms.score_fp8(qc, qs, tc, ts, off, lens, ids, co, out=out)))
+        else:
+            t.append(best_time(lambda: tms.score_dense(q, tok, off, lens, ids, co, out=out)))
+    assert t[0] < 1.35 * t[1], t
+
+
+@pytest.mark.parametrize("dtype", ["f16", "fp8", "f32"])
+@pytest.mark.parametrize("lists", [(20_000, 9000), (0, 15_000, 0, 1, 15_000, 0), (900,) * 32, (700,) * 43, (400,) * 70,
+                                   (1, 30_000), (60,) * 500 + (9000,) + (0,) * 100])
+def test_sampled_lists_write_every_candidate_once(cuda_lib, dtype, lists):
+    """Enough candidates for the lists' lengths to be sampled, short and long
+    documents by list and bad ids among them: every candidate has the bits that
+    its query and document give in a list of all documents."""
+    import torch
+    from paper_2606_26439_gb300 import tms
+    g = np.random.default_rng(len(lists))
+    n_docs = 400
+    ln = np.where(np.arange(n_docs) < 200, g.integers(1, 12, n_docs), g.integers(40, 90, n_docs)).astype(np.int32)
+    ln[7] = 0
+    base = "f32" if dtype == "f32" else "f16"
+    tok, off, lens = synth.device_dense_corpus(ln, 64, base, 86)
+    nQ = len(lists)
+    q = synth.device_unit_rows(nQ * 9, 64, base, 86, 1).view(nQ, 9, 64)
+    cands = [g.integers(0, 200, n) + 200 * (i % 3 == 1) for i, n in enumerate(lists)]
+    flat = np.concatenate(cands).astype(np.int32)
+    flat[::1000] = n_docs
+    co = torch.from_numpy(np.concatenate([[0], np.cumsum(lists)]).astype(np.int64)).cuda()
+    ids, every = torch.from_numpy(flat).cuda(), torch.arange(n_docs, dtype=torch.int32, device="cuda")
+    out = torch.full((len(flat),), 12345.0, device="cuda")
+    if dtype == "fp8":
+        (qc, qs), (tc, ts) = tms.quantize_e4m3(q), tms.quantize_e4m3(tok)
+        tms.score_fp8(qc, qs, tc, ts, off, lens, ids, co, out=out)
+        full = tms.score_fp8_shared(qc, qs, tc, ts, off, lens, every)
+    else:
+        tms.score_dense(q, tok, off, lens, ids, co, out=out)
+        if dtype == "f16":
+            full = tms.score_dense_shared(q, tok, off, lens, every)
+        else:
+            one = torch.tensor([0, n_docs], dtype=torch.int64, device="cuda")
+            full = torch.stack([tms.score_dense(q[i:i + 1], tok, off, lens, every, one) for i in range(nQ)])
+    torch.cuda.synchronize()
+    assert tms.device_error() == tms.TMS_DEVERR_BAD_ID
+    of = torch.repeat_interleave(torch.arange(nQ, device="cuda"), co.diff())
+    bad = ids == n_docs
+    want = full[of, ids.long().clamp_max(n_docs - 1)]
+    assert torch.isnan(out[bad]).all()
+    assert torch.equal(out[~bad].view(torch.int32), want[~bad].view(torch.int32))
