@@ -15,7 +15,10 @@
 // are sampled first, the same ones by every CTA, and where a list's documents
 // are longer than the average by a quarter, the parts are of equal estimated
 // work: 232 and 199.  Like lists keep parts of equal count, whose balance no
-// estimate reaches, and pay up to 1 us (16 x 1,000, fp16: 66.1 and 66.8).
+// estimate reaches, and pay up to 1 us (16 x 1,000, fp16: 66.1 and 66.8).  The
+// PQ kernel has no spare bandwidth to make up for uneven parts: the same lists
+// of 30,000, fp32 table, took 5,387 us in parts of equal count (2,952 with every
+// query dealt to every CTA), now 2,052.
 #pragma once
 
 #include "tms_common.cuh"
@@ -26,7 +29,6 @@ namespace deal {
 
 constexpr int kGroups = 32;   // lists told apart, one per lane; more are taken as groups of consecutive ones
 constexpr int kSums = 32;     // sums of 32 samples each: four for each of up to 8 groups, two for up to 16, else one
-constexpr int kDocRows = 16;  // what a document costs beside its rows, in rows
 
 struct Lists {
     const int64_t* offsets;  // [n_queries + 1]
@@ -57,11 +59,12 @@ struct Groups {
 };
 
 // Sums of 32 sampled candidates' rows each (rounded up to UNIT rows per
-// document), to sums[kSums] in shared memory; the warps share the work.  The
+// document, and DOC more for what it costs beside them), to sums[kSums] in
+// shared memory; the warps share the work.  The
 // samples are runs of eight neighbours, evenly spaced: a scattered load takes a
 // cycle for each of its lines, and twice as many samples of a place each took
 // 3 us.  Two loads, one after the other, whatever the lists.
-template <int UNIT>
+template <int UNIT, int DOC>
 __device__ __forceinline__ void sample(const Lists& l, int* sums, int warp, int warps) {
     constexpr int kBatch = 8;
     const int lane = threadIdx.x & 31;
@@ -83,7 +86,7 @@ __device__ __forceinline__ void sample(const Lists& l, int* sums, int warp, int 
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
             const int rows = (min(max(x[b], 0), 1 << 20) + UNIT - 1) & ~(UNIT - 1);
-            const int s = __reduce_add_sync(0xffffffffu, rows + kDocRows);
+            const int s = __reduce_add_sync(0xffffffffu, rows + DOC);
             if (lane == 0 && t0 + b * warps < tasks) sums[t0 + b * warps] = s;
         }
     }
@@ -169,19 +172,35 @@ struct Columns {
         rem = end - c0 - (tall - 1) * w;
         wide = rem * tall;
     }
-    // Entry at place p, c0 <= p < end.
-    __device__ __forceinline__ int at(int p) const {
-        int x = p - c0, col, t;
+    // Column and place in it of place p, c0 <= p < end.
+    __device__ __forceinline__ void find(int p, int* col, int* t) const {
+        int x = p - c0;
         if (x < wide) {
-            col = x / tall;
-            t = x - col * tall;
+            *col = x / tall;
+            *t = x - *col * tall;
         } else {
             x -= wide;
-            col = x / (tall - 1);
-            t = x - col * (tall - 1);
-            col += rem;
+            *col = x / (tall - 1);
+            *t = x - *col * (tall - 1);
+            *col += rem;
         }
-        return c0 + t * w + col;
+    }
+    __device__ __forceinline__ int entry(int col, int t) const { return c0 + t * w + col; }
+    // Entry at place p, c0 <= p < end.
+    __device__ __forceinline__ int at(int p) const {
+        int col, t;
+        find(p, &col, &t);
+        return entry(col, t);
+    }
+    // Entry `more` places on from (col, t), still before end: a part spans a
+    // column or two, so this needs no division.
+    __device__ __forceinline__ int ahead(int col, int t, int more) const {
+        t += more;
+        for (int h = col < rem ? tall : tall - 1; t >= h; h = col < rem ? tall : tall - 1) {
+            t -= h;
+            ++col;
+        }
+        return entry(col, t);
     }
 };
 

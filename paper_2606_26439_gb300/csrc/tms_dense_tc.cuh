@@ -1292,7 +1292,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
         if constexpr (!SH) {
             // nothing to do here yet: the lists' lengths for the planner
             if (a.sampled) {
-                deal::sample<8>(a.lists(), deal_sums, warp - kEpiWarp, kEpiWarps + fin_warps(SH));
+                deal::sample<8, 16>(a.lists(), deal_sums, warp - kEpiWarp, kEpiWarps + fin_warps(SH));
                 __threadfence_block();
                 named_barrier_arrive<1, kDealThreads>();
             }

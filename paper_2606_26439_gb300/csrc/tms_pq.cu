@@ -29,6 +29,7 @@
 #include <algorithm>
 
 #include "tms_common.cuh"
+#include "tms_deal.cuh"
 #include "tms_internal.h"
 
 namespace tms {
@@ -79,6 +80,7 @@ struct Args {
     int n_queries;
     int nq;
     int K;
+    int sampled;       // score_kernel_staged: parts by estimated work (tms_deal.cuh)
     long long budget;  // SM cycles a wait may last (<= 0: kWaitBudgetCycles)
 };
 
@@ -337,8 +339,7 @@ __device__ __forceinline__ void gather_groups(const CodeRow<M>& c, uint32_t tbl,
 }
 
 struct PendingMeta {
-    int64_t f;  // candidate, -1: none
-    bool done;  // no cells left
+    int f;  // candidate, -1: none left
     int id;
     int64_t off;
     int len;
@@ -348,52 +349,9 @@ struct PendingMeta {
 // a code >= k still reads inside the allocation.
 __host__ __device__ constexpr int staged_table_bytes(int M) { return ((M / 8 - 1) * (4096 / M) + 256) * 256; }
 
-// One CTA's share of the candidates.  The flat list of all queries' candidates
-// is cut into gridDim.x equal parts; a CTA works on the queries its part
-// meets, so it stages the table of one or two queries and not of every one (at
-// 17 us a chunk then, and 152 CTAs, 16 queries x 50,000 candidates spent 1.1
-// of 6.7 ms on it and 16 x 1,000 with 100 query tokens 3.4 of 4.1 ms).  Within
-// a query, the W CTAs that meet it take its candidates in turn, so that
-// neighbours in the list, often alike in length, are spread over them: cell
-// u = col R + t of a W x R grid is candidate t W + col, and the CTAs take
-// consecutive cells in proportion to their parts (the last row's cells past
-// the list's end are empty).
-struct Share {
-    int64_t c0;    // the query's first candidate
-    int len;       // its candidates
-    int n;         // cells of this CTA; 0: it does not meet the query
-    int w, rows;   // W and R
-    int col0, t0;  // the first cell's column and row
-
-    __device__ __forceinline__ Share(const Args& a, int q) : n(0) {
-        c0 = __ldg(a.cand_offsets + q);
-        int64_t c1 = __ldg(a.cand_offsets + q + 1);
-        c0 = c0 < 0 ? 0 : (c0 > a.n_cand ? a.n_cand : c0);
-        c1 = c1 < c0 ? c0 : (c1 > a.n_cand ? a.n_cand : c1);
-        const int64_t grid = gridDim.x, b = blockIdx.x;
-        const int64_t lo = max(a.n_cand * b / grid, c0), hi = min(a.n_cand * (b + 1) / grid, c1);
-        if (lo >= hi) return;
-        len = static_cast<int>(c1 - c0);
-        w = static_cast<int>((c1 * grid - 1) / a.n_cand - ((c0 + 1) * grid - 1) / a.n_cand) + 1;
-        rows = (len + w - 1) / w;
-        const int64_t cells = static_cast<int64_t>(rows) * w;
-        const int64_t u0 = (lo - c0) * cells / len, u1 = (hi - c0) * cells / len;
-        n = static_cast<int>(u1 - u0);
-        col0 = static_cast<int>(u0 / rows);
-        t0 = static_cast<int>(u0 - static_cast<int64_t>(col0) * rows);
-    }
-    // Candidate of cell li, or -1 (an empty cell).
-    __device__ __forceinline__ int64_t at(int li) const {
-        int64_t t = static_cast<int64_t>(t0) + li;
-        int col = col0;
-        while (t >= rows) {
-            t -= rows;
-            ++col;
-        }
-        const int64_t j = t * w + col;
-        return j < len ? c0 + j : -1;
-    }
-};
+// Candidates per CTA from which the lists' lengths are sampled: below, the
+// chunks' staging is most of the time.
+constexpr int kMinSampled = 64;
 
 // Words (.x .y .z .w: four codes) of four subspaces, rotated by kq.
 __device__ __forceinline__ void rotate4(uint4 (&v)[4], int kq) {
@@ -454,10 +412,35 @@ __global__ void __launch_bounds__(kWarps * 32, 1) score_kernel_staged(const Args
         atomicOr(a.err, TMS_DEVERR_BAD_CSR);
     uint32_t issued = 0, consumed = 0;  // pieces of this warp (buffer = count & 1)
 
+    // This CTA's part of the flat candidate list (tms_deal.cuh): it stages the
+    // table of one or two queries and not of every one (at 17 us a chunk then,
+    // and 152 CTAs, 16 queries x 50,000 candidates spent 1.1 of 6.7 ms on it and
+    // 16 x 1,000 with 100 query tokens 3.4 of 4.1 ms).
+    const deal::Lists lists{a.cand_offsets, a.cand_ids, a.lengths, a.n_docs, a.n_queries, static_cast<int>(a.n_cand)};
+    __shared__ int deal_sums[deal::kSums];
+    __shared__ deal::Part shared_part;
+    deal::Part part = deal::equal_part(lists);
+    if (a.sampled) {
+        deal::sample<16, 40>(lists, deal_sums, warp, kWarps);
+        __syncthreads();
+        if (warp == 0) {
+            deal::uneven_part(lists, deal_sums, &part);
+            if (lane == 0) shared_part = part;
+        }
+        __syncthreads();
+        part = shared_part;
+    }
+    const float parts = static_cast<float>(static_cast<int>(gridDim.x)) / static_cast<float>(lists.total);
+
     for (int q = 0; q < a.n_queries; ++q) {
-        const Share share(a, q);
-        const int n_local = share.n;
-        if (n_local == 0) continue;
+        deal::Columns cols;
+        cols.c0 = deal::bound(lists, q), cols.end = deal::bound(lists, q + 1);
+        const int first = max(part.lo, cols.c0);
+        const int n_local = min(part.hi, cols.end) - first;
+        if (n_local <= 0) continue;
+        cols.enter(cols.c0, cols.end, part.uneven ? deal::per_candidate(lists, deal_sums, q) : parts);
+        int col0, t0;
+        cols.find(first, &col0, &t0);
         for (int ch = 0; ch < nchunks; ++ch) {
             __syncthreads();
             // Table chunk -> shared memory, zeros for codes >= k and query
@@ -552,10 +535,9 @@ __global__ void __launch_bounds__(kWarps * 32, 1) score_kernel_staged(const Args
                 if (lane == 0) li = atomicAdd(&next_local, 1);
                 return __shfl_sync(0xffffffffu, li, 0);
             };
-            auto fetch = [&](int li) {  // issue the metadata loads of cell li's candidate
+            auto fetch = [&](int li) {  // issue the metadata loads of the li-th candidate
                 PendingMeta m;
-                m.done = li >= n_local;
-                m.f = m.done ? -1 : share.at(li);
+                m.f = li < n_local ? cols.ahead(col0, t0, li) : -1;
                 m.id = -1;
                 m.off = 0;
                 m.len = 0;
@@ -573,14 +555,10 @@ __global__ void __launch_bounds__(kWarps * 32, 1) score_kernel_staged(const Args
             PendingMeta pend = fetch(grab());
             auto take = [&](int64_t& f, int64_t& off, int& len) {
                 for (;;) {
-                    if (pend.done) {
-                        f = -1;
-                        return;
-                    }
+                    f = pend.f;
+                    if (f < 0) return;
                     const PendingMeta cur = pend;
                     pend = fetch(grab());
-                    f = cur.f;
-                    if (f < 0) continue;
                     int status = 0;
                     if (cur.id < 0 || cur.id >= a.n_docs)
                         status = 1;
@@ -769,6 +747,7 @@ tms_status score(const float* lut, int n_queries, int nq, int m, int k, const ui
     a.n_queries = n_queries;
     a.nq = nq;
     a.K = k;
+    a.sampled = n_queries > 1 && n_cand / dev.sm_count >= kMinSampled;
     // The last subspace group is sized for 256 codes so that a code >= k
     // still indexes inside the allocation.
     const int smem = ((m / 4 - 1) * k + 256) * 32 * 4;

@@ -77,10 +77,10 @@ def _uneven(kind, n_long, n_short, seed):
     return ln, torch.from_numpy(flat).cuda(), torch.from_numpy(co).cuda()
 
 
-@pytest.mark.parametrize("dtype", ["f16", "fp8", "f32"])
+@pytest.mark.parametrize("dtype", ["f16", "fp8", "f32", "pq", "pq_f16"])
 def test_lists_of_unlike_lengths_are_balanced(cuda_lib, dtype):
     """One list of 180-token documents beside fifteen of 32-token ones, against
-    the same documents mixed in every list: about the same time (1.8 to 2.3
+    the same documents mixed in every list: about the same time (1.8 to 2.6
     times in parts of equal count)."""
     import torch
     from paper_2606_26439_gb300 import tms
@@ -88,6 +88,14 @@ def test_lists_of_unlike_lengths_are_balanced(cuda_lib, dtype):
     t = []
     for kind in ("apart", "mixed"):
         ln, ids, co = _uneven(kind, n, n, 85)
+        if dtype.startswith("pq"):
+            codes = torch.randint(0, 256, (int(ln.sum()), 16), dtype=torch.uint8, device="cuda")
+            off, lens = (torch.from_numpy(x).cuda() for x in (synth.offsets_of(ln), ln.astype(np.int32)))
+            table = torch.randn((16, 32, 16, 256), device="cuda")
+            out = torch.empty(len(ids), device="cuda")
+            t.append(best_time(lambda: tms.score_pq(table, codes, off, lens, ids, co, out=out,
+                                                    f16_table=dtype == "pq_f16"), 5))
+            continue
         tok, off, lens = synth.device_dense_corpus(ln, 128, "f32" if dtype == "f32" else "f16", 85)
         q = synth.device_unit_rows(16 * 32, 128, "f32" if dtype == "f32" else "f16", 85, 1).view(16, 32, 128)
         out = torch.empty(len(ids), device="cuda")
@@ -99,7 +107,7 @@ def test_lists_of_unlike_lengths_are_balanced(cuda_lib, dtype):
     assert t[0] < 1.35 * t[1], t
 
 
-@pytest.mark.parametrize("dtype", ["f16", "fp8", "f32"])
+@pytest.mark.parametrize("dtype", ["f16", "fp8", "f32", "pq", "pq_f16"])
 @pytest.mark.parametrize("lists", [(20_000, 9000), (0, 15_000, 0, 1, 15_000, 0), (900,) * 32, (700,) * 43, (400,) * 70,
                                    (1, 30_000), (60,) * 500 + (9000,) + (0,) * 100])
 def test_sampled_lists_write_every_candidate_once(cuda_lib, dtype, lists):
@@ -115,6 +123,7 @@ def test_sampled_lists_write_every_candidate_once(cuda_lib, dtype, lists):
     base = "f32" if dtype == "f32" else "f16"
     tok, off, lens = synth.device_dense_corpus(ln, 64, base, 86)
     nQ = len(lists)
+    one = torch.tensor([0, n_docs], dtype=torch.int64, device="cuda")
     q = synth.device_unit_rows(nQ * 9, 64, base, 86, 1).view(nQ, 9, 64)
     cands = [g.integers(0, 200, n) + 200 * (i % 3 == 1) for i, n in enumerate(lists)]
     flat = np.concatenate(cands).astype(np.int32)
@@ -122,7 +131,13 @@ def test_sampled_lists_write_every_candidate_once(cuda_lib, dtype, lists):
     co = torch.from_numpy(np.concatenate([[0], np.cumsum(lists)]).astype(np.int64)).cuda()
     ids, every = torch.from_numpy(flat).cuda(), torch.arange(n_docs, dtype=torch.int32, device="cuda")
     out = torch.full((len(flat),), 12345.0, device="cuda")
-    if dtype == "fp8":
+    if dtype.startswith("pq"):
+        table = torch.randn((nQ, 9, 32, 100), device="cuda")
+        codes = torch.randint(0, 100, (int(ln.sum()), 32), dtype=torch.uint8, device="cuda")
+        score = lambda i, *x, **k: tms.score_pq(table[i], codes, off, lens, *x, f16_table=dtype == "pq_f16", **k)  # noqa: E731
+        score(slice(None), ids, co, out=out)
+        full = torch.stack([score(slice(i, i + 1), every, one) for i in range(nQ)])
+    elif dtype == "fp8":
         (qc, qs), (tc, ts) = tms.quantize_e4m3(q), tms.quantize_e4m3(tok)
         tms.score_fp8(qc, qs, tc, ts, off, lens, ids, co, out=out)
         full = tms.score_fp8_shared(qc, qs, tc, ts, off, lens, every)
@@ -131,7 +146,6 @@ def test_sampled_lists_write_every_candidate_once(cuda_lib, dtype, lists):
         if dtype == "f16":
             full = tms.score_dense_shared(q, tok, off, lens, every)
         else:
-            one = torch.tensor([0, n_docs], dtype=torch.int64, device="cuda")
             full = torch.stack([tms.score_dense(q[i:i + 1], tok, off, lens, every, one) for i in range(nQ)])
     torch.cuda.synchronize()
     assert tms.device_error() == tms.TMS_DEVERR_BAD_ID
