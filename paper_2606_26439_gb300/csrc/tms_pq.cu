@@ -365,6 +365,71 @@ __device__ __forceinline__ void rotate4(uint4 (&v)[4], int kq) {
     }
 }
 
+// Table chunk -> shared memory, zeros for codes >= k and query tokens >= nq.  A
+// warp fills 16 rows x one 128-byte half (slo) per task: lane (ii, kq) loads
+// four codes from 4 kq on of each of the half's four subspaces of query token
+// ii -- 64 bytes of eight table rows per instruction -- and stores them in an
+// order that kq rotates over the subspaces, so that a store's 32 words fall in
+// 32 banks.  A 128 KB chunk took 17 us with scalar loads of 32 rows each (32,768
+// lines looked up in L1, one a cycle) and takes 5.3 with these (2,048): 3.7 TB/s
+// from L2 over all SMs, whether two or four tasks of a warp are in flight.
+// Table rows that are not 16-byte aligned (ALIGNED false) take four loads of
+// the same 64 bytes instead of one: K = 250, one list of 100 candidates 37.5 us,
+// 55.4 with 32 rows per load; fp16 table 31.5 and 43.8.
+template <int M, bool H16, bool ALIGNED>
+__device__ __forceinline__ void stage_chunk(const float* src, int nq, int K, int ch, float* lut_s, int warp,
+                                            int lane) {
+    constexpr int KS = 4096 / M;        // table rows per block
+    constexpr int QC = H16 ? 16 : kQC;  // query tokens per chunk
+    const int ii = lane & 7;
+    const int kq = lane >> 3;
+    constexpr int kTasks = staged_table_bytes(M) / 256 / 16 * 2;
+#pragma unroll 2
+    for (int task = warp; task < kTasks; task += kWarps) {
+        const int slo = task & 1;
+        const int rho0 = (task >> 1) * 16;  // KS is a multiple of 16
+        const int shi = min(rho0 / KS, M / 8 - 1);
+        const int kk = rho0 - shi * KS + 4 * kq;
+        const int mb = 4 * (2 * shi + slo);
+        uint4 v[4];
+#pragma unroll
+        for (int ml = 0; ml < 4; ++ml) {
+            auto load = [&](int qi) {
+                const float* p = src + (static_cast<int64_t>(qi) * M + mb + ml) * K + kk;
+                if constexpr (ALIGNED)
+                    return qi < nq && kk < K ? __ldg(reinterpret_cast<const float4*>(p))
+                                               : make_float4(0.f, 0.f, 0.f, 0.f);
+                const int n = qi < nq ? K - kk : 0;
+                return make_float4(n > 0 ? __ldg(p) : 0.f, n > 1 ? __ldg(p + 1) : 0.f,
+                                   n > 2 ? __ldg(p + 2) : 0.f, n > 3 ? __ldg(p + 3) : 0.f);
+            };
+            if constexpr (H16) {  // query tokens 2 ii and 2 ii + 1, rounded to nearest fp16
+                const float4 x = load(ch * QC + 2 * ii), y = load(ch * QC + 2 * ii + 1);
+                v[ml] = make_uint4(pack_f16x2(x.x, y.x), pack_f16x2(x.y, y.y), pack_f16x2(x.z, y.z),
+                                   pack_f16x2(x.w, y.w));
+            } else {
+                const float4 x = load(ch * QC + ii);
+                v[ml] = make_uint4(__float_as_uint(x.x), __float_as_uint(x.y), __float_as_uint(x.z),
+                                   __float_as_uint(x.w));
+            }
+        }
+        rotate4(v, kq);
+        uint32_t* dst = reinterpret_cast<uint32_t*>(lut_s) + (rho0 + 4 * kq) * 64 + slo * 32 + ii;
+#pragma unroll
+        for (int st = 0; st < 4; ++st) {
+            uint32_t* d = dst + ((st + kq) & 3) * 8;
+            d[0] = v[st].x, d[64] = v[st].y, d[128] = v[st].z, d[192] = v[st].w;
+        }
+    }
+}
+
+// Out of line: inlined a second time, it cost the gather loop 1.6% (fp16 table).
+template <int M, bool H16>
+__device__ __noinline__ void stage_chunk_any(const float* src, int nq, int K, int ch, float* lut_s, int warp,
+                                             int lane) {
+    stage_chunk<M, H16, false>(src, nq, K, ch, lut_s, warp, lane);
+}
+
 template <int M, bool H16>
 __global__ void __launch_bounds__(kWarps * 32, 1) score_kernel_staged(const Args a, int lut_bytes) {
     griddep_wait();
@@ -443,90 +508,11 @@ __global__ void __launch_bounds__(kWarps * 32, 1) score_kernel_staged(const Args
         cols.find(first, &col0, &t0);
         for (int ch = 0; ch < nchunks; ++ch) {
             __syncthreads();
-            // Table chunk -> shared memory, zeros for codes >= k and query
-            // tokens >= nq.  A warp fills 16 rows x one 128-byte half (slo) per
-            // task: lane (ii, kq) loads four codes from 4 kq on of each of the
-            // half's four subspaces of query token ii -- 64 bytes of eight
-            // table rows per instruction -- and stores them in an order that
-            // kq rotates over the subspaces, so that a store's 32 words fall
-            // in 32 banks.  A 128 KB chunk took 17 us with scalar loads of 32
-            // rows each (32,768 lines looked up in L1, one a cycle) and takes
-            // 5.3 with these (2,048): 3.7 TB/s from L2 over all SMs, whether
-            // two or four tasks of a warp are in flight.
             const float* src = a.lut + static_cast<int64_t>(q) * a.nq * M * K;
-            const int ii = lane & 7;
-            if ((K & 3) == 0) {
-                constexpr int kTasks = staged_table_bytes(M) / 256 / 16 * 2;
-                const int kq = lane >> 3;
-#pragma unroll 2
-                for (int task = warp; task < kTasks; task += kWarps) {
-                    const int slo = task & 1;
-                    const int rho0 = (task >> 1) * 16;  // KS is a multiple of 16
-                    const int shi = min(rho0 / KS, M / 8 - 1);
-                    const int kk = rho0 - shi * KS + 4 * kq;
-                    const int mb = 4 * (2 * shi + slo);
-                    uint4 v[4];
-#pragma unroll
-                    for (int ml = 0; ml < 4; ++ml) {
-                        auto load = [&](int qi) {
-                            return qi < a.nq && kk < K
-                                       ? __ldg(reinterpret_cast<const float4*>(
-                                             src + (static_cast<int64_t>(qi) * M + mb + ml) * K + kk))
-                                       : make_float4(0.f, 0.f, 0.f, 0.f);
-                        };
-                        if constexpr (H16) {  // query tokens 2 ii and 2 ii + 1, rounded to nearest fp16
-                            const float4 x = load(ch * QC + 2 * ii), y = load(ch * QC + 2 * ii + 1);
-                            v[ml] = make_uint4(pack_f16x2(x.x, y.x), pack_f16x2(x.y, y.y), pack_f16x2(x.z, y.z),
-                                               pack_f16x2(x.w, y.w));
-                        } else {
-                            const float4 x = load(ch * QC + ii);
-                            v[ml] = make_uint4(__float_as_uint(x.x), __float_as_uint(x.y), __float_as_uint(x.z),
-                                               __float_as_uint(x.w));
-                        }
-                    }
-                    rotate4(v, kq);
-                    uint32_t* dst = reinterpret_cast<uint32_t*>(lut_s) + (rho0 + 4 * kq) * 64 + slo * 32 + ii;
-#pragma unroll
-                    for (int st = 0; st < 4; ++st) {
-                        uint32_t* d = dst + ((st + kq) & 3) * 8;
-                        d[0] = v[st].x, d[64] = v[st].y, d[128] = v[st].z, d[192] = v[st].w;
-                    }
-                }
-            } else {  // rows of any alignment: a lane reads 8 consecutive codes of one
-                const int ml = lane >> 3;
-                const int tasks = (lut_bytes / 256 / 8) * 2;
-                for (int task = warp; task < tasks; task += kWarps) {
-                    const int slo = task & 1;
-                    const int rho0 = (task >> 1) * 8;               // KS is a multiple of 8
-                    const int shi = min(rho0 / KS, M / 8 - 1);
-                    const int kk0 = rho0 - shi * KS;
-                    const int m = 4 * (2 * shi + slo) + ml;
-                    float* dst = lut_s + rho0 * 64 + slo * 32 + ml * 8 + ii;
-                    if constexpr (H16) {  // query tokens 2 ii and 2 ii + 1, rounded to nearest fp16
-                        const int qi = ch * QC + 2 * ii;
-                        const float* r0 = src + (static_cast<int64_t>(qi) * M + m) * K;
-                        const float* r1 = r0 + static_cast<int64_t>(M) * K;
-                        const bool ok0 = qi < a.nq, ok1 = qi + 1 < a.nq;
-#pragma unroll
-                        for (int x = 0; x < 8; ++x) {
-                            const int kk = kk0 + x;
-                            const float t0 = (ok0 && kk < K) ? __ldg(r0 + kk) : 0.f;
-                            const float t1 = (ok1 && kk < K) ? __ldg(r1 + kk) : 0.f;
-                            const __half2 h = __floats2half2_rn(t0, t1);
-                            dst[x * 64] = *reinterpret_cast<const float*>(&h);
-                        }
-                    } else {
-                        const int qi = ch * QC + ii;
-                        const float* r0 = src + (static_cast<int64_t>(qi) * M + m) * K;
-                        const bool ok0 = qi < a.nq;
-#pragma unroll
-                        for (int x = 0; x < 8; ++x) {
-                            const int kk = kk0 + x;
-                            dst[x * 64] = (ok0 && kk < K) ? __ldg(r0 + kk) : 0.f;
-                        }
-                    }
-                }
-            }
+            if ((K & 3) == 0)
+                stage_chunk<M, H16, true>(src, a.nq, K, ch, lut_s, warp, lane);
+            else
+                stage_chunk_any<M, H16>(src, a.nq, K, ch, lut_s, warp, lane);
             if (threadIdx.x == 0) next_local = 0;
             __syncthreads();
 

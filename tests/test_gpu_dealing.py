@@ -154,3 +154,22 @@ def test_sampled_lists_write_every_candidate_once(cuda_lib, dtype, lists):
     want = full[of, ids.long().clamp_max(n_docs - 1)]
     assert torch.isnan(out[bad]).all()
     assert torch.equal(out[~bad].view(torch.int32), want[~bad].view(torch.int32))
+
+
+@pytest.mark.parametrize("f16", [False, True])
+def test_table_rows_of_any_alignment_are_staged_alike(cuda_lib, f16):
+    """One short list, where staging the table is most of the time, with 255
+    centroids (rows not 16-byte aligned) against 256: 1.1 times (1.6 when a load
+    touched 32 rows)."""
+    import torch
+    from paper_2606_26439_gb300 import tms
+    ln = synth.lengths_fixed(100, 100)
+    codes = torch.randint(0, 255, (int(ln.sum()), 16), dtype=torch.uint8, device="cuda")
+    off, lens = (torch.from_numpy(x).cuda() for x in (synth.offsets_of(ln), ln.astype(np.int32)))
+    ids, co = torch.arange(100, dtype=torch.int32, device="cuda"), torch.tensor([0, 100], device="cuda")
+    out = torch.empty(100, device="cuda")
+    t = []
+    for k in (255, 256):
+        table = torch.randn((1, 32, 16, k), device="cuda")
+        t.append(best_time(lambda: tms.score_pq(table, codes, off, lens, ids, co, out=out, f16_table=f16), 50))
+    assert t[0] < 1.4 * t[1], t
