@@ -77,17 +77,17 @@ typedef enum { TMS_F16 = 0, TMS_BF16 = 1, TMS_F32 = 2 } tms_dtype;
  * Limits: 1 <= nq <= 128; 8 <= d <= 1024 with d % 8 == 0 (16-byte rows);
  * 1 <= n_queries <= 4096; n_tokens < 2^31; queries, doc_tokens and every
  * index array 16-byte aligned.  For fp16/bf16 the query tile stays in
- * shared memory when it fits beside the document stages (nq * d * 2 bytes,
- * nq rounded up to 32 and d to 64, up to 188,416) and is otherwise streamed
- * from L2 with each 128-byte dimension chunk of the documents (Section 3's
- * dimension tiling applied to the query as well), so every nq and d above
- * is supported.  fp16/bf16 run on the tensor cores
+ * shared memory when it leaves room for three stages of documents (nq * d * 2
+ * bytes, nq rounded up to 32 and d to 64, up to 114,688) and is otherwise
+ * streamed from L2 with each 128-byte dimension chunk of the documents
+ * (Section 3's dimension tiling applied to the query as well), so every nq
+ * and d above is supported.  fp16/bf16 run on the tensor cores
  * (tcgen05, fp32 accumulation in tensor memory); fp32 runs split TF32 on
  * the tensor cores (x = hi + lo, hi = x with its 13 low mantissa bits
  * cleared, lo the exact rest; hi.hi + hi.lo + lo.hi, FP32-level accuracy)
- * when its doubled query tile fits, else an
- * exact fp32 CUDA-core kernel (any supported nq, d).  A candidate with a bad id or row range scores NaN and sets
- * TMS_DEVERR_BAD_ID / TMS_DEVERR_BAD_RANGE.
+ * for ceil(nq / 32) * ceil(d / 32) <= 18 and d <= 544, else an exact fp32
+ * CUDA-core kernel (any supported nq, d).  A candidate with a bad id or row
+ * range scores NaN and sets TMS_DEVERR_BAD_ID / TMS_DEVERR_BAD_RANGE.
  */
 tms_status tms_score_dense(const void *queries, tms_dtype dtype, int n_queries, int nq, int d,
                            const void *doc_tokens, int64_t n_tokens,

@@ -266,35 +266,12 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                  : "memory");
 }
 
-// Load 32 consecutive fp32 columns of this warp's 32 TMEM lanes (one lane
-// per thread) and wait for them.  The wait names every output register so
-// no use can be scheduled before it.
 // max(a, b, c) in one instruction; NaN inputs are ignored unless all are
 // NaN (as fmaxf ignores one).
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
     float r;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
-}
-
-// max(m, v[0..31]) with three-input maxima: 16 instructions.
-__device__ __forceinline__ float fold_max32(float m, const float (&v)[32]) {
-    float a[11];
-#pragma unroll
-    for (int i = 0; i < 10; ++i) a[i] = fmax3(v[3 * i], v[3 * i + 1], v[3 * i + 2]);
-    a[10] = fmaxf(v[30], v[31]);
-    const float b0 = fmax3(a[0], a[1], a[2]), b1 = fmax3(a[3], a[4], a[5]), b2 = fmax3(a[6], a[7], a[8]);
-    const float b3 = fmax3(a[9], a[10], m);
-    return fmax3(fmaxf(b0, b1), b2, b3);
-}
-
-// max(m, v[lo..hi)) (0 <= lo < hi <= 32): the columns outside [lo, hi)
-// are dropped (-inf) before the three-input fold.
-__device__ __forceinline__ float fold_max32_range(float m, const float (&v)[32], int lo, int hi) {
-    float w[32];
-#pragma unroll
-    for (int c = 0; c < 32; ++c) w[c] = (c >= lo && c < hi) ? v[c] : -INFINITY;
-    return fold_max32(m, w);
 }
 
 // (a, b) *= (x, y) in one packed instruction; each product is rounded as a
@@ -385,6 +362,9 @@ __device__ __forceinline__ void tmem_ld_blocks(uint32_t taddr, uint32_t (&r)[2][
                  : "memory");
 }
 
+// Load 32 consecutive fp32 columns of this warp's 32 TMEM lanes (one lane
+// per thread) and wait for them.  The wait names every output register so
+// no use can be scheduled before it.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     uint32_t r[32];
     tmem_ld32_issue(taddr, r);
@@ -408,20 +388,6 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
-// Max of v over the lanes in `mask` (every lane in mask must execute it),
-// returned to each of them.  NaN inputs are ignored like fmaxf.
-__device__ __forceinline__ float redux_max(float v, unsigned mask) {
-    float r;
-    asm volatile("redux.sync.max.f32 %0, %1, %2;" : "=f"(r) : "f"(v), "r"(mask));
-    return r;
 }
 
 }  // namespace tms

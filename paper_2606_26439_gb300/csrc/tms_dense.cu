@@ -1,7 +1,8 @@
 // tms_dense.cu -- dense MaxSim entry points for fp16 / bf16 / fp32 rows.
 //
 // fp16 / bf16 run the tensor-core kernel of tms_dense_tc.cuh; fp32 too (split
-// TF32) where its doubled query tile fits, else an exact-fp32 CUDA-core kernel.
+// TF32) for up to 18 pairs of a 32-token query block and a 32-element chunk and
+// up to 17 chunks, else an exact-fp32 CUDA-core kernel.
 #include "tms_dense_tc.cuh"
 
 namespace tms {
@@ -200,7 +201,7 @@ tms_status score_dense(const void* queries, tms_dtype dtype, int n_queries, int 
 
     if (dtype == TMS_F32) {
         // split TF32 on the tensor cores; the exact CUDA-core kernel below
-        // covers the shapes whose query tile does not fit
+        // covers the shapes that plan_tc's rule leaves out
         a.nchunks = (d + dense::chunk_elems(dense::kTF32) - 1) / dense::chunk_elems(dense::kTF32);
         st = tune ? dense::tune_tc<1, false, dense::kTF32>(dev, queries, dtype, n_queries, nq, d, doc_tokens, n_tokens,
                                                            a, stream, n_timed)

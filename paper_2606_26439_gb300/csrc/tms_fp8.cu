@@ -71,8 +71,10 @@ __device__ __forceinline__ uint32_t encode2(float a, float b) {
 // loaded before their arithmetic.
 //
 // Few lanes per row, so that a row's shuffles and its two reciprocals are
-// spread over up to 32 elements per lane; every access still covers whole
-// 32-byte sectors.  Bound by HBM once the arithmetic is small enough.  4 M
+// spread over up to 32 elements per lane; for d > 64 every access still covers
+// whole 32-byte sectors (narrower rows store 8-byte pieces of them, and 200 M
+// fp16 elements take 105 us at d = 64, 132 at 32, 121 at 16, against 92 at 128;
+// one warp per row took 820 to 3,155).  Bound by HBM once the arithmetic is small enough.  4 M
 // fp16 rows of 128 (1.55 GB): one warp per row with 8-byte loads, an IEEE
 // division and a one-element conversion per code took 1,042 us (ALU 48%
 // busy, DRAM 18%); 16 lanes per row with one unit each 349 us (issue 61%
