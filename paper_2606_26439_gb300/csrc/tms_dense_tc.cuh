@@ -302,7 +302,7 @@ struct Work<true> {
     int64_t full;           // items of all full rounds
     int ql, cl, jl;         // last round: group, first candidate, stride
 
-    __device__ __forceinline__ explicit Work(const Args& a) {
+    __device__ __forceinline__ Work(const Args& a, const int*) {
         const int b = blockIdx.x, grid = gridDim.x;
         auto count = [&](int c, int j) {
             return c < j && c < a.n_cand ? static_cast<int>((a.n_cand - c + j - 1) / j) : 0;
@@ -330,57 +330,61 @@ struct Work<true> {
     }
 };
 
+// Few members: they stay in the planner's registers beside its windows (with the
+// list's pointers and the part held here too, short FP8 rows took 2% longer).
 template <>
 struct Work<false> {
-    deal::Lists lists;
-    const int* sums;  // see deal::per_candidate
-    deal::Part part;
-    int64_t n;  // items of this CTA
-    int q;      // this lane's query
+    int64_t n;         // items of this CTA
+    int lo;            // its first place in the flat list
+    int q;             // this lane's query
     deal::Columns cols;
-    float parts;  // parts (CTAs) per candidate, equal parts
+    float parts;       // parts (CTAs) per candidate; -1: parts of equal work, see deal::per_candidate
+    const int* sums;
 
-    __device__ __forceinline__ explicit Work(const Args& a)
-        : lists(a.lists()), sums(nullptr), part(deal::equal_part(lists)) {
-        parts = static_cast<float>(static_cast<int>(gridDim.x)) / static_cast<float>(lists.total);
-        begin();
+    __device__ __forceinline__ Work(const Args& a, const int* deal_sums) : sums(deal_sums) {
+        const deal::Part p = deal::equal_part(a.lists());
+        parts = static_cast<float>(static_cast<int>(gridDim.x)) / static_cast<float>(static_cast<int>(a.n_flat));
+        begin(a, p);
     }
     // The sampled lengths are in `s`: whether the part is another one for them.
-    __device__ __forceinline__ bool recut(int* s) {
-        sums = s;
-        if (!deal::uneven_part(lists, s, &part)) return false;
-        begin();
+    __device__ __forceinline__ bool recut(const Args& a, int* s) {
+        deal::Part p;
+        if (!deal::uneven_part(a.lists(), s, &p)) return false;
+        parts = -1.f;
+        begin(a, p);
         return true;
     }
-    __device__ __forceinline__ void begin() {
-        n = part.hi - part.lo;
+    __device__ __forceinline__ void begin(const Args& a, deal::Part p) {
+        lo = p.lo;
+        n = p.hi - p.lo;
         // the first query that ends past lo, 32 candidates for it at a time
         const int lane = threadIdx.x & 31;
         int base = 0;
-        for (int span = lists.n_queries - 1; span > 0;) {
+        for (int span = a.n_queries - 1; span > 0;) {
             const int step = (span + 31) / 32;
             const int last = min((lane + 1) * step, span) - 1;  // of this lane's piece
-            const bool before = lane * step < span && __ldg(lists.offsets + base + last + 1) <= part.lo;
+            const bool before = lane * step < span && __ldg(a.cand_offsets + base + last + 1) <= lo;
             const int pieces = __popc(__ballot_sync(0xffffffffu, before));
             base += min(pieces * step, span);
             span = min(step, span - min(pieces * step, span)) - 1;
         }
-        enter(base);
+        enter(a, base);
     }
-    __device__ __forceinline__ void enter(int query) {
+    __device__ __forceinline__ void enter(const Args& a, int query) {
         q = query;
+        const deal::Lists lists = a.lists();
         // one query: the first ids need not wait for its bounds
-        const bool one = lists.n_queries == 1;
+        const bool one = a.n_queries == 1;
         cols.enter(one ? 0 : deal::bound(lists, q), one ? lists.total : deal::bound(lists, q + 1),
-                   part.uneven ? deal::per_candidate(lists, sums, q) : parts);
+                   parts < 0.f ? deal::per_candidate(lists, sums, q) : parts);
     }
     // Item k < n: its query and its flat index.
     __device__ __forceinline__ void at(const Args& a, int64_t k, int* query, int* pos) {
-        const int p = part.lo + static_cast<int>(k);
+        const int p = lo + static_cast<int>(k);
         if (p >= cols.end && q < a.n_queries - 1) {
             int next = q + 1;
-            while (next < a.n_queries - 1 && p >= deal::bound(lists, next + 1)) ++next;
-            enter(next);
+            while (next < a.n_queries - 1 && p >= deal::bound(a.lists(), next + 1)) ++next;
+            enter(a, next);
         }
         *query = q;
         *pos = p < cols.c0 || p >= cols.end ? p : cols.at(p);  // outside: not a valid list
@@ -681,7 +685,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
             atomicOr(a.err, TMS_DEVERR_BAD_CSR);
         // three-window metadata pipeline: ids two windows ahead, offsets
         // and lengths one window ahead, the current window in registers.
-        Work<SH> work(a);
+        Work<SH> work(a, SH ? nullptr : deal_sums);
         struct Item {
             int q, pos, id;  // query (group), entry of the list (per-query lists: flat index), document
         };
@@ -707,7 +711,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
             // the samples' loads ran beside these
             if (a.sampled) {
                 named_barrier_sync<1, kDealThreads>();
-                if (work.recut(deal_sums)) first_windows();
+                if (work.recut(a, deal_sums)) first_windows();
             }
         }
 
