@@ -374,8 +374,8 @@ __device__ __forceinline__ void rotate4(uint4 (&v)[4], int kq) {
 // lines looked up in L1, one a cycle) and takes 5.3 with these (2,048): 3.7 TB/s
 // from L2 over all SMs, whether two or four tasks of a warp are in flight.
 // Table rows that are not 16-byte aligned (ALIGNED false) take four loads of
-// the same 64 bytes instead of one: K = 250, one list of 100 candidates 37.5 us,
-// 55.4 with 32 rows per load; fp16 table 31.5 and 43.8.
+// the same 64 bytes instead of one: K = 250, one list of 100 candidates 37.3 us,
+// 55.4 with 32 rows per load; fp16 table 30.7 and 43.8.
 template <int M, bool H16, bool ALIGNED>
 __device__ __forceinline__ void stage_chunk(const float* src, int nq, int K, int ch, float* lut_s, int warp,
                                             int lane) {
@@ -384,7 +384,7 @@ __device__ __forceinline__ void stage_chunk(const float* src, int nq, int K, int
     const int ii = lane & 7;
     const int kq = lane >> 3;
     constexpr int kTasks = staged_table_bytes(M) / 256 / 16 * 2;
-#pragma unroll 2
+#pragma unroll (ALIGNED || H16 ? 2 : 4)
     for (int task = warp; task < kTasks; task += kWarps) {
         const int slo = task & 1;
         const int rho0 = (task >> 1) * 16;  // KS is a multiple of 16
@@ -423,14 +423,17 @@ __device__ __forceinline__ void stage_chunk(const float* src, int nq, int K, int
     }
 }
 
-// Out of line: inlined a second time, it cost the gather loop 1.6% (fp16 table).
-template <int M, bool H16>
-__device__ __noinline__ void stage_chunk_any(const float* src, int nq, int K, int ch, float* lut_s, int warp,
-                                             int lane) {
-    stage_chunk<M, H16, false>(src, nq, K, ch, lut_s, warp, lane);
+template <int M, bool H16, bool ALIGNED>
+__device__ __noinline__ void stage_chunk_apart(const float* src, int nq, int K, int ch, float* lut_s, int warp,
+                                               int lane) {
+    stage_chunk<M, H16, ALIGNED>(src, nq, K, ch, lut_s, warp, lane);
 }
 
-template <int M, bool H16>
+// ALIGNED: the table's rows are 16-byte aligned (k % 4 == 0); a kernel of its
+// own for each way of staging.  The gather loop of the fp16 table with M = 16
+// has no register to spare and is 1.5% faster beside a staging out of line (16
+// x 10,000: 661 and 652 us); the fp32 table's is 0.7%, M = 32's 1.3% slower.
+template <int M, bool H16, bool ALIGNED>
 __global__ void __launch_bounds__(kWarps * 32, 1) score_kernel_staged(const Args a, int lut_bytes) {
     griddep_wait();
     griddep_launch_dependents();
@@ -509,10 +512,10 @@ __global__ void __launch_bounds__(kWarps * 32, 1) score_kernel_staged(const Args
         for (int ch = 0; ch < nchunks; ++ch) {
             __syncthreads();
             const float* src = a.lut + static_cast<int64_t>(q) * a.nq * M * K;
-            if ((K & 3) == 0)
-                stage_chunk<M, H16, true>(src, a.nq, K, ch, lut_s, warp, lane);
+            if constexpr (H16 && ALIGNED && M == 16)
+                stage_chunk_apart<M, H16, ALIGNED>(src, a.nq, K, ch, lut_s, warp, lane);
             else
-                stage_chunk_any<M, H16>(src, a.nq, K, ch, lut_s, warp, lane);
+                stage_chunk<M, H16, ALIGNED>(src, a.nq, K, ch, lut_s, warp, lane);
             if (threadIdx.x == 0) next_local = 0;
             __syncthreads();
 
@@ -757,10 +760,14 @@ tms_status score(const float* lut, int n_queries, int nq, int m, int k, const ui
         e = plain(score_kernel<4>);
     else if (m == 8)
         e = plain(score_kernel<8>);
+    else if (m == 16 && k % 4 == 0)
+        e = half ? staged(score_kernel_staged<16, true, true>) : staged(score_kernel_staged<16, false, true>);
     else if (m == 16)
-        e = half ? staged(score_kernel_staged<16, true>) : staged(score_kernel_staged<16, false>);
+        e = half ? staged(score_kernel_staged<16, true, false>) : staged(score_kernel_staged<16, false, false>);
+    else if (k % 4 == 0)
+        e = half ? staged(score_kernel_staged<32, true, true>) : staged(score_kernel_staged<32, false, true>);
     else
-        e = half ? staged(score_kernel_staged<32, true>) : staged(score_kernel_staged<32, false>);
+        e = half ? staged(score_kernel_staged<32, true, false>) : staged(score_kernel_staged<32, false, false>);
     if (e != cudaSuccess) return launch_status(e);
     return launch_status(cudaGetLastError());
 }
