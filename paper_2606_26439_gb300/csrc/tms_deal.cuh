@@ -94,29 +94,35 @@ __device__ __forceinline__ void sample(const Lists& l, int* sums, int warp, int 
 
 struct Part {
     int lo, hi;   // entries [lo, hi) of the flat list
-    bool uneven;  // parts of equal estimated work: see per_candidate
+    bool uneven;  // parts of equal estimated work
 };
 
+// In shared memory; what follows it there is aligned to 16 bytes.
+struct alignas(16) Shared {
+    int sums[kSums];  // of sampled rows; where the parts are uneven, then CTAs per candidate of each group (float)
+    Part part;        // uneven false: the parts are of equal count
+};
+static_assert(sizeof(Shared) % 16 == 0, "the regions after it stay aligned");
+
 // This CTA's part of equal count.
-__device__ __forceinline__ Part equal_part(const Lists& l) {
+__device__ __forceinline__ Part equal_part(int total) {
     const int grid = gridDim.x, block = blockIdx.x;
-    const int each = l.total / grid, more = l.total - each * grid;
+    const int each = total / grid, more = total - each * grid;
     auto start = [&](int b) { return each * b + more * b / grid; };  // total * b / grid
     return Part{start(block), start(block + 1), false};
 }
 
-// This CTA's part of equal estimated work, if the lists are unlike enough for
-// it; false: leave `p` as it is.  One warp, the same outcome in every CTA; `sums`
-// as sample left them, afterwards sums[g] is the parts per candidate of group
-// g, as a float.
-__device__ __forceinline__ bool uneven_part(const Lists& l, int* sums, Part* p) {
+// This CTA's part of equal estimated work to sh.part, if the lists are unlike
+// enough for it; else sh.part.uneven is false.  One warp, the same outcome in
+// every CTA; sh.sums as sample left them.
+__device__ __forceinline__ void uneven_part(const Lists& l, Shared& sh) {
     const int lane = threadIdx.x & 31;
     const int grid = gridDim.x;
     const Groups groups(l);
     const int first = groups.first, n = groups.n;
     int s = 0;  // the group's sampled rows
     if (lane < groups.count)
-        for (int r = 0; r < 1 << groups.sums; ++r) s += sums[(lane << groups.sums) + r];
+        for (int r = 0; r < 1 << groups.sums; ++r) s += sh.sums[(lane << groups.sums) + r];
     float all = static_cast<float>(n) * static_cast<float>(s);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
@@ -124,7 +130,10 @@ __device__ __forceinline__ bool uneven_part(const Lists& l, int* sums, Part* p) 
     // half a part or more (lengths uniform on [32, 180]: three standard errors
     // of the mean of 64 samples are 15%)
     const bool longer = n > l.total / grid / 2 && static_cast<float>(s) * static_cast<float>(l.total) > 1.25f * all;
-    if (!__any_sync(0xffffffffu, longer) || __any_sync(0xffffffffu, n < 0)) return false;
+    if (!__any_sync(0xffffffffu, longer) || __any_sync(0xffffffffu, n < 0)) {
+        if (lane == 0) sh.part.uneven = false;
+        return;
+    }
     const unsigned long long w = static_cast<unsigned long long>(n) * static_cast<unsigned>(s);  // estimated work
     unsigned long long end = w;                                                                  // and its prefix
 #pragma unroll
@@ -142,17 +151,10 @@ __device__ __forceinline__ bool uneven_part(const Lists& l, int* sums, Part* p) 
         const float x = static_cast<float>(t - (ge - gw)) / static_cast<float>(gw) * static_cast<float>(gn);
         return gf + min(gn, static_cast<int>(x));
     };
-    *p = Part{place(blockIdx.x), place(blockIdx.x + 1), true};
-    __syncwarp();  // every lane has read the sums
-    if (lane < groups.count)
-        sums[lane] = __float_as_int(static_cast<float>(s) * static_cast<float>(grid) / static_cast<float>(work));
-    __syncwarp();
-    return true;
-}
-
-// Parts (CTAs) per candidate of query q, where the parts are uneven.
-__device__ __forceinline__ float per_candidate(const Lists& l, const int* sums, int q) {
-    return __int_as_float(sums[((q + 1) * min(l.n_queries, kGroups) - 1) / l.n_queries]);
+    const Part p{place(blockIdx.x), place(blockIdx.x + 1), true};
+    if (lane == 0) sh.part = p;
+    if (lane < groups.count)  // every lane has read the sums before the votes
+        sh.sums[lane] = __float_as_int(static_cast<float>(s) * static_cast<float>(grid) / static_cast<float>(work));
 }
 
 // Entries [c0, end) of one query, taken in turn by the w or so CTAs that meet
@@ -163,7 +165,9 @@ struct Columns {
     int c0, end;
     int w, wide, tall, rem;
 
-    // `parts`: CTAs per candidate, or any number that all CTAs agree on.
+    // `parts`: CTAs per candidate, or any number that all CTAs agree on: those
+    // of the list's group where the parts are uneven and each group is one list,
+    // else of all lists (of many, a CTA or two meet one anyway).
     __device__ __forceinline__ void enter(int first, int last, float parts) {
         c0 = first, end = last;
         if (c0 >= end) return;

@@ -200,10 +200,6 @@ struct Args {
     int pq_k;                   // kPQ: centroids per subspace (codes >= pq_k read zeros)
     long long budget;           // SM cycles a pipeline wait may last (<= 0: kWaitBudgetCycles)
     int fault;                  // diagnostics: kFaultHoldAccumulator, else 0
-
-    __device__ __forceinline__ deal::Lists lists() const {
-        return deal::Lists{cand_offsets, cand_ids, lengths, n_docs, n_queries, static_cast<int>(n_flat)};
-    }
 };
 
 // Stands in for the row scale of a column past its document's end.
@@ -259,7 +255,7 @@ __host__ __device__ inline Layout make_layout(int stages, int qslots, int nchunk
     L.fin_off = L.um_off + um_slots(nchunks) * L.um_stride;
     L.bias_off = (L.fin_off + (sh ? epi_warps(h) : 1) * kFinWarpBytes + 127) & ~127;
     L.deal_off = L.bias_off + 256;
-    L.sc_off = L.deal_off + (sh ? 0 : deal::kSums * 4);
+    L.sc_off = L.deal_off + (sh ? 0 : static_cast<int>(sizeof(deal::Shared)));
     L.cb_off = L.sc_off + (f8 ? st_ring(str) * str * 4 : 0);  // F8: [st_ring][str] column scales
     L.code_off = L.cb_off + (kind == kPQ ? kPqCbBytes : 0);                        // kPQ: fp16 codebook
     L.st_off = L.code_off + (kind == kPQ ? kCodeRing * str * kPqM : 0);  // kPQ: code-row ring
@@ -302,7 +298,7 @@ struct Work<true> {
     int64_t full;           // items of all full rounds
     int ql, cl, jl;         // last round: group, first candidate, stride
 
-    __device__ __forceinline__ Work(const Args& a, const int*) {
+    __device__ __forceinline__ Work(const Args& a, const deal::Shared&) {
         const int b = blockIdx.x, grid = gridDim.x;
         auto count = [&](int c, int j) {
             return c < j && c < a.n_cand ? static_cast<int>((a.n_cand - c + j - 1) / j) : 0;
@@ -334,24 +330,22 @@ struct Work<true> {
 // list's pointers and the part held here too, short FP8 rows took 2% longer).
 template <>
 struct Work<false> {
-    int64_t n;         // items of this CTA
-    int lo;            // its first place in the flat list
-    int q;             // this lane's query
+    int64_t n;  // items of this CTA
+    int lo;     // its first place in the flat list
+    int q;      // this lane's query
     deal::Columns cols;
-    float parts;       // parts (CTAs) per candidate; -1: parts of equal work, see deal::per_candidate
-    const int* sums;
+    float parts;  // CTAs per candidate; -1: of each list, in `dealt`
+    const deal::Shared& dealt;
 
-    __device__ __forceinline__ Work(const Args& a, const int* deal_sums) : sums(deal_sums) {
-        const deal::Part p = deal::equal_part(a.lists());
+    __device__ __forceinline__ Work(const Args& a, const deal::Shared& sh) : dealt(sh) {
         parts = static_cast<float>(static_cast<int>(gridDim.x)) / static_cast<float>(static_cast<int>(a.n_flat));
-        begin(a, p);
+        begin(a, deal::equal_part(static_cast<int>(a.n_flat)));
     }
-    // The sampled lengths are in `s`: whether the part is another one for them.
-    __device__ __forceinline__ bool recut(const Args& a, int* s) {
-        deal::Part p;
-        if (!deal::uneven_part(a.lists(), s, &p)) return false;
-        parts = -1.f;
-        begin(a, p);
+    // The part by the lists' lengths, if it is another one.
+    __device__ __forceinline__ bool recut(const Args& a) {
+        if (!dealt.part.uneven) return false;
+        if (a.n_queries <= deal::kGroups) parts = -1.f;
+        begin(a, dealt.part);
         return true;
     }
     __device__ __forceinline__ void begin(const Args& a, deal::Part p) {
@@ -370,26 +364,48 @@ struct Work<false> {
         }
         enter(a, base);
     }
+    __device__ __forceinline__ int bound(const Args& a, int i) const {
+        const int64_t x = __ldg(a.cand_offsets + i);
+        return static_cast<int>(x < 0 ? 0 : (x > a.n_flat ? a.n_flat : x));
+    }
     __device__ __forceinline__ void enter(const Args& a, int query) {
         q = query;
-        const deal::Lists lists = a.lists();
-        // one query: the first ids need not wait for its bounds
-        const bool one = a.n_queries == 1;
-        cols.enter(one ? 0 : deal::bound(lists, q), one ? lists.total : deal::bound(lists, q + 1),
-                   parts < 0.f ? deal::per_candidate(lists, sums, q) : parts);
+        int c0 = 0, end = static_cast<int>(a.n_flat);  // one query: the first ids need not wait for its bounds
+        if (a.n_queries > 1) c0 = bound(a, q), end = bound(a, q + 1);
+        cols.enter(c0, end, parts < 0.f ? __int_as_float(dealt.sums[q]) : parts);
     }
     // Item k < n: its query and its flat index.
     __device__ __forceinline__ void at(const Args& a, int64_t k, int* query, int* pos) {
         const int p = lo + static_cast<int>(k);
         if (p >= cols.end && q < a.n_queries - 1) {
             int next = q + 1;
-            while (next < a.n_queries - 1 && p >= deal::bound(a.lists(), next + 1)) ++next;
+            while (next < a.n_queries - 1 && p >= bound(a, next + 1)) ++next;
             enter(a, next);
         }
         *query = q;
         *pos = p < cols.c0 || p >= cols.end ? p : cols.at(p);  // outside: not a valid list
     }
 };
+
+// The lists' lengths for the planner, by WARPS warps that have nothing to do yet
+// (`warp` of them, the last one decides).  Out of line: passes of one list, which
+// do not call it, fetch their instructions cold as well (1 x 10,000 and top-k
+// 0.6 us longer with it inlined).
+template <int WARPS>
+__device__ __noinline__ void sample_lists(const int64_t* offsets, const int32_t* ids, const int32_t* lengths,
+                                          int64_t n_docs, int n_queries, int total, deal::Shared* dealt, int warp) {
+    const deal::Lists l{offsets, ids, lengths, n_docs, n_queries, total};
+    deal::sample<8, 16>(l, dealt->sums, warp, WARPS);
+    if (warp == WARPS - 1) {
+        named_barrier_sync<2, 32 * WARPS>();
+        deal::uneven_part(l, *dealt);
+        __threadfence_block();
+        named_barrier_arrive<1, 64>();  // with the planner
+    } else {
+        __threadfence_block();
+        named_barrier_arrive<2, 32 * WARPS>();
+    }
+}
 
 __device__ __forceinline__ Meta load_meta(const Args& a, int id) {
     Meta m;
@@ -500,7 +516,6 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
     constexpr int kHelpers = help_warps(KIND);
     constexpr int kHelpWarp = kFinWarp + fin_warps(SH);    // TF / kPQ: the first splitter / decompressor
     constexpr int kStRing = st_ring(STR);
-    constexpr int kDealThreads = 32 * (1 + kEpiWarps + fin_warps(SH));  // the planner and the warps that sample for it
     static_assert(KACC >= 2 && TCOLS * CTAS <= 512, "tensor memory of one SM");
 
     extern __shared__ uint8_t smem_raw[];
@@ -520,7 +535,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
     uint8_t* um_base = smem + L.um_off;    // per-query lists: [UMS][unit][block][row] row maxima
     uint8_t* fin_base = smem + L.fin_off;  // finished-document rows
     float* bias = reinterpret_cast<float*>(smem + L.bias_off);  // [8][8]: entry [n][j] 0 for j < n, else -inf
-    int* deal_sums = reinterpret_cast<int*>(smem + L.deal_off);  // per-query lists: see tms_deal.cuh
+    deal::Shared& dealt = *reinterpret_cast<deal::Shared*>(smem + L.deal_off);  // per-query lists: see tms_deal.cuh
     float* sc = reinterpret_cast<float*>(smem + L.sc_off);      // F8: [kStRing][STR] scale of each column
     StSlot* slots = reinterpret_cast<StSlot*>(smem + L.st_off);
     uint8_t* cb = smem + L.cb_off;           // kPQ: fp16 codebook, entry (code, m) at (code * 16 + m) * 16
@@ -685,7 +700,7 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
             atomicOr(a.err, TMS_DEVERR_BAD_CSR);
         // three-window metadata pipeline: ids two windows ahead, offsets
         // and lengths one window ahead, the current window in registers.
-        Work<SH> work(a, SH ? nullptr : deal_sums);
+        Work<SH> work(a, dealt);
         struct Item {
             int q, pos, id;  // query (group), entry of the list (per-query lists: flat index), document
         };
@@ -699,19 +714,16 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
         };
         Item now, then, later;
         Meta cur, nxt;
-        auto first_windows = [&]() {
+        for (bool recut = !SH && a.sampled;; recut = false) {
             now = item(lane);
             cur = load_meta(a, now.id);
             then = item(32 + lane);
             nxt = load_meta(a, then.id);
             later = item(64 + lane);
-        };
-        first_windows();
-        if constexpr (!SH) {
-            // the samples' loads ran beside these
-            if (a.sampled) {
-                named_barrier_sync<1, kDealThreads>();
-                if (work.recut(a, deal_sums)) first_windows();
+            if (!recut) break;
+            if constexpr (!SH) {
+                named_barrier_sync<1, 64>();  // the samples' loads ran beside these
+                if (!work.recut(a)) break;
             }
         }
 
@@ -1296,9 +1308,8 @@ __global__ void __launch_bounds__(kernel_threads(KIND, H, SH), CTAS)
         if constexpr (!SH) {
             // nothing to do here yet: the lists' lengths for the planner
             if (a.sampled) {
-                deal::sample<8, 16>(a.lists(), deal_sums, warp - kEpiWarp, kEpiWarps + fin_warps(SH));
-                __threadfence_block();
-                named_barrier_arrive<1, kDealThreads>();
+                sample_lists<kEpiWarps + fin_warps(SH)>(a.cand_offsets, a.cand_ids, a.lengths, a.n_docs, a.n_queries,
+                                                        static_cast<int>(a.n_flat), &dealt, warp - kEpiWarp);
             }
         }
         const bool finisher = !SH && warp >= kFinWarp;

@@ -485,18 +485,14 @@ __global__ void __launch_bounds__(kWarps * 32, 1) score_kernel_staged(const Args
     // and 152 CTAs, 16 queries x 50,000 candidates spent 1.1 of 6.7 ms on it and
     // 16 x 1,000 with 100 query tokens 3.4 of 4.1 ms).
     const deal::Lists lists{a.cand_offsets, a.cand_ids, a.lengths, a.n_docs, a.n_queries, static_cast<int>(a.n_cand)};
-    __shared__ int deal_sums[deal::kSums];
-    __shared__ deal::Part shared_part;
-    deal::Part part = deal::equal_part(lists);
+    __shared__ deal::Shared dealt;
+    deal::Part part = deal::equal_part(lists.total);
     if (a.sampled) {
-        deal::sample<16, 40>(lists, deal_sums, warp, kWarps);
+        deal::sample<16, 40>(lists, dealt.sums, warp, kWarps);
         __syncthreads();
-        if (warp == 0) {
-            deal::uneven_part(lists, deal_sums, &part);
-            if (lane == 0) shared_part = part;
-        }
+        if (warp == 0) deal::uneven_part(lists, dealt);
         __syncthreads();
-        part = shared_part;
+        if (dealt.part.uneven) part = dealt.part;
     }
     const float parts = static_cast<float>(static_cast<int>(gridDim.x)) / static_cast<float>(lists.total);
 
@@ -506,7 +502,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) score_kernel_staged(const Args
         const int first = max(part.lo, cols.c0);
         const int n_local = min(part.hi, cols.end) - first;
         if (n_local <= 0) continue;
-        cols.enter(cols.c0, cols.end, part.uneven ? deal::per_candidate(lists, deal_sums, q) : parts);
+        const bool own = part.uneven && a.n_queries <= deal::kGroups;
+        cols.enter(cols.c0, cols.end, own ? __int_as_float(dealt.sums[q]) : parts);
         int col0, t0;
         cols.find(first, &col0, &t0);
         for (int ch = 0; ch < nchunks; ++ch) {
