@@ -15,7 +15,7 @@
 // are sampled first, the same ones by every CTA, and where a list's documents
 // are longer than the average by a quarter, the parts are of equal estimated
 // work: 232 and 199.  Like lists keep parts of equal count, whose balance no
-// estimate reaches, and pay 0.5 to 1.6 us (16 x 1,000, fp16: 66.7 and 68.2).  The
+// estimate reaches, and pay 0.5 to 1.5 us (16 x 1,000, fp16: 66.2 and 66.8).  The
 // PQ kernel has no spare bandwidth to make up for uneven parts: the same lists
 // of 30,000, fp32 table, took 5,387 us in parts of equal count (2,952 with every
 // query dealt to every CTA), now 2,052.

@@ -23,8 +23,8 @@
 // costs of the pipeline -- barrier round trips, commits, MMA issue -- are
 // paid once per super-tile, typically two to three documents.
 //
-//   * Planner warp: takes the candidates 32 at a time, one per lane
-//     (metadata, validity, query, -inf / NaN for empty / bad documents),
+//   * Planner warp: takes the CTA's candidates (Work) 32 at a time, one per
+//     lane (metadata, validity, query, -inf / NaN for empty / bad documents),
 //     places their units in super-tiles with one scan and publishes each
 //     super-tile as one record -- header, tile list, documents that end in
 //     it -- with a single barrier arrival.  It also loads each query's tile
@@ -237,7 +237,8 @@ constexpr int kFinWarpBytes = kFinRows * 33 * 4 + kFinRows * 8;
 // accumulator rows that nothing reads.  A stage holds the full super-tile
 // of str rows, so the document operand (N <= str) never reads past it.
 // TF: the query region and every stage have a lo twin right after them.
-// F8: per super-tile record slot, the row scale of every column.
+// F8: per super-tile record slot, the row scale of every column.  Per-query
+// lists: the sampled lengths (tms_deal.cuh).
 // Streamed query (qslots = 0, qrows = 128 H): no resident query region;
 // each chunk stage holds the str document rows, then the qrows query rows
 // of the same dimension chunk.
@@ -1700,8 +1701,8 @@ inline int config_shapes(Config* out) {
 // Without a tuned or forced configuration: one CTA per SM with 256-row
 // super-tiles (about two documents per MMA run); two CTAs with 128-row ones
 // for short rows; one CTA with 128-row ones for eight queries of three or four
-// chunks, split TF32 and what leaves no room for more (plan_tc has the lines
-// and the figures).  KIND selects the row type; kE4M3 ignores `dtype` (rows
+// chunks and split TF32; the query streamed where its tile leaves too few stages
+// (plan_tc has the lines and the figures).  KIND selects the row type; kE4M3 ignores `dtype` (rows
 // are E4M3 codes; t_scales in `a`).  The caller sets a.nchunks =
 // ceil(d / chunk_elems(KIND)), and a.bpc: per-query ceil(nq / 32), shared mode
 // the group size.  `force` (the autotuner's) overrides the choice;
