@@ -45,8 +45,8 @@ def test_shared_lists_of_few_candidates(cuda_lib, queries, cand):
 
 
 def test_one_shared_candidate_uses_every_cta(cuda_lib):
-    """4,096 queries x 1 document against 256 x 16, the same work: 1.4 times
-    (6 when a round took 16 groups of queries on as many CTAs)."""
+    """4,096 queries x 1 document against 256 x 16, the same work: 0.8 times
+    (3.4 when a round took 16 groups of queries on as many CTAs)."""
     import torch
     from paper_2606_26439_gb300 import tms
     tok, off, ln = synth.device_dense_corpus(synth.lengths_fixed(16, 128), 128, "f16", 82)
@@ -80,8 +80,8 @@ def _uneven(kind, n_long, n_short, seed):
 @pytest.mark.parametrize("dtype", ["f16", "fp8", "f32", "pq", "pq_f16"])
 def test_lists_of_unlike_lengths_are_balanced(cuda_lib, dtype):
     """One list of 180-token documents beside fifteen of 32-token ones, against
-    the same documents mixed in every list: about the same time (1.8 to 2.6
-    times in parts of equal count)."""
+    the same documents mixed in every list: 0.95 to 1.16 times (1.8 to 2.6 in
+    parts of equal count)."""
     import torch
     from paper_2606_26439_gb300 import tms
     n = 4000 if dtype == "f32" else 10_000
@@ -159,8 +159,8 @@ def test_sampled_lists_write_every_candidate_once(cuda_lib, dtype, lists):
 @pytest.mark.parametrize("f16", [False, True])
 def test_table_rows_of_any_alignment_are_staged_alike(cuda_lib, f16):
     """One short list, where staging the table is most of the time, with 255
-    centroids (rows not 16-byte aligned) against 256: 1.1 times (1.6 when a load
-    touched 32 rows)."""
+    centroids (rows not 16-byte aligned) against 256: 0.97 times, fp16 table 1.15
+    (1.6 when a load touched 32 rows)."""
     import torch
     from paper_2606_26439_gb300 import tms
     ln = synth.lengths_fixed(100, 100)
